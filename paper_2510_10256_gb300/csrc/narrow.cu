@@ -7,6 +7,7 @@
 #include "bound32.cuh"
 #include "geometry.cuh"
 #include "frest.cuh"
+#include "pairhess.cuh"
 #include "pairs.cuh"
 #include "prims.cuh"
 #include "scene.cuh"
@@ -513,13 +514,10 @@ __global__ void k_unique_write(int64_t m, const uint64_t* __restrict__ k, const 
   atomicAdd(&row_cnt[key >> bits_n], 1u);
 }
 
-// --- analytic derivatives of the squared distance in relative variables ---
-// z_m = sum_i C[m][i] x_i (m < nz) with C rows summing to zero.
-//   PP:    z0 = b - a                       s = |z0|^2
-//   PE:    z0 = w = q - e0, z1 = u = e1-e0  s = |w|^2 - (w.u)^2/|u|^2
-//   plane: z0 = w, z1 = u, z2 = v           s = (w.(u x v))^2 / |u x v|^2
-// (point-triangle face: w = p-t0, u = t1-t0, v = t2-t0; edge-edge interior:
-//  w = b0-a0, u = a1-a0, v = b1-b0.)
+// Distance types as difference vectors z_m = sum_i C[m][i] x_i (m <= kind):
+//   point-point: z0 = b - a;  point-edge: z0 = w = q - e0, z1 = u = e1 - e0;
+//   plane: z0 = w, z1 = u, z2 = v (point-triangle face: w = p - t0, u = t1 - t0,
+//   v = t2 - t0; edge-edge interior: w = b0 - a0, u = a1 - a0, v = b1 - b0).
 struct TypeInfo {
   int8_t kind;   // 0 PP, 1 PE, 2 plane
   int8_t C[3][4];
@@ -546,223 +544,11 @@ __constant__ TypeInfo c_ee_types[9] = {
     {2, {{-1, 0, 1, 0}, {-1, 1, 0, 0}, {0, 0, -1, 1}}},
 };
 
-// Orthonormal bases of the complement of rigid translations of the points a
-// stencil type involves: K4[i][a] for 4 points (entries +-1/2), K3 for 3.
+// Orthonormal basis of the complement of rigid translations of four points
 __constant__ double c_K4[4][3] = {{0.5, 0.5, 0.5}, {0.5, -0.5, -0.5}, {-0.5, 0.5, -0.5}, {-0.5, -0.5, 0.5}};
-__constant__ double c_K3[3][2] = {{0.70710678118654752440, 0.40824829046386301637},
-                                  {-0.70710678118654752440, 0.40824829046386301637},
-                                  {0.0, -0.81649658092772603273}};
 
 __host__ __device__ __forceinline__ int tri_idx(int i, int j, int D) {  // packed upper triangle, i <= j
   return i * D - (i * (i - 1)) / 2 + (j - i);
-}
-
-__host__ __device__ __forceinline__ double& zh(double* H, int r, int c) { return H[r * 9 + c]; }
-
-// gradient gs[9] and Hessian Hs[81] (row-major, 3x3 blocks of z) of s
-__host__ __device__ void s_derivs(int kind, const d3* z, double* gs, double* Hs) {
-  for (int i = 0; i < 81; ++i) Hs[i] = 0.0;
-  for (int i = 0; i < 9; ++i) gs[i] = 0.0;
-  if (kind == 0) {
-    gs[0] = 2.0 * z[0].x;
-    gs[1] = 2.0 * z[0].y;
-    gs[2] = 2.0 * z[0].z;
-    zh(Hs, 0, 0) = zh(Hs, 1, 1) = zh(Hs, 2, 2) = 2.0;
-    return;
-  }
-  if (kind == 1) {
-    const double w[3] = {z[0].x, z[0].y, z[0].z}, u[3] = {z[1].x, z[1].y, z[1].z};
-    const double al = w[0] * u[0] + w[1] * u[1] + w[2] * u[2];
-    const double be = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    const double ibe = 1.0 / be;  // one division; the rest multiply
-    const double ga = al * ibe;
-    for (int k = 0; k < 3; ++k) {
-      gs[k] = 2.0 * w[k] - 2.0 * ga * u[k];
-      gs[3 + k] = -2.0 * ga * w[k] + 2.0 * ga * ga * u[k];
-    }
-    for (int i = 0; i < 3; ++i)
-      for (int j = 0; j < 3; ++j) {
-        const double dij = (i == j) ? 1.0 : 0.0;
-        const double ww = 2.0 * dij - 2.0 * u[i] * u[j] * ibe;
-        const double wu = -2.0 * u[i] * w[j] * ibe - 2.0 * ga * dij + 4.0 * ga * u[i] * u[j] * ibe;
-        const double uu = -2.0 * w[i] * w[j] * ibe + 4.0 * ga * (w[i] * u[j] + u[i] * w[j]) * ibe +
-                          2.0 * ga * ga * dij - 8.0 * ga * ga * u[i] * u[j] * ibe;
-        zh(Hs, i, j) = ww;
-        zh(Hs, i, 3 + j) = wu;
-        zh(Hs, 3 + j, i) = wu;
-        zh(Hs, 3 + i, 3 + j) = uu;
-      }
-    return;
-  }
-  // plane: s = g^2 / N, g = w.(u x v), N = |u x v|^2
-  const d3 w = z[0], u = z[1], v = z[2];
-  const double nx = u.y * v.z - u.z * v.y, ny = u.z * v.x - u.x * v.z, nz = u.x * v.y - u.y * v.x;
-  const double g = w.x * nx + w.y * ny + w.z * nz;
-  const double uu = u.x * u.x + u.y * u.y + u.z * u.z;
-  const double vv = v.x * v.x + v.y * v.y + v.z * v.z;
-  const double uv = u.x * v.x + u.y * v.y + u.z * v.z;
-  const double N = nx * nx + ny * ny + nz * nz;
-  // grad g: (n, v x w, w x u)
-  double gg[9] = {nx,
-                  ny,
-                  nz,
-                  v.y * w.z - v.z * w.y,
-                  v.z * w.x - v.x * w.z,
-                  v.x * w.y - v.y * w.x,
-                  w.y * u.z - w.z * u.y,
-                  w.z * u.x - w.x * u.z,
-                  w.x * u.y - w.y * u.x};
-  // grad N: (0, 2 vv u - 2 uv v, 2 uu v - 2 uv u)
-  const double ua[3] = {u.x, u.y, u.z}, va[3] = {v.x, v.y, v.z}, wa[3] = {w.x, w.y, w.z};
-  double gN[9];
-  for (int k = 0; k < 3; ++k) {
-    gN[k] = 0.0;
-    gN[3 + k] = 2.0 * vv * ua[k] - 2.0 * uv * va[k];
-    gN[6 + k] = 2.0 * uu * va[k] - 2.0 * uv * ua[k];
-  }
-  const double iN = 1.0 / N;
-  const double a1 = 2.0 * g * iN, a2 = g * g * iN * iN;
-  for (int k = 0; k < 9; ++k) gs[k] = a1 * gg[k] - a2 * gN[k];
-  // Hessian
-  const double c_gg = 2.0 * iN;              // grad g grad g^T
-  const double c_hg = 2.0 * g * iN;          // hess g
-  const double c_gN = -2.0 * g * iN * iN;    // (grad g grad N^T + grad N grad g^T)
-  const double c_hN = -g * g * iN * iN;      // hess N
-  const double c_NN = 2.0 * g * g * iN * iN * iN;  // grad N grad N^T
-  for (int r = 0; r < 9; ++r)
-    for (int c = 0; c < 9; ++c)
-      Hs[r * 9 + c] = c_gg * gg[r] * gg[c] + c_gN * (gg[r] * gN[c] + gN[r] * gg[c]) + c_NN * gN[r] * gN[c];
-  // hess g: blocks (w,u) = -[v]x, (w,v) = [u]x, (u,v) = -[w]x and transposes
-  auto skew_add = [&](int rb, int cb, const double* a, double sc) {
-    // adds sc * [a]x to block (rb, cb) and sc * [a]x^T to block (cb, rb)
-    const double m[3][3] = {{0.0, -a[2], a[1]}, {a[2], 0.0, -a[0]}, {-a[1], a[0], 0.0}};
-    for (int i = 0; i < 3; ++i)
-      for (int j = 0; j < 3; ++j) {
-        Hs[(3 * rb + i) * 9 + 3 * cb + j] += sc * m[i][j];
-        Hs[(3 * cb + j) * 9 + 3 * rb + i] += sc * m[i][j];
-      }
-  };
-  skew_add(0, 1, va, -c_hg);
-  skew_add(0, 2, ua, c_hg);
-  skew_add(1, 2, wa, -c_hg);
-  // hess N: (u,u) 2 vv I - 2 v v^T ; (v,v) 2 uu I - 2 u u^T ; (u,v) 4 u v^T - 2 v u^T - 2 uv I
-  for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 3; ++j) {
-      const double dij = (i == j) ? 1.0 : 0.0;
-      Hs[(3 + i) * 9 + 3 + j] += c_hN * (2.0 * vv * dij - 2.0 * va[i] * va[j]);
-      Hs[(6 + i) * 9 + 6 + j] += c_hN * (2.0 * uu * dij - 2.0 * ua[i] * ua[j]);
-      const double uvb = c_hN * (4.0 * ua[i] * va[j] - 2.0 * va[i] * ua[j] - 2.0 * uv * dij);
-      Hs[(3 + i) * 9 + 6 + j] += uvb;
-      Hs[(6 + j) * 9 + 3 + i] += uvb;
-    }
-}
-
-// Reduced barrier Hessian of a plane-type pair (point-triangle face,
-// edge-edge interior) in the translation-free coordinates y of its four
-// points, z = (M x I) y, differentiating the distance itself:
-//   d = |g| / sqrt(N),  g = w.(u x v),  N = |n|^2,  n = u x v,
-//   grad d = sg gam (grad g - h grad N),  gam = 1/sqrt(N), h = g / (2N), sg = sign g,
-//   hess d = sg gam (hess g - h hess N - (grad g grad N^T + grad N grad g^T) / (2N)
-//                    + (3h / (2N)) grad N grad N^T),
-//   B = kappa b'' grad d grad d^T + kappa b' hess d.
-// (Through s = d^2 instead, B = (b'' - b'/d) grad d grad d^T + b'/(2d) hess s
-// adds and then cancels a term of order |grad g|^2 / N, which for
-// near-parallel edges or slender triangles costs about 1/sin of the angle
-// in digits.)  With q_b = M[2][b] u - M[1][b] v (so dn/dy_b = [q_b]x):
-//   grad_y g = (M^T x I) grad_z g,   grad_y N = (M^T x I) grad_z N,
-//   hess_y g, block (a,b) = [r_ab]x,
-//     r_ab = -(M0a M1b - M1a M0b) v + (M0a M2b - M2a M0b) u - (M1a M2b - M2a M1b) w,
-//   hess_y N, block (a,b) = 2 (q_a.q_b) I - 2 q_b q_a^T + 2 (M2a M1b - M1a M2b) [n]x.
-// With e = grad_y g - h grad_y N the rank-one part is
-//   kappa b'' gam^2 e e^T - (s1 / 2N)(e gN^T + gN e^T) + (h s1 / 2N) gN gN^T,
-// s1 = kappa b' sg gam, gN = grad_y N.  Writes grad_z d (gd, 9) and the
-// packed upper triangle of B (Bq, 45); kb1 = kappa b', kb2 = kappa b''.
-__host__ __device__ __forceinline__ void plane_reduced(const double (&z)[3][3], const double (&M)[3][3], double kb1,
-                                                       double kb2, double (&gd)[9], double (&Bq)[45]) {
-  const double* w = z[0];
-  const double* u = z[1];
-  const double* v = z[2];
-  const double n[3] = {u[1] * v[2] - u[2] * v[1], u[2] * v[0] - u[0] * v[2], u[0] * v[1] - u[1] * v[0]};
-  const double g = w[0] * n[0] + w[1] * n[1] + w[2] * n[2];
-  const double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-  const double vv = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-  const double uv = u[0] * v[0] + u[1] * v[1] + u[2] * v[2];
-  const double N = n[0] * n[0] + n[1] * n[1] + n[2] * n[2];
-  const double gam = 1.0 / sqrt(N), iN = gam * gam;
-  const double sg = g >= 0.0 ? 1.0 : -1.0;
-  const double h = 0.5 * g * iN;
-  // z-space gradients of g and N: (n, v x w, w x u) and (0, 2 vv u - 2 uv v, 2 uu v - 2 uv u)
-  const double gg[3][3] = {{n[0], n[1], n[2]},
-                           {v[1] * w[2] - v[2] * w[1], v[2] * w[0] - v[0] * w[2], v[0] * w[1] - v[1] * w[0]},
-                           {w[1] * u[2] - w[2] * u[1], w[2] * u[0] - w[0] * u[2], w[0] * u[1] - w[1] * u[0]}};
-  double gN[3][3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    gN[0][k] = 0.0;
-    gN[1][k] = 2.0 * vv * u[k] - 2.0 * uv * v[k];
-    gN[2][k] = 2.0 * uu * v[k] - 2.0 * uv * u[k];
-  }
-  const double sgam = sg * gam;
-#pragma unroll
-  for (int m = 0; m < 3; ++m)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) gd[3 * m + k] = sgam * (gg[m][k] - h * gN[m][k]);
-  // y-space vectors
-  double e[3][3], gNY[3][3], q[3][3];
-#pragma unroll
-  for (int b = 0; b < 3; ++b)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      gNY[b][k] = M[1][b] * gN[1][k] + M[2][b] * gN[2][k];
-      e[b][k] = M[0][b] * gg[0][k] + M[1][b] * gg[1][k] + M[2][b] * gg[2][k] - h * gNY[b][k];
-      q[b][k] = M[2][b] * u[k] - M[1][b] * v[k];
-    }
-  const double s1 = kb1 * sgam;
-  const double A1 = kb2 * iN, B1 = -0.5 * s1 * iN, C1 = 0.5 * h * s1 * iN;
-  const double kN = -2.0 * s1 * h;  // times hess N / 2
-  const double kg = s1;             // times hess g
-  double U[3][3], W[3][3];
-#pragma unroll
-  for (int b = 0; b < 3; ++b)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      U[b][k] = A1 * e[b][k] + B1 * gNY[b][k];
-      W[b][k] = B1 * e[b][k] + C1 * gNY[b][k];
-    }
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = a; b < 3; ++b) {
-      const double G = q[a][0] * q[b][0] + q[a][1] * q[b][1] + q[a][2] * q[b][2];
-      double X[3][3];  // [r]x part of the off-diagonal blocks
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) X[i][j] = 0.0;
-      if (a < b) {
-        const double mu = M[2][a] * M[1][b] - M[1][a] * M[2][b];
-        const double m01 = M[0][a] * M[1][b] - M[1][a] * M[0][b];
-        const double m02 = M[0][a] * M[2][b] - M[2][a] * M[0][b];
-        const double m12 = M[1][a] * M[2][b] - M[2][a] * M[1][b];
-        double r[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) r[k] = kg * (m02 * u[k] - m01 * v[k] - m12 * w[k]) + kN * mu * n[k];
-        X[0][1] = -r[2];
-        X[0][2] = r[1];
-        X[1][0] = r[2];
-        X[1][2] = -r[0];
-        X[2][0] = -r[1];
-        X[2][1] = r[0];
-      }
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = (a == b ? i : 0); j < 3; ++j) {
-          double val = e[a][i] * U[b][j] + gNY[a][i] * W[b][j] - kN * q[b][i] * q[a][j] + X[i][j];
-          if (i == j) val += kN * G;
-          Bq[tri_idx(3 * a + i, 3 * b + j, 9)] = val;
-        }
-    }
 }
 
 __device__ __forceinline__ int64_t find_block(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
@@ -778,7 +564,7 @@ __device__ __forceinline__ int64_t find_block(const int32_t* __restrict__ row_pt
 
 struct HessArgs {
   int64_t na;
-  const uint32_t* __restrict__ order;  // prep thread -> active pair index
+  const uint32_t* __restrict__ order;  // thread -> active pair index
   const uint32_t* __restrict__ aidx;
   const uint64_t* __restrict__ cand;
   const double* __restrict__ cd;
@@ -800,17 +586,12 @@ struct HessArgs {
   double* __restrict__ val;
   double* __restrict__ grad;
   unsigned long long* __restrict__ status;
-  // reduced matrices handed to the projection kernels: B packed upper
-  // triangle, element-major ([e * cap + slot]); slot -> active pair index
+  unsigned int* __restrict__ n9;   // face / line-line pairs (and mollified ones)
+  unsigned int* __restrict__ n6;   // point-edge pairs nearly on the edge's line (|w| |u| > 64 |u x w|)
+  unsigned int* __restrict__ n4;   // the other point-edge pairs
+  // CB_EE_MOLLIFIER: the queued 9x9 matrices of the mollified pairs, packed upper triangle, element-major
+  // ([e * cap + slot], slot = the pair's place in mlist)
   double* __restrict__ B9;
-  double* __restrict__ B6;
-  double* __restrict__ B4;        // point-edge pairs in their own frame: p, r, Y (7), 2x2 (3), frame (9)
-  uint32_t* __restrict__ slot9;
-  uint32_t* __restrict__ slot6;
-  uint32_t* __restrict__ slot4;
-  unsigned int* __restrict__ n9;
-  unsigned int* __restrict__ n6;
-  unsigned int* __restrict__ n4;
   int64_t cap;
   // CB_EE_MOLLIFIER: pairs handled by k_moll_hess (hmoll null: none)
   const uint8_t* __restrict__ hmoll;
@@ -820,108 +601,46 @@ struct HessArgs {
 };
 
 
-__device__ __forceinline__ void add_block(const HessArgs& A, int r, int c, const double* blk, bool transpose) {
-  const int64_t bi = find_block(A.row_ptr, A.col, r, c);
-  if (bi >= A.row_ptr[r + 1] || A.col[bi] != c) {
-    atomicOr(A.status, (unsigned long long)CB_DEV_CAPACITY);  // pattern miss: never expected
+// entries c[0..NC) of row r: their block indices, -1 where the pattern has none
+// (the searches advance together, so their loads overlap)
+template <int NC>
+__device__ __forceinline__ void find_blocks(const HessArgs& A, int r, const int (&c)[NC], int64_t (&out)[NC]) {
+  const int b = A.row_ptr[r], e = A.row_ptr[r + 1];
+  int lo[NC], hi[NC];
+#pragma unroll
+  for (int k = 0; k < NC; ++k) {
+    lo[k] = b;
+    hi[k] = e;
+  }
+  for (int len = e - b; len > 0; len >>= 1) {
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      if (lo[k] >= hi[k]) continue;
+      const int mid = (lo[k] + hi[k]) >> 1;
+      if (A.col[mid] < c[k]) lo[k] = mid + 1;
+      else hi[k] = mid;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < NC; ++k) out[k] = lo[k] < e && A.col[lo[k]] == c[k] ? (int64_t)lo[k] : -1;
+}
+
+// a 3x3 block into the BSR values (transposed if tr); a pattern miss is never expected
+__device__ __forceinline__ void add_block(const HessArgs& A, int64_t bi, const double (&blk)[9], bool tr) {
+  if (bi < 0) {
+    atomicOr(A.status, (unsigned long long)CB_DEV_CAPACITY);
     return;
   }
   double* dst = A.val + 9 * bi;
-  for (int al = 0; al < 3; ++al)
-    for (int be = 0; be < 3; ++be) atomicAdd(&dst[3 * al + be], transpose ? blk[3 * be + al] : blk[3 * al + be]);
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) atomicAdd(&dst[3 * i + j], tr ? blk[3 * j + i] : blk[3 * i + j]);
 }
 
-// The reduced matrix of one pair, B = c1 gB gB^T + c2 (M x I)^T hess s (M x I)
-// with gB = (M x I)^T grad d, written as a packed upper triangle into the
-// queue (element-major: entry e of slot at e * cap + slot).  D = 9 goes with
-// three z-vectors (plane types), D = 6 with two (point-edge).
-template <int D, int NZ>
-__host__ __device__ __forceinline__ void write_reduced(double* __restrict__ Bo, int64_t cap, unsigned slot,
-                                              const double (&M)[3][3], const double* gd, const double* Hs,
-                                              double c1, double c2) {
-  constexpr int NB = D / 3;
-  double gB[D];
-#pragma unroll
-  for (int ab = 0; ab < NB; ++ab)
-#pragma unroll
-    for (int al = 0; al < 3; ++al) {
-      double v = 0.0;
-#pragma unroll
-      for (int m = 0; m < NZ; ++m) v += M[m][ab] * gd[3 * m + al];
-      gB[3 * ab + al] = v;
-    }
-#pragma unroll
-  for (int row = 0; row < D; ++row) {
-    const int ab = row / 3, al = row % 3;
-#pragma unroll
-    for (int col = row; col < D; ++col) {
-      const int bb = col / 3, be = col % 3;
-      double h = 0.0;
-#pragma unroll
-      for (int m = 0; m < NZ; ++m) {
-        double hm = 0.0;
-#pragma unroll
-        for (int m2 = 0; m2 < NZ; ++m2) hm += M[m2][bb] * Hs[(3 * m + al) * 9 + 3 * m2 + be];
-        h += M[m][ab] * hm;
-      }
-      Bo[(size_t)tri_idx(row, col, D) * cap + slot] = c1 * gB[row] * gB[col] + c2 * h;
-    }
-  }
-}
-
-// Point-edge pairs in their own frame: the 6x6 reduced matrix (rows 3 ab + al,
-// al the local axis) has no coupling between the e3 rows (2, 5) and the
-// rest, so it splits into an in-plane 4x4 block (rows 0, 1, 3, 4) and an
-// out-of-plane 2x2 block (rows 2, 5).
-// At w' = (wx, wy, 0), u' = (lu, 0, 0) the Hessian of s = |w|^2 - (w.u)^2/|u|^2
-// has, per pair of axes, these 2x2 blocks over (w, u) (rows: first axis):
-//   (x, x): 0;  (x, y): [[0, -2 wy/lu], [0, 2 wx wy/lu^2]];  (y, x): its transpose;
-//   (y, y): [[2, -2 wx/lu], [-2 wx/lu, 2 (wx^2 - wy^2)/lu^2]];
-//   (z, z): [[2, -2 wx/lu], [-2 wx/lu, 2 wx^2/lu^2]];  the rest 0,
-// and grad d = (g0, g1) on the y axis only.  With H_z = c1 grad d grad d^T +
-// c2 hess s, block (ab, al; bb, be) of B is (M^T H_z[al, be] M)[ab][bb].  So
-// the 4x4 block, in the order (x of both reduced points, y of both), is
-//   [[0, p r^T], [r p^T, Y]],  p_ab = M[0][ab] hxy01 + M[1][ab] hxy11,
-//   r_bb = M[1][bb],  Y = (M^T H_z[y, y] M)
-// (the (x, x) block is zero and the (x, y) block has rank one).  Queued:
-// p (2), r (2), Y (3, packed), the 2x2 block (3, packed) and the frame R
-// (row-major, columns e1 e2 e3; 9).  il = 1 / lu.
-__device__ __forceinline__ void write_reduced_pe_local(double* __restrict__ Bo, int64_t cap, unsigned slot,
-                                                       const double (&M)[3][3], double g0, double g1, double wx,
-                                                       double wy, double il, double c1, double c2,
-                                                       const double (&Rf)[9]) {
-  const double hxy01 = c2 * (-2.0 * wy * il), hxy11 = c2 * (2.0 * wx * wy * il * il);
-  const double hwu = -2.0 * wx * il;
-  const double Hyy[2][2] = {{c1 * g0 * g0 + 2.0 * c2, c1 * g0 * g1 + c2 * hwu},
-                            {c1 * g0 * g1 + c2 * hwu, c1 * g1 * g1 + c2 * 2.0 * (wx * wx - wy * wy) * il * il}};
-  const double Hzz[2][2] = {{2.0 * c2, c2 * hwu}, {c2 * hwu, c2 * 2.0 * wx * wx * il * il}};
-  auto mhm = [&](const double (&H)[2][2], int ab, int bb) {
-    double v = 0.0;
-#pragma unroll
-    for (int m = 0; m < 2; ++m)
-#pragma unroll
-      for (int m2 = 0; m2 < 2; ++m2) v += M[m][ab] * H[m][m2] * M[m2][bb];
-    return v;
-  };
-  const double e[10] = {M[0][0] * hxy01 + M[1][0] * hxy11,
-                        M[0][1] * hxy01 + M[1][1] * hxy11,
-                        M[1][0],
-                        M[1][1],
-                        mhm(Hyy, 0, 0),
-                        mhm(Hyy, 0, 1),
-                        mhm(Hyy, 1, 1),
-                        mhm(Hzz, 0, 0),
-                        mhm(Hzz, 0, 1),
-                        mhm(Hzz, 1, 1)};
-#pragma unroll
-  for (int k = 0; k < 10; ++k) Bo[(size_t)k * cap + slot] = e[k];
-#pragma unroll
-  for (int k = 0; k < 9; ++k) Bo[(size_t)(10 + k) * cap + slot] = Rf[k];
-}
-
-// Active pairs in the order k_hess_prep takes them: face / line-line pairs
+// Active pairs in the order k_pair_hess takes them: face / line-line pairs
 // (the branch with the most FP64 work) first, the other pairs from the end
-// backwards, so that a warp of the prep kernel runs one branch rather than
+// backwards, so that a warp of that kernel runs one branch rather than
 // both with few lanes each.  Warp-aggregated appends; inside each group the
 // order follows warp arrival.
 struct MollArgs {                   // CB_EE_MOLLIFIER scenes only (mp null: no mollifier)
@@ -949,7 +668,7 @@ __global__ void k_kind_split(int64_t na, const uint32_t* __restrict__ aidx, cons
     plane = (cb_key_type(key) == CB_KEY_PT ? c_pt_types[ty] : c_ee_types[ty]).kind == 2;
     if (MA.mp && cb_key_type(key) != CB_KEY_PT) {
       // edge-edge pair below its mollifier threshold: its energy, gradient
-      // and 9x9 matrix come from k_moll_hess instead of k_hess_prep
+      // and 9x9 matrix come from k_moll_hess instead of k_pair_hess
       const uint32_t i = cb_key_i(key), j = cb_key_j(key);
       const int a0 = MA.ev0[i], a1 = MA.ev1[i], b0 = MA.ev0[j], b1 = MA.ev1[j];
       if (MA.mp[MA.vsc[a0]].mollify) {
@@ -977,46 +696,34 @@ __global__ void k_kind_split(int64_t na, const uint32_t* __restrict__ aidx, cons
   }
 }
 
-// Stage (d), part 1, one thread per active pair: barrier value and
-// derivatives, energy, gradient scatter, and the Hessian in the orthonormal
-// translation-free basis of the points the distance type involves,
-// B = (M x I)^T H_z (M x I) with M = C K.  Point-point stencils are projected
-// in closed form here; the others are queued for the projection kernels.
-__global__ void __launch_bounds__(128) k_hess_prep(HessArgs A) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// Stage (d), one thread per active pair: barrier value and derivatives,
+// energy, gradient scatter, the PSD-projected Hessian in closed form
+// (pairhess.cuh) and its scatter into the BSR values.  PAIR_T threads a block:
+// the work is a few hundred to a thousand FP64 instructions per warp, of which
+// an SM completes one per ~19 cycles with four warps resident, so small blocks
+// spread a short list over more SMs and cost a long one nothing.
+constexpr int PAIR_T = 64;
+
+// v[i] for an index known only at run time, without a local-memory array
+__device__ __forceinline__ int pick(const int (&v)[4], int i) {
+  return i == 0 ? v[0] : (i == 1 ? v[1] : (i == 2 ? v[2] : v[3]));
+}
+
+__global__ void __launch_bounds__(PAIR_T) k_pair_hess(HessArgs A) {
+  const int64_t t = (int64_t)blockIdx.x * PAIR_T + threadIdx.x;
   int64_t a = t < A.na ? (int64_t)A.order[t] : A.na;
   if (A.hmoll && a < A.na && A.hmoll[a]) a = A.na;  // mollified edge-edge pair: k_moll_hess
   double e_local = 0.0;
-  int mem = -1;
-  int want = 0;  // 9 or 6: reduced dimension of the queued matrix
-  // the reduced matrix (packed upper triangle), written once the queue slot is known
-  double Bq[45];
-  double gd[9], M[3][3], Rf[9];
-  double c1 = 0.0, c2 = 0.0;
-  int nz = 0;
+  int mem = -1, counted = 0;  // 9, 6, 4: the statistics' kinds
   if (a < A.na) {
     const uint32_t c = A.aidx[a];
-    const uint64_t key = A.cand[c];
-    Stencil s = stencil_of(key, A.ev0, A.ev1, A.tv, A.T);
+    const Stencil s = stencil_of(A.cand[c], A.ev0, A.ev1, A.tv, A.T);
     const int ty = A.ctype[c];
     const TypeInfo& TI = s.ee ? c_ee_types[ty] : c_pt_types[ty];
     const int kind = TI.kind;
-    nz = kind + 1;
     d3 X[4];
+#pragma unroll
     for (int i = 0; i < 4; ++i) X[i] = load3(A.x, A.n, s.v[i]);
-    d3 Pl[4];
-    for (int i = 0; i < 4; ++i) Pl[i] = mk3(X[i].x - X[0].x, X[i].y - X[0].y, X[i].z - X[0].z);
-    d3 z[3];
-    for (int m = 0; m < 3; ++m) {
-      double zx = 0, zy = 0, zz = 0;
-      for (int i = 1; i < 4; ++i) {
-        const double cm = (double)TI.C[m][i];
-        zx += cm * Pl[i].x;
-        zy += cm * Pl[i].y;
-        zz += cm * Pl[i].z;
-      }
-      z[m] = mk3(zx, zy, zz);
-    }
     const double d = A.cd[c];
     mem = A.vsc[s.v[0]];
     const PassParams P = member_pass(A.mp[mem]);
@@ -1025,153 +732,154 @@ __global__ void __launch_bounds__(128) k_hess_prep(HessArgs A) {
     const double y = d - xi_p;
     double b, b1, b2;
     barrier_b012(y, dh_p, b, b1, b2);
-    const double kap = P.kappa;
-    e_local = kap * b;
-    // Point-edge: in the frame e1 along the edge (u), e3 normal to the plane
-    // of the edge and the point (u x w), the configuration is symmetric under
-    // e3 -> -e3, so hess s and grad d have no coupling between the e3
-    // components and the others: the reduced matrix splits into an in-plane
-    // 4x4 and an out-of-plane 2x2 block.  Evaluated at the local coordinates
-    // w' = (w.e1, w.e2, 0), u' = (|u|, 0, 0) the coupling entries are exactly
-    // zero.  The frame's direction error is about 1e-16 |w| |u| / |u x w|;
-    // beyond a ratio of 64 the pair stays on the generic 6x6 path.
-    bool pe_local = false;
-    d3 zl[3];
-    double piu = 0.0;  // 1 / |u| of a point-edge pair in its frame
-    if (kind == 1) {
-      const d3 w = z[0], u = z[1];
-      const d3 n = mk3(u.y * w.z - u.z * w.y, u.z * w.x - u.x * w.z, u.x * w.y - u.y * w.x);
-      // squared lengths; the conditioning test |w||u| <= 64 |u x w| squared
-      const double nn2 = n.x * n.x + n.y * n.y + n.z * n.z;
-      const double uu2 = u.x * u.x + u.y * u.y + u.z * u.z;
-      const double ww2 = w.x * w.x + w.y * w.y + w.z * w.z;
-      if (nn2 > 0.0 && ww2 * uu2 <= 4096.0 * nn2) {
-        const double iu = rsqrt(uu2), inn = rsqrt(nn2), lu = uu2 * iu;
-        piu = iu;
-        const d3 e1 = mk3(u.x * iu, u.y * iu, u.z * iu), e3 = mk3(n.x * inn, n.y * inn, n.z * inn);
-        const d3 e2 = mk3(e3.y * e1.z - e3.z * e1.y, e3.z * e1.x - e3.x * e1.z, e3.x * e1.y - e3.y * e1.x);
-        zl[0] = mk3(w.x * e1.x + w.y * e1.y + w.z * e1.z, w.x * e2.x + w.y * e2.y + w.z * e2.z, 0.0);
-        zl[1] = mk3(lu, 0.0, 0.0);
-        zl[2] = mk3(0.0, 0.0, 0.0);
-        Rf[0] = e1.x; Rf[1] = e2.x; Rf[2] = e3.x;
-        Rf[3] = e1.y; Rf[4] = e2.y; Rf[5] = e3.y;
-        Rf[6] = e1.z; Rf[7] = e2.z; Rf[8] = e3.z;
-        pe_local = true;
+    e_local = P.kappa * b;
+    const double g1 = P.kappa * b1, beta = P.kappa * b2;
+    const bool out = y > 0.0;  // inside the offset the energy is +inf and the pair adds no Hessian
+    double z[3][3];
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      double zx = 0, zy = 0, zz = 0;
+#pragma unroll
+      for (int i = 1; i < 4; ++i) {
+        const double cm = (double)TI.C[m][i];
+        zx += cm * (X[i].x - X[0].x);
+        zy += cm * (X[i].y - X[0].y);
+        zz += cm * (X[i].z - X[0].z);
       }
+      z[m][0] = zx;
+      z[m][1] = zy;
+      z[m][2] = zz;
     }
-    const double i2d = 0.5 / d;
-    c1 = kap * (b2 - b1 * (2.0 * i2d));
-    c2 = kap * b1 * i2d;
-    if (kind > 0) {
-      // M = C K: the z-vectors in the orthonormal translation-free basis of
-      // the points the type involves
-      int pts[4], np = 0;
-      for (int i = 0; i < 4; ++i) {
-        bool used = false;
-        for (int m = 0; m < nz; ++m) used |= TI.C[m][i] != 0;
-        if (used) pts[np++] = i;
+    auto grad_add = [&](int v, double cw, const double (&n)[3]) {
+#pragma unroll
+      for (int al = 0; al < 3; ++al) atomicAdd(&A.grad[(size_t)al * A.n + v], g1 * cw * n[al]);
+    };
+    if (kind == 2) {
+      counted = 9;
+      cbh::PlaneBlocks Q;
+      cbh::plane_blocks(s.ee, z[0], z[1], z[2], d, beta, -g1, Q);
+      if (A.grad)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) grad_add(s.v[q], Q.c[q], Q.n);
+      if (out) {
+        int64_t at[4][4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) find_blocks<4>(A, s.v[q], s.v, at[q]);
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+          for (int r = p; r < 4; ++r) {
+            double blk[9];
+            cbh::plane_block(Q, p, r, blk);
+            add_block(A, at[p][r], blk, false);
+            if (r > p) add_block(A, at[r][p], blk, true);
+          }
       }
-      const int nb = np - 1;
-      for (int m = 0; m < 3; ++m)
-        for (int bb = 0; bb < 3; ++bb) {
-          double v = 0.0;
-          if (m < nz && bb < nb)
-            for (int q = 0; q < np; ++q)
-              v += (double)TI.C[m][pts[q]] * (np == 4 ? c_K4[q][bb] : c_K3[q][bb]);
-          M[m][bb] = v;
+    } else if (kind == 1) {
+      // r = w - t u with one rounding per component, its part along u (t's rounding) then removed: n keeps full
+      // accuracy however close the point lies to the edge
+      const double(&w)[3] = z[0];
+      const double(&u)[3] = z[1];
+      const double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2], iu = rsqrt(uu), iuu = iu * iu;
+      double tp = (w[0] * u[0] + w[1] * u[1] + w[2] * u[2]) * iuu, r[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) r[k] = fma(-tp, u[k], w[k]);
+      const double dt = (r[0] * u[0] + r[1] * u[1] + r[2] * u[2]) * iuu;
+      tp += dt;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) r[k] = fma(-dt, u[k], r[k]);
+      const double rr = r[0] * r[0] + r[1] * r[1] + r[2] * r[2], ir = rsqrt(rr);
+      const double ww = w[0] * w[0] + w[1] * w[1] + w[2] * w[2];
+      counted = ww <= 4096.0 * rr ? 4 : 6;
+      cbh::EdgeBlocks Q;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        Q.n[k] = r[k] * ir;
+        Q.e[k] = u[k] * iu;
+      }
+      cbh::edge_blocks(tp, iu, d, beta, -g1, Q);
+      // the stencil points q, e0, e1: w = q - e0, u = e1 - e0, up to the sign of both
+      int v3[3];
+      {
+        int qi = 0, ai = 0, bi = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int cw = TI.C[0][i], cu = TI.C[1][i];
+          if (cw > 0) qi = i;
+          if (cw < 0) ai = i;
+          if (cu > 0) bi = i;
         }
-    }
-    if (pe_local) {
-      // In the frame (w' = (wx, wy, 0), u' = (lu, 0, 0), s = wy^2) grad s has
-      // only the y components 2 wy (w) and -2 wx wy / lu (u); hess s is
-      // formed in write_reduced_pe_local
-      const double pwx = zl[0].x, pwy = zl[0].y;
-      for (int k = 0; k < 9; ++k) gd[k] = 0.0;
-      gd[1] = 2.0 * pwy * i2d;
-      gd[4] = -2.0 * pwx * pwy * piu * i2d;
-      write_reduced_pe_local(Bq, 1, 0, M, gd[1], gd[4], pwx, pwy, piu, c1, c2, Rf);
-      want = 4;
-    } else if (kind == 2) {
-      const double zz[3][3] = {{z[0].x, z[0].y, z[0].z}, {z[1].x, z[1].y, z[1].z}, {z[2].x, z[2].y, z[2].z}};
-      plane_reduced(zz, M, kap * b1, kap * b2, gd, Bq);
-      want = 9;
+        v3[0] = pick(s.v, qi);
+        v3[1] = pick(s.v, ai);
+        v3[2] = pick(s.v, bi);
+      }
+      if (A.grad)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) grad_add(v3[q], Q.c[q], Q.n);
+      if (out) {
+        int64_t at[3][3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) find_blocks<3>(A, v3[q], v3, at[q]);
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+#pragma unroll
+          for (int q = p; q < 3; ++q) {
+            double blk[9];
+            cbh::edge_block(Q, p, q, blk);
+            add_block(A, at[p][q], blk, false);
+            if (q > p) add_block(A, at[q][p], blk, true);
+          }
+      }
     } else {
-      double gs[9], Hs[81];
-      s_derivs(kind, z, gs, Hs);
-      for (int k = 0; k < 9; ++k) gd[k] = gs[k] * i2d;
-      if (kind == 1) {
-        write_reduced<6, 2>(Bq, 1, 0, M, gd, Hs, c1, c2);
-        want = 6;
+      // point-point: kappa b'' n n^T + (kappa b'/d)(I - n n^T), each part clamped
+      const double id = 1.0 / d;
+      const double n[3] = {z[0][0] * id, z[0][1] * id, z[0][2] * id};
+      int v2[2];
+      {
+        int pi = 0, mi = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (TI.C[0][i] > 0) pi = i;
+          if (TI.C[0][i] < 0) mi = i;
+        }
+        v2[0] = pick(s.v, pi);
+        v2[1] = pick(s.v, mi);
       }
-    }
-    if (A.grad) {
-      // grad d in world axes (rotated back from the frame when in it)
-      double gw[9];
-      for (int m = 0; m < 3; ++m)
+      if (A.grad) {
+        grad_add(v2[0], 1.0, n);
+        grad_add(v2[1], -1.0, n);
+      }
+      if (out) {
+        const double lam_n = fmax(beta, 0.0), lam_t = fmax(g1 * id, 0.0);
+        double blk[9], neg[9];
+#pragma unroll
         for (int i = 0; i < 3; ++i)
-          gw[3 * m + i] = pe_local ? Rf[3 * i] * gd[3 * m] + Rf[3 * i + 1] * gd[3 * m + 1] + Rf[3 * i + 2] * gd[3 * m + 2]
-                                   : gd[3 * m + i];
-      for (int i = 0; i < 4; ++i) {
-        bool used = false;
-        for (int m = 0; m < nz; ++m) used |= TI.C[m][i] != 0;
-        if (!used) continue;
-        for (int al = 0; al < 3; ++al) {
-          double v = 0.0;
-          for (int m = 0; m < nz; ++m) v += (double)TI.C[m][i] * gw[3 * m + al];
-          atomicAdd(&A.grad[(size_t)al * A.n + s.v[i]], kap * b1 * v);
-        }
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            blk[3 * i + j] = lam_n * n[i] * n[j] + lam_t * ((i == j ? 1.0 : 0.0) - n[i] * n[j]);
+            neg[3 * i + j] = -blk[3 * i + j];
+          }
+        int64_t at[2][2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) find_blocks<2>(A, v2[q], v2, at[q]);
+        add_block(A, at[0][0], blk, false);
+        add_block(A, at[1][1], blk, false);
+        add_block(A, at[0][1], neg, false);
+        add_block(A, at[1][0], neg, false);
       }
-    }
-    if (kind == 0) {
-      // point-point: H_z = kappa b'' n n^T + (kappa b'/d)(I - n n^T); clamp each part
-      const double nh[3] = {gd[0], gd[1], gd[2]};
-      const double lam_n = fmax(kap * b2, 0.0), lam_t = fmax(kap * b1 * (2.0 * i2d), 0.0);
-      double Hz[9];
-      for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j)
-          Hz[3 * i + j] = lam_n * nh[i] * nh[j] + lam_t * ((i == j ? 1.0 : 0.0) - nh[i] * nh[j]);
-      for (int i = 0; i < 4; ++i)
-        for (int j = 0; j < 4; ++j) {
-          const int cc = TI.C[0][i] * TI.C[0][j];
-          if (cc == 0) continue;
-          double blk[9];
-          for (int q = 0; q < 9; ++q) blk[q] = (double)cc * Hz[q];
-          add_block(A, s.v[i], s.v[j], blk, false);
-        }
     }
   }
-  // queue slot (warp-aggregated allocation), then the reduced matrix, packed
-  // upper triangle, element-major (point-edge pairs in their frame: the
-  // 4x4 and 2x2 blocks and the frame)
-  const unsigned lane = threadIdx.x & 31;
-  const unsigned lt = (1u << lane) - 1u;
-  unsigned slot = 0;
 #pragma unroll
   for (int which = 0; which < 3; ++which) {
-    const int Dw = which == 0 ? 9 : (which == 1 ? 6 : 4);
-    const unsigned m = __ballot_sync(0xffffffffu, want == Dw);
-    if (!m) continue;
-    unsigned base = 0;
-    const int leader = __ffs(m) - 1;
-    if ((int)lane == leader)
-      base = atomicAdd(which == 0 ? A.n9 : (which == 1 ? A.n6 : A.n4), (unsigned)__popc(m));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (want == Dw) slot = base + __popc(m & lt);
-  }
-  if (want != 0) {
-    double* Bo = want == 9 ? A.B9 : (want == 6 ? A.B6 : A.B4);
-    const int ne = want == 9 ? 45 : (want == 6 ? 21 : 19);
-#pragma unroll
-    for (int e = 0; e < 45; ++e)
-      if (e < ne) Bo[(size_t)e * A.cap + slot] = Bq[e];
-    (want == 9 ? A.slot9 : (want == 6 ? A.slot6 : A.slot4))[slot] = (uint32_t)a;
+    const unsigned m = __ballot_sync(0xffffffffu, counted == (which == 0 ? 9 : (which == 1 ? 6 : 4)));
+    if (m && (threadIdx.x & 31) == 0) atomicAdd(which == 0 ? A.n9 : (which == 1 ? A.n6 : A.n4), (unsigned)__popc(m));
   }
   member_energy_add(A.macc, mem, e_local);
 }
 
 // ---- IPC's edge-edge mollifier (CB_EE_MOLLIFIER) -------------------------
 // A mollified pair's energy m(c) kappa b(d) depends on all four points
-// whatever its distance type, so it leaves the reduced paths of k_hess_prep.
+// whatever its distance type, so it leaves the closed forms of k_pair_hess.
 // Its gradient and Hessian are formed here from analytic derivatives of the
 // typed distance d and of c = |e0 x e1|^2, written in the difference vectors
 // the distance is a function of and mapped to the four points:
@@ -1186,7 +894,7 @@ __global__ void __launch_bounds__(128) k_hess_prep(HessArgs A) {
 //   H = kappa (m (b'' gd gd^T + b' Hd) + b' m' (gc gd^T + gd gc^T)
 //              + b (m'' gc gc^T + m' Hc)),
 // and the 9x9 matrix of the four-point translation-free basis
-// (B = (K4 x I)^T H (K4 x I)) is queued for k_hess_proj<9>.
+// (B = (K4 x I)^T H (K4 x I)) is queued for the 9x9 projection.
 struct LocalDeriv {
   int nb;                  // difference vectors (blocks of 3)
   int plus[3], minus[3];   // block b = x[plus[b]] - x[minus[b]] (stencil points 0..3)
@@ -1427,11 +1135,11 @@ __global__ void __launch_bounds__(128) k_moll_hess(HessArgs A) {
             if (i != j) Bf[(3 * p2 + be) * 9 + 3 * p1 + al] += w;
           }
       }
-    const unsigned slot = atomicAdd(A.n9, 1u);
     for (int i = 0; i < 9; ++i)
-      for (int j = i; j < 9; ++j) A.B9[(size_t)tri_idx(i, j, 9) * A.cap + slot] = Bf[i * 9 + j];
-    A.slot9[slot] = a;
+      for (int j = i; j < 9; ++j) A.B9[(size_t)tri_idx(i, j, 9) * A.cap + t] = Bf[i * 9 + j];
   }
+  const unsigned mm = __ballot_sync(0xffffffffu, mem >= 0);
+  if (mm && (threadIdx.x & 31) == 0) atomicAdd(A.n9, (unsigned)__popc(mm));
   member_energy_add(A.macc, mem, e_local);
 }
 
@@ -1662,16 +1370,12 @@ __device__ __forceinline__ void hadamard_scatter(const HessArgs& A, const Stenci
     }
 }
 
-template <int D>
-struct ProjSmem {
-  static constexpr int NP = D * (D + 1) / 2;
-  // per thread: V (D*D doubles, column-major; the FP32 eigenvectors occupy its
-  // first D*D floats during the FP32 phase) | A (NP doubles; the FP32 matrix in
-  // its first NP floats during the FP32 phase, then the FP64 matrix, then B+)
-  static constexpr int PER_THREAD = (D * D + NP) * 8;
-};
+// per thread: V (D*D doubles, column-major; the FP32 eigenvectors occupy its
+// first D*D floats during the FP32 phase) | A (D(D+1)/2 doubles; the FP32 matrix
+// in its first floats during the FP32 phase, then the FP64 matrix, then B+)
+constexpr int PROJ_SMEM = (81 + 45) * 8;
 
-// Stage (d), part 2, one thread per queued pair: PSD projection of the D x D
+// Mollified pairs, one thread per queued pair: PSD projection of the 9x9
 // reduced matrix and the BSR scatter.  The input B stays in registers; the
 // eigenvectors V and the working matrix A live in shared memory laid out
 // element-major ([element][thread]), so a warp touches 32 consecutive words
@@ -1682,12 +1386,12 @@ struct ProjSmem {
 // Projection onto the PSD cone is non-expansive in the Frobenius norm, so the
 // projected matrix is exact to 1e-14 of ||B||.  B+ is mapped back to the
 // involved points with K (x) I and scattered.
-template <int D, int S>
+template <int S>
 __global__ void __launch_bounds__(S) k_hess_proj(HessArgs A) {
-  constexpr int NP = D * (D + 1) / 2;
+  constexpr int D = 9, NP = D * (D + 1) / 2;
   extern __shared__ double smem[];
   const int tid = threadIdx.x;
-  const int64_t m = (int64_t)*(D == 9 ? A.n9 : A.n6);
+  const int64_t m = (int64_t)*A.nmoll;
   // grid-stride over the queue, S pairs per step; the loop bound is the same
   // for every thread of a block, and a thread past the end leaves only in the
   // block's last step, after its last barrier
@@ -1701,14 +1405,13 @@ __global__ void __launch_bounds__(S) k_hess_proj(HessArgs A) {
     float* V32 = (float*)smem + tid;                    // FP32 V, same indexing, inside the V region
     float* A32 = (float*)(smem + D * D * S) + tid;      // FP32 A, same indexing, inside the A region
     const bool act = w < m;                             // no early exit before the last barrier
-    const double* Bg = D == 9 ? A.B9 : A.B6;
-    const uint32_t a = act ? (D == 9 ? A.slot9 : A.slot6)[w] : 0u;
+    const uint32_t a = act ? A.mlist[w] : 0u;
     // B stays in registers until B+ is formed
     double Br[NP];
     double mx = 0.0;
 #pragma unroll
     for (int e = 0; e < NP; ++e) {
-      Br[e] = act ? Bg[(size_t)e * A.cap + w] : 0.0;
+      Br[e] = act ? A.B9[(size_t)e * A.cap + w] : 0.0;
       mx = fmax(mx, fabs(Br[e]));
     }
     const bool work = act && mx != 0.0;
@@ -1790,8 +1493,8 @@ __global__ void __launch_bounds__(S) k_hess_proj(HessArgs A) {
     const bool from_b = nneg < npos;
     const int nterm = from_b ? nneg : npos;
     const int wterm = __reduce_max_sync(__activemask(), nterm);
-    double* Bs = Ad;  // B+ replaces A (for D = 9 scaled by 1/4, the square of K4's entries)
-    constexpr double bsc = D == 9 ? 0.25 : 1.0;
+    double* Bs = Ad;  // B+ replaces A (scaled by 1/4, the square of K4's entries)
+    constexpr double bsc = 0.25;
 #pragma unroll
     for (int e = 0; e < NP; ++e) Bs[e * S] = from_b ? Br[e] * bsc : 0.0;
     for (int j = 0; j < wterm; ++j) {
@@ -1819,53 +1522,7 @@ __global__ void __launch_bounds__(S) k_hess_proj(HessArgs A) {
     }
     const uint32_t c = A.aidx[a];
     const Stencil st = stencil_of(A.cand[c], A.ev0, A.ev1, A.tv, A.T);
-    if constexpr (D == 9) {
-      // the plane types involve all four points, in stencil order
-      hadamard_scatter(A, st, Bs, S);
-    } else {
-      // scatter: block (q1, q2) of the involved points
-      //   = sum_ab K[q1][ab] R[q2][ab],  R[q2][ab] = sum_bb K[q2][bb] B+[ab, bb]
-      // (3x3 blocks; R for one q2 at a time)
-      const TypeInfo& TI = st.ee ? c_ee_types[A.ctype[c]] : c_pt_types[A.ctype[c]];
-      const int nz = TI.kind + 1;
-      int pts[4], np = 0;
-      for (int i = 0; i < 4; ++i) {
-        bool used = false;
-        for (int mm = 0; mm < nz; ++mm) used |= TI.C[mm][i] != 0;
-        if (used) pts[np++] = i;
-      }
-      constexpr int NB = D / 3;
-      for (int q2 = 0; q2 < np; ++q2) {
-        double R[NB][9];
-#pragma unroll
-        for (int ab = 0; ab < NB; ++ab)
-#pragma unroll
-          for (int al = 0; al < 3; ++al)
-#pragma unroll
-            for (int be = 0; be < 3; ++be) {
-              double v = 0.0;
-#pragma unroll
-              for (int bb = 0; bb < NB; ++bb) {
-                const int r = 3 * ab + al, cl = 3 * bb + be;
-                v += c_K3[q2][bb] * Bs[(r <= cl ? tri_idx(r, cl, D) : tri_idx(cl, r, D)) * S];
-              }
-              R[ab][3 * al + be] = v;
-            }
-        for (int q1 = 0; q1 <= q2; ++q1) {
-          double blk[9];
-#pragma unroll
-          for (int e = 0; e < 9; ++e) {
-            double v = 0.0;
-#pragma unroll
-            for (int ab = 0; ab < NB; ++ab) v += c_K3[q1][ab] * R[ab][e];
-            blk[e] = v;
-          }
-          const int r = st.v[pts[q1]], cc = st.v[pts[q2]];
-          add_block(A, r, cc, blk, false);
-          if (q1 != q2) add_block(A, cc, r, blk, true);
-        }
-      }
-    }
+    hadamard_scatter(A, st, Bs, S);
   }
 }
 
@@ -1884,7 +1541,7 @@ __global__ void __launch_bounds__(S) k_hess_proj(HessArgs A) {
 // columns), so a sweep is 9 rounds of 18 FP64 instructions per lane
 // instead of 36 rotations in sequence.  Each lane computes its own row's
 // rotation, the same bits in every lane of the pair's two rows.  The arithmetic is
-// otherwise that of k_hess_proj<9>: FP32 Jacobi on the scaled matrix to
+// otherwise that of k_hess_proj: FP32 Jacobi on the scaled matrix to
 // the same tolerance, FP64 modified Gram-Schmidt, A = V^T B V, FP64 sweeps
 // with FP32 tangents and FP64-normalised rotations to an off-diagonal norm
 // of 1e-14 ||A||, B+ from the positive eigenpairs, the Hadamard scatter.
@@ -1974,20 +1631,20 @@ __device__ __forceinline__ void pl_rotation<double>(const double* As, int r, int
   sg = r == p ? -t * c : t * c;
 }
 
-__device__ __forceinline__ void proj_lanes_block(const HessArgs& A, int block) {
+__global__ void __launch_bounds__(PL_THREADS) k_hess_proj_lanes(HessArgs A) {
   extern __shared__ double pl_smem[];
   const int seg = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r = lane / 3, t = lane - 3 * r;  // row r (< 9 for lanes 0..26), third t
   const bool row = lane < 27;
-  const int64_t w = (int64_t)block * PL_PAIRS + seg;
-  if (w >= (int64_t)*A.n9) return;  // the whole warp leaves together
+  const int64_t w = (int64_t)blockIdx.x * PL_PAIRS + seg;
+  if (w >= (int64_t)*A.nmoll) return;  // the whole warp leaves together
   double* As = pl_smem + (size_t)seg * PL_SMEM;  // A[i][j] at [9 i + j]
   double* Xs = As + 81;                          // A J; later the Hadamard staging
   double* Vs = Xs + 108;                         // V[i][k]: component i of eigenvector k
   float* A32 = (float*)(Vs + 81);
   float* X32 = A32 + 81;
   float* V32 = X32 + 81;
-  const uint32_t a = A.slot9[w];
+  const uint32_t a = A.mlist[w];
   double Br[9];  // row r of B
   double mx = 0.0;
 #pragma unroll
@@ -2139,353 +1796,20 @@ __device__ __forceinline__ void proj_lanes_block(const HessArgs& A, int block) {
   }
 }
 
-// k_hess_proj<D> over at most one resident wave of blocks (the occupancy
-// looked up once per scene)
-template <int D>
+// k_hess_proj over at most one resident wave of blocks (the occupancy looked
+// up once per scene)
 cb_status launch_proj(cb_scene* s, const HessArgs& A, int64_t cap, cudaStream_t st) {
-  const int smem = ProjSmem<D>::PER_THREAD * PROJ_THREADS;
-  int& occ = s->proj_occ[D == 9 ? 0 : 1];
-  CB_CUDA(cudaFuncSetAttribute(k_hess_proj<D, PROJ_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  const int smem = PROJ_SMEM * PROJ_THREADS;
+  int& occ = s->proj_occ;
+  CB_CUDA(cudaFuncSetAttribute(k_hess_proj<PROJ_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   if (occ <= 0) {
-    CB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_hess_proj<D, PROJ_THREADS>, PROJ_THREADS, smem));
+    CB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_hess_proj<PROJ_THREADS>, PROJ_THREADS, smem));
     occ = std::max(1, occ);
   }
   const int64_t g = std::min<int64_t>(cb_grid(cap, PROJ_THREADS), (int64_t)s->n_sms * occ);
-  k_hess_proj<D, PROJ_THREADS><<<(int)std::max<int64_t>(1, g), PROJ_THREADS, smem, cb_count(st)>>>(A);
+  k_hess_proj<PROJ_THREADS><<<(int)std::max<int64_t>(1, g), PROJ_THREADS, smem, cb_count(st)>>>(A);
   CB_CUDA(cudaGetLastError());
   return CB_OK;
-}
-
-// Register-resident versions of the two Jacobi phases for the 4x4 block of
-// the point-edge path: the same arithmetic as jacobi_packed / jacobi_refine64
-// on arrays held in registers (every loop unrolled, every index static).  V
-// is column-major: row i of column k at V[k * D + i].
-template <typename R, int D>
-__device__ __forceinline__ void jacobi_reg(R (&Am)[D * (D + 1) / 2], R (&V)[D * D], const R tol2,
-                                           const int max_sweeps) {
-  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    R off = 0, fro = 0;
-#pragma unroll
-    for (int i = 0; i < D; ++i) {
-      fro += Am[tri_idx(i, i, D)] * Am[tri_idx(i, i, D)];
-#pragma unroll
-      for (int j = i + 1; j < D; ++j) off += R(2) * Am[tri_idx(i, j, D)] * Am[tri_idx(i, j, D)];
-    }
-    fro += off;
-    if (fro == R(0) || off <= tol2 * fro) break;
-    const R skip = R(1e-16) * sqrt(fro);
-#pragma unroll
-    for (int p = 0; p < D - 1; ++p)
-#pragma unroll
-      for (int q = p + 1; q < D; ++q) {
-        const R apq = Am[tri_idx(p, q, D)];
-        if (fabs(apq) <= skip) continue;
-        const R app = Am[tri_idx(p, p, D)], aqq = Am[tri_idx(q, q, D)];
-        const R tau = (aqq - app) / (R(2) * apq);
-        const R t = (tau >= R(0) ? R(1) : R(-1)) / (fabs(tau) + sqrt(R(1) + tau * tau));
-        const R c = R(1) / sqrt(R(1) + t * t), s = t * c;
-        Am[tri_idx(p, p, D)] = app - t * apq;
-        Am[tri_idx(q, q, D)] = aqq + t * apq;
-        Am[tri_idx(p, q, D)] = R(0);
-#pragma unroll
-        for (int k = 0; k < D; ++k) {
-          if (k == p || k == q) continue;
-          const int ikp = k < p ? tri_idx(k, p, D) : tri_idx(p, k, D);
-          const int ikq = k < q ? tri_idx(k, q, D) : tri_idx(q, k, D);
-          const R akp = Am[ikp], akq = Am[ikq];
-          Am[ikp] = c * akp - s * akq;
-          Am[ikq] = s * akp + c * akq;
-        }
-#pragma unroll
-        for (int k = 0; k < D; ++k) {
-          const R vkp = V[p * D + k], vkq = V[q * D + k];
-          V[p * D + k] = c * vkp - s * vkq;
-          V[q * D + k] = s * vkp + c * vkq;
-        }
-      }
-  }
-}
-
-template <int D>
-__device__ __forceinline__ void jacobi_refine64_reg(double (&Am)[D * (D + 1) / 2], double (&V)[D * D],
-                                                    const double tol2, const int max_sweeps) {
-  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    double off = 0, fro = 0;
-#pragma unroll
-    for (int i = 0; i < D; ++i) {
-      fro += Am[tri_idx(i, i, D)] * Am[tri_idx(i, i, D)];
-#pragma unroll
-      for (int j = i + 1; j < D; ++j) off += 2.0 * Am[tri_idx(i, j, D)] * Am[tri_idx(i, j, D)];
-    }
-    fro += off;
-    if (fro == 0.0 || off <= tol2 * fro) break;
-    const double nrm = sqrt(fro);
-    const double skip = 1e-16 * nrm;
-    const double inv = 1.0 / nrm;
-#pragma unroll
-    for (int p = 0; p < D - 1; ++p)
-#pragma unroll
-      for (int q = p + 1; q < D; ++q) {
-        const double apq = Am[tri_idx(p, q, D)];
-        if (fabs(apq) <= skip) continue;
-        const double app = Am[tri_idx(p, p, D)], aqq = Am[tri_idx(q, q, D)];
-        const float apq32 = (float)(apq * inv), dd32 = (float)((aqq - app) * inv);
-        const float tau = dd32 / (2.f * apq32);
-        const float t32 = (tau >= 0.f ? 1.f : -1.f) / (fabsf(tau) + sqrtf(1.f + tau * tau));
-        const double t = (double)t32;
-        const double c = rsqrt_refined(1.0 + t * t), s = t * c;
-        const double cc = c * c, ss = s * s, cs = c * s;
-        Am[tri_idx(p, p, D)] = cc * app - 2.0 * cs * apq + ss * aqq;
-        Am[tri_idx(q, q, D)] = ss * app + 2.0 * cs * apq + cc * aqq;
-        Am[tri_idx(p, q, D)] = cs * (app - aqq) + (cc - ss) * apq;
-#pragma unroll
-        for (int k = 0; k < D; ++k) {
-          if (k == p || k == q) continue;
-          const int ikp = k < p ? tri_idx(k, p, D) : tri_idx(p, k, D);
-          const int ikq = k < q ? tri_idx(k, q, D) : tri_idx(q, k, D);
-          const double akp = Am[ikp], akq = Am[ikq];
-          Am[ikp] = c * akp - s * akq;
-          Am[ikq] = s * akp + c * akq;
-        }
-#pragma unroll
-        for (int k = 0; k < D; ++k) {
-          const double vkp = V[p * D + k], vkq = V[q * D + k];
-          V[p * D + k] = c * vkp - s * vkq;
-          V[q * D + k] = s * vkp + c * vkq;
-        }
-      }
-  }
-}
-
-// PSD projection of a small symmetric D x D (packed upper triangle) in
-// registers: FP32 Jacobi, FP64 Gram-Schmidt, A = V^T B V, FP64 sweeps, then
-// B+ from the side with fewer eigenpairs (as k_hess_proj).
-template <int D>
-__device__ __forceinline__ void psd_small(const double (&B)[D * (D + 1) / 2], double (&P)[D * (D + 1) / 2]) {
-  constexpr int NP = D * (D + 1) / 2;
-  double mx = 0.0;
-#pragma unroll
-  for (int e = 0; e < NP; ++e) mx = fmax(mx, fabs(B[e]));
-  if (mx == 0.0) {
-#pragma unroll
-    for (int e = 0; e < NP; ++e) P[e] = 0.0;
-    return;
-  }
-  double V[D * D], Am[NP];
-  {
-    float A32[NP], V32[D * D];
-    const double inv = 1.0 / mx;
-#pragma unroll
-    for (int e = 0; e < NP; ++e) A32[e] = (float)(B[e] * inv);
-#pragma unroll
-    for (int e = 0; e < D * D; ++e) V32[e] = (e % (D + 1) == 0) ? 1.f : 0.f;
-    jacobi_reg<float, D>(A32, V32, PROJ_FP32_TOL2, 12);
-#pragma unroll
-    for (int k = 0; k < D; ++k) {
-#pragma unroll
-      for (int i = 0; i < D; ++i) V[k * D + i] = (double)V32[k * D + i];
-#pragma unroll
-      for (int j = 0; j < k; ++j) {
-        double dp = 0.0;
-#pragma unroll
-        for (int i = 0; i < D; ++i) dp += V[j * D + i] * V[k * D + i];
-#pragma unroll
-        for (int i = 0; i < D; ++i) V[k * D + i] -= dp * V[j * D + i];
-      }
-      double nn = 0.0;
-#pragma unroll
-      for (int i = 0; i < D; ++i) nn += V[k * D + i] * V[k * D + i];
-      nn = rsqrt_refined(nn);
-#pragma unroll
-      for (int i = 0; i < D; ++i) V[k * D + i] *= nn;
-    }
-  }
-#pragma unroll
-  for (int l = 0; l < D; ++l) {
-    double t[D];
-#pragma unroll
-    for (int i = 0; i < D; ++i) {
-      double v = 0.0;
-#pragma unroll
-      for (int j = 0; j < D; ++j) v += B[i <= j ? tri_idx(i, j, D) : tri_idx(j, i, D)] * V[l * D + j];
-      t[i] = v;
-    }
-#pragma unroll
-    for (int k = 0; k <= l; ++k) {
-      double v = 0.0;
-#pragma unroll
-      for (int i = 0; i < D; ++i) v += V[k * D + i] * t[i];
-      Am[tri_idx(k, l, D)] = v;
-    }
-  }
-  jacobi_refine64_reg<D>(Am, V, 1e-28, 12);
-  double lam[D];
-  int npos = 0, nneg = 0;
-#pragma unroll
-  for (int k = 0; k < D; ++k) {
-    lam[k] = Am[tri_idx(k, k, D)];
-    npos += lam[k] > 0.0;
-    nneg += lam[k] < 0.0;
-  }
-  const bool from_b = nneg < npos;
-#pragma unroll
-  for (int e = 0; e < NP; ++e) P[e] = from_b ? B[e] : 0.0;
-#pragma unroll
-  for (int k = 0; k < D; ++k) {
-    const double wk = from_b ? (lam[k] < 0.0 ? -lam[k] : 0.0) : (lam[k] > 0.0 ? lam[k] : 0.0);
-    if (wk == 0.0) continue;
-#pragma unroll
-    for (int i = 0; i < D; ++i) {
-      const double wi = wk * V[k * D + i];
-#pragma unroll
-      for (int j = i; j < D; ++j) P[tri_idx(i, j, D)] += wi * V[k * D + j];
-    }
-  }
-}
-
-// PSD projection of a symmetric 2x2 [[a, b], [b, c]] in closed form: with
-// h = (a - c)/2, r = hypot(h, b), m = (a + c)/2 the eigenvalues are m +- r;
-// if one is positive and one negative the result is l+ v v^T with
-// v v^T = [[h + r, b], [b, r - h]] / (2 r), each entry formed without
-// cancellation (h + r = b^2 / (r - h) when h < 0, and the mirror case), and
-// l+ = m + r or det / (m - r) whichever avoids cancellation.
-__device__ __forceinline__ void psd2(double a, double b, double c, double& pa, double& pb, double& pc) {
-  const double h = 0.5 * (a - c), m = 0.5 * (a + c);
-  const double r = hypot(h, b);
-  const double lp = m + r, lm = m - r;
-  if (lm >= 0.0) {
-    pa = a;
-    pb = b;
-    pc = c;
-    return;
-  }
-  if (lp <= 0.0) {
-    pa = pb = pc = 0.0;
-    return;
-  }
-  const double det = fma(a, c, -b * b);
-  const double lpos = m >= 0.0 ? lp : det / lm;
-  const double hp = h >= 0.0 ? h + r : (b * b) / (r - h);
-  const double hm = h >= 0.0 ? (b * b) / (r + h) : r - h;
-  const double sc = lpos / (2.0 * r);
-  pa = sc * hp;
-  pb = sc * b;
-  pc = sc * hm;
-}
-
-// Stage (d), part 2 for point-edge pairs queued in their own frame.  The
-// in-plane 4x4 block [[0, p r^T], [r p^T, Y]] (x of both reduced points, then
-// y) has the null vector (p_perp, 0) and equals Q T Q^T with
-// Q = [[p/|p|, 0], [0, I]] (orthonormal columns) and the 3x3
-// T = [[0, |p| r^T], [|p| r, Y]], so its projection is Q T+ Q^T: a 3x3
-// eigenproblem instead of a 4x4.  The 2x2 block is projected in closed form,
-// the 6x6 result rotated back block by block (B+ = (I x R) B'+ (I x R)^T) and
-// scattered as in k_hess_proj<6>.
-__device__ __forceinline__ void proj_pe_block(const HessArgs& A, int block) {
-  const int64_t w = (int64_t)block * 128 + threadIdx.x;
-  if (w >= (int64_t)*A.n4) return;
-  const uint32_t a = A.slot4[w];
-  double q[10], R[9];
-#pragma unroll
-  for (int e = 0; e < 10; ++e) q[e] = A.B4[(size_t)e * A.cap + w];
-#pragma unroll
-  for (int k = 0; k < 9; ++k) R[k] = A.B4[(size_t)(10 + k) * A.cap + w];
-  const double pn = sqrt(q[0] * q[0] + q[1] * q[1]);
-  double ph0 = 1.0, ph1 = 0.0;
-  if (pn > 0.0) {
-    const double ipn = 1.0 / pn;
-    ph0 = q[0] * ipn;
-    ph1 = q[1] * ipn;
-  }
-  const double T[6] = {0.0, pn * q[2], pn * q[3], q[4], q[5], q[6]};
-  double Tp[6], p2[3];
-  psd_small<3>(T, Tp);
-  psd2(q[7], q[8], q[9], p2[0], p2[1], p2[2]);
-  // Q T+ Q^T in the order (0x, 0y, 1x, 1y), packed
-  const double P4[10] = {ph0 * ph0 * Tp[0], ph0 * Tp[1], ph0 * ph1 * Tp[0], ph0 * Tp[2], Tp[3],
-                         ph1 * Tp[1],       Tp[4],       ph1 * ph1 * Tp[0], ph1 * Tp[2], Tp[5]};
-  // Back to the three points and to world axes.  Local block (ab, bb) of the
-  // reduced matrix: L_ab,bb = [[in-plane 2x2 from P4, 0], [0, e3-e3 entry from
-  // p2]]; block (q1, q2) of the points is R L'(q1, q2) R^T with
-  // L'(q1, q2) = sum K3[q1][ab] K3[q2][bb] L_ab,bb.  K3's rows are (c, s),
-  // (-c, s), (0, -2s), c = 1/sqrt2, s = 1/sqrt6, so with X = L00/2,
-  // Y = L11/6, W = L11/3, S = cs (L01 + L10), Dm = cs (L01 - L10),
-  // Z = 2cs L01 (cs = 1/sqrt12):
-  //   L'00 = X + S + Y, L'11 = X - S + Y, L'22 = 2W,
-  //   L'01 = -X + Dm + Y, L'02 = -Z - W, L'12 = Z - W.
-  constexpr double cs = 0.28867513459481288225;  // 1/sqrt(12)
-  const double L00[2][2] = {{P4[0], P4[1]}, {P4[1], P4[4]}}, L01[2][2] = {{P4[2], P4[3]}, {P4[5], P4[6]}},
-               L11[2][2] = {{P4[7], P4[8]}, {P4[8], P4[9]}};
-  double Lq[6][2][2], zq[6];  // 00, 11, 22, 01, 02, 12
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const double X = 0.5 * L00[i][j], Y = L11[i][j] * (1.0 / 6.0), W = L11[i][j] * (1.0 / 3.0);
-      const double S = cs * (L01[i][j] + L01[j][i]), Dm = cs * (L01[i][j] - L01[j][i]), Z = 2.0 * cs * L01[i][j];
-      Lq[0][i][j] = X + S + Y;
-      Lq[1][i][j] = X - S + Y;
-      Lq[2][i][j] = 2.0 * W;
-      Lq[3][i][j] = -X + Dm + Y;
-      Lq[4][i][j] = -Z - W;
-      Lq[5][i][j] = Z - W;
-    }
-  {
-    const double X = 0.5 * p2[0], Y = p2[2] * (1.0 / 6.0), W = p2[2] * (1.0 / 3.0), S = 2.0 * cs * p2[1],
-                 Z = 2.0 * cs * p2[1];
-    zq[0] = X + S + Y;
-    zq[1] = X - S + Y;
-    zq[2] = 2.0 * W;
-    zq[3] = -X + Y;
-    zq[4] = -Z - W;
-    zq[5] = Z - W;
-  }
-  // world block: E2 A2 E2^T + z e3 e3^T, E2 = (e1, e2) = columns 0, 1 of R
-  auto world = [&](const double (&A2)[2][2], double z, double (&w)[9]) {
-    double T[3][2];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int bb = 0; bb < 2; ++bb) T[i][bb] = R[3 * i] * A2[0][bb] + R[3 * i + 1] * A2[1][bb];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      const double ze = z * R[3 * i + 2];
-#pragma unroll
-      for (int j = 0; j < 3; ++j) w[3 * i + j] = T[i][0] * R[3 * j] + T[i][1] * R[3 * j + 1] + ze * R[3 * j + 2];
-    }
-  };
-  // scatter: the three points the point-edge type involves, in stencil order
-  const uint32_t c = A.aidx[a];
-  const Stencil st = stencil_of(A.cand[c], A.ev0, A.ev1, A.tv, A.T);
-  const TypeInfo& TI = st.ee ? c_ee_types[A.ctype[c]] : c_pt_types[A.ctype[c]];
-  int pts[4], np = 0;
-  for (int i = 0; i < 4; ++i) {
-    bool used = false;
-    for (int mm = 0; mm < 2; ++mm) used |= TI.C[mm][i] != 0;
-    if (used) pts[np++] = i;
-  }
-  const int qa[6] = {0, 1, 2, 0, 0, 1}, qb[6] = {0, 1, 2, 1, 2, 2};
-#pragma unroll
-  for (int k = 0; k < 6; ++k) {
-    double blk[9];
-    world(Lq[k], zq[k], blk);
-    const int r = st.v[pts[qa[k]]], cc = st.v[pts[qb[k]]];
-    add_block(A, r, cc, blk, false);
-    if (k >= 3) add_block(A, cc, r, blk, true);
-  }
-}
-
-// the point-edge pairs projected in their own frame, one thread per pair
-__global__ void __launch_bounds__(128) k_hess_proj_pe(HessArgs A) { proj_pe_block(A, blockIdx.x); }
-
-// Short queues (a small scene): the warp-per-pair 9x9 projection in blocks
-// [0, nb9) and the point-edge pairs in the blocks after them, one launch, so
-// that the two independent queues run side by side (both only add into the
-// BSR values, atomically) instead of one after the other.
-__global__ void __launch_bounds__(PL_THREADS) k_hess_proj_short(HessArgs A, int nb9) {
-  static_assert(PL_THREADS == 128, "both halves run 128-thread blocks");
-  if ((int)blockIdx.x < nb9) proj_lanes_block(A, blockIdx.x);
-  else proj_pe_block(A, blockIdx.x - nb9);
 }
 
 __global__ void k_energy_final(int count, const unsigned long long* __restrict__ macc, double* __restrict__ out) {
@@ -2857,16 +2181,8 @@ cb_status barrier_run(cb_scene* s, const double* x, double* energy, double* grad
     A.val = bp<double>(s->bsr_val);
     A.grad = grad;
     A.status = status;
-    CB_TRY(buf_ensure(s->hB9, sizeof(double) * 45 * (size_t)na, st));
-    CB_TRY(buf_ensure(s->hB6, sizeof(double) * 21 * (size_t)na, st));
-    CB_TRY(buf_ensure(s->hB4, sizeof(double) * 19 * (size_t)na, st));
-    CB_TRY(buf_ensure(s->hslot, sizeof(uint32_t) * 3 * (size_t)na, st));
+    if (mollify) CB_TRY(buf_ensure(s->hB9, sizeof(double) * 45 * (size_t)na, st));
     A.B9 = bp<double>(s->hB9);
-    A.B6 = bp<double>(s->hB6);
-    A.B4 = bp<double>(s->hB4);
-    A.slot9 = bp<uint32_t>(s->hslot);
-    A.slot6 = bp<uint32_t>(s->hslot) + na;
-    A.slot4 = bp<uint32_t>(s->hslot) + 2 * na;
     A.n9 = (unsigned int*)(sc + SC_N9);
     A.n6 = (unsigned int*)(sc + SC_N6);
     A.n4 = (unsigned int*)(sc + SC_N4);
@@ -2876,22 +2192,19 @@ cb_status barrier_run(cb_scene* s, const double* x, double* energy, double* grad
     A.nmoll = (const unsigned*)(sc + SC_NMOLL);
     A.elen2 = bp<double>(s->elen2);
     if (s->timing) cudaEventRecord(s->ev[10], st);
-    k_hess_prep<<<cb_grid(na, 128), 128, 0, cb_count(st)>>>(A);
-    if (mollify) k_moll_hess<<<cb_grid(na, 128), 128, 0, cb_count(st)>>>(A);
+    k_pair_hess<<<cb_grid(na, PAIR_T), PAIR_T, 0, cb_count(st)>>>(A);
     CB_CUDA(cudaGetLastError());
-    // the three queues' lengths stay on the device: every projection kernel
-    // reads its own, the point-edge one over a grid for all active pairs, the
-    // shared-memory ones over at most one wave of blocks (grid-stride)
-    if (na <= PL_MAX_ACTIVE) {
-      const int smem = PL_SMEM * (int)sizeof(double) * PL_PAIRS;
-      const int nb9 = (int)((na + PL_PAIRS - 1) / PL_PAIRS);
-      k_hess_proj_short<<<nb9 + (int)cb_grid(na, 128), PL_THREADS, smem, cb_count(st)>>>(A, nb9);
+    if (mollify) {
+      // the queue's length stays on the device; a warp per pair while the queue is short
+      k_moll_hess<<<cb_grid(na, 128), 128, 0, cb_count(st)>>>(A);
+      if (na <= PL_MAX_ACTIVE) {
+        const int smem = PL_SMEM * (int)sizeof(double) * PL_PAIRS;
+        k_hess_proj_lanes<<<(int)((na + PL_PAIRS - 1) / PL_PAIRS), PL_THREADS, smem, cb_count(st)>>>(A);
+      } else {
+        CB_TRY(launch_proj(s, A, na, st));
+      }
       CB_CUDA(cudaGetLastError());
-    } else {
-      k_hess_proj_pe<<<cb_grid(na, 128), 128, 0, cb_count(st)>>>(A);
-      CB_TRY(launch_proj<9>(s, A, na, st));
     }
-    CB_TRY(launch_proj<6>(s, A, na, st));
     if (s->timing) cudaEventRecord(s->ev[11], st);
     CB_CUDA(cudaGetLastError());
   }

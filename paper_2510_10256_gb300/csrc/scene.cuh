@@ -142,7 +142,7 @@ struct cb_scene {
   cudaStream_t last_stream = nullptr;
   int device = 0;
   int n_sms = 152;      // multiprocessors of the device (caps of grid-stride launches: a few blocks per SM)
-  int proj_occ[2] = {0, 0};  // resident blocks per SM of k_hess_proj<9> and <6> (0: not looked up yet)
+  int proj_occ = 0;     // resident blocks per SM of k_hess_proj (0: not looked up yet)
 
   // topology on device
   DevBuf ev0, ev1;      // int32 [E]
@@ -201,8 +201,7 @@ struct cb_scene {
   DevBuf horder;        // uint32 active pair indices in prep order (face / line-line pairs first)
   DevBuf hmoll;         // uint8 [na] mollified edge-edge pair (CB_EE_MOLLIFIER), handled by k_moll_hess
   DevBuf mlist;         // uint32 active indices of the mollified pairs
-  DevBuf hB9, hB6, hB4;  // queued reduced Hessians (packed, element-major); hB4: point-edge in its own frame
-  DevBuf hslot;          // uint32 [2][na] active index of each queued matrix
+  DevBuf hB9;           // CB_EE_MOLLIFIER: queued reduced Hessians (packed, element-major)
   DevBuf xf, pf;         // float [3][n]: centred FP32 copies of x and of p
   DevBuf dlist;          // uint32: candidates / CCD pairs queued for the FP64 phase
   DevBuf ccd_keys;      // uint64 [nccd]
@@ -252,7 +251,7 @@ enum {
   SC_N9 = 9,
   SC_N6 = 10,
   SC_NLIST = 11,        // two uint32 counters: point-triangle and edge-edge pairs for the exact distance
-  SC_N4 = 14,           // point-edge pairs queued in their own frame
+  SC_N4 = 14,           // point-edge pairs (but for SC_N6's)
   SC_NU = 15,           // CCD pairs left unresolved by the first step
   SC_FP32_PAIRS = 12,   // broad phase of contact_build: pairs passing the FP32 box test
   SC_FP64_DECIDED = 13, // ... of which the FP64 boxes decided

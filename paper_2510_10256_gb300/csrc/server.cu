@@ -187,10 +187,9 @@ cb_status cb_scene_reserve(cb_scene* s, int64_t n_candidates, int64_t n_ccd, int
   CB_TRY(buf_ensure(s->bflag, sizeof(uint32_t) * 16 * na, st));
   CB_TRY(buf_ensure(s->bpos, sizeof(uint32_t) * (16 * na + 1), st));
   CB_TRY(buf_ensure(s->horder, sizeof(uint32_t) * na, st));
-  CB_TRY(buf_ensure(s->hB9, sizeof(double) * 45 * na, st));
-  CB_TRY(buf_ensure(s->hB6, sizeof(double) * 21 * na, st));
-  CB_TRY(buf_ensure(s->hB4, sizeof(double) * 19 * na, st));
-  CB_TRY(buf_ensure(s->hslot, sizeof(uint32_t) * 3 * na, st));
+  bool mollify = false;
+  for (const MemberParams& m : s->hmp) mollify |= m.mollify != 0;
+  if (mollify) CB_TRY(buf_ensure(s->hB9, sizeof(double) * 45 * na, st));
   // CCD candidates (stage e)
   CB_TRY(buf_ensure(s->ccd_keys, sizeof(uint64_t) * nq, st));
   CB_TRY(buf_ensure(s->ccd_t, sizeof(double) * nq, st));
