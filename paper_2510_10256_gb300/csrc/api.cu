@@ -88,7 +88,7 @@ static void scene_release(cb_scene* s) {
                     &s->rloop, &s->rlast, &s->elen2, &s->hmoll, &s->mlist, &s->ruv, &s->frest,
                     &s->frest_dbar, &s->frest_j, &s->frow_pt, &s->frow_ee, &s->dbar_comp, &s->cand, &s->klass, &s->cand_alt, &s->klass_alt, &s->cd, &s->cflag, &s->cpos, &s->ctype, &s->ccls, &s->aidx,
                     &s->bkey[0], &s->bkey[1], &s->bflag, &s->bpos, &s->bsr_row, &s->bsr_col, &s->bsr_val,
-                    &s->row_cnt, &s->hB9, &s->horder, &s->xf, &s->pf, &s->dlist, &s->mp, &s->vsc, &s->macc, &s->ccd_keys, &s->ccd_t, &s->ccd_cls, &s->ccd_lb, &s->ccd_flag, &s->ccd_pos, &s->ccd_list, &s->ccd_ulist, &s->scan_tmp, &s->hist,
+                    &s->row_cnt, &s->hB9, &s->horder, &s->xf, &s->pf, &s->dlist, &s->mp, &s->vsc, &s->macc, &s->ccd_keys, &s->ccd_t, &s->ccd_cls, &s->ccd_list, &s->ccd_ulist, &s->scan_tmp, &s->hist,
                     &s->fr_key, &s->fr_st, &s->fr_dat, &s->fr_hw, &s->dev_scalars};
   for (DevBuf* b : bufs) buf_free(*b, st);
   for (BroadWork* w : {&s->bw, &s->bwc}) {
@@ -859,14 +859,15 @@ cb_status cb_get_ccd(cb_scene* s, uint64_t* keys, double* t, uint8_t* klass, int
     std::vector<uint8_t> cc;
     CB_TRY(dl(k, s->ccd_keys, s->n_ccd, st));
     if (t) CB_TRY(dl(tt, s->ccd_t, s->n_ccd, st));
-    if (klass) CB_TRY(dl(cc, s->ccd_cls, s->n_ccd, st));
+    CB_TRY(dl(cc, s->ccd_cls, s->n_ccd, st));
     CB_CUDA(cudaStreamSynchronize(st));
     std::vector<uint32_t> order;
     sort_keys(k, &order);
     for (size_t q = 0; q < k.size(); ++q) {
       if (keys) keys[q] = k[q];
-      if (t) t[q] = tt[order[q]];
-      if (klass) klass[q] = cc[order[q]];
+      const uint8_t c = cc[order[q]];
+      if (t) t[q] = (c & CB_CCD_ONE) ? 1.0 : tt[order[q]];
+      if (klass) klass[q] = (uint8_t)(c & ~CB_CCD_ONE);
     }
   }
   return CB_OK;

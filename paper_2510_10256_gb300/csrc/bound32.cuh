@@ -93,8 +93,12 @@ __device__ __forceinline__ void closest_on_segments(f3 p0, f3 p1, f3 q0, f3 q1, 
 
 // Lower bound of the distance of a stencil whose vertices are x_i = c + P_i,
 // given FP32 copies Pf_i of (x_i - c); X = max |x - c| over the scene.
-// Returns 0 when no useful bound exists.
-__device__ __forceinline__ float lower_bound(bool ee, f3 W0, f3 W1, f3 W2, f3 W3, float X) {
+// Returns 0 when no useful bound exists.  With UB also an upper bound: the
+// distance between the two approximate closest points, which lie on the
+// primitives to within the rounding of their convex combinations (at most 12 u R
+// a point, beside the errors above).
+template <bool UB>
+__device__ __forceinline__ float stencil_bounds(bool ee, f3 W0, f3 W1, f3 W2, f3 W3, float X, float& ub) {
   const f3 P0 = f3{0.f, 0.f, 0.f}, P1 = fsub3(W1, W0), P2 = fsub3(W2, W0), P3 = fsub3(W3, W0);
   const float R = fmaxf(fmaxabs3(P1), fmaxf(fmaxabs3(P2), fmaxabs3(P3)));
   f3 a;
@@ -112,13 +116,21 @@ __device__ __forceinline__ float lower_bound(bool ee, f3 W0, f3 W1, f3 W2, f3 W3
     smax = fmaxf(fdot3(a, P2), fdot3(a, P3));
   }
   const float an = sqrtf(fdot3(a, a));
-  if (!(an > 0.f)) return 0.f;
   const float u = 5.9604645e-8f;  // 2^-24
+  if (UB) ub = an * (1.f + 16.f * u) + 4.f * (16.f * u * R + 3.5f * u * (X + R));
+  if (!(an > 0.f)) return 0.f;
   const float a1 = fabsf(a.x) + fabsf(a.y) + fabsf(a.z);
   const float s = (smin - smax) - 4.f * (6.f * u * a1 * R);
   if (!(s > 0.f)) return 0.f;
   const float lb = s / (an * (1.f + 16.f * u)) - 4.f * (3.5f * u * (X + R));
   return lb > 0.f ? lb : 0.f;
+}
+__device__ __forceinline__ float lower_bound(bool ee, f3 W0, f3 W1, f3 W2, f3 W3, float X) {
+  float ub;
+  return stencil_bounds<false>(ee, W0, W1, W2, W3, X, ub);
+}
+__device__ __forceinline__ float distance_bounds(bool ee, f3 W0, f3 W1, f3 W2, f3 W3, float X, float& ub) {
+  return stencil_bounds<true>(ee, W0, W1, W2, W3, X, ub);
 }
 
 }  // namespace cbb

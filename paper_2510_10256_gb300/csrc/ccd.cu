@@ -11,24 +11,22 @@
 // below s g0.  alpha = min(1, min_p t_p).
 //
 // Only the minimum is needed, so the step bound is computed exactly without
-// iterating every pair to its end: the additive CCD iterate t only grows, and
-// t_p >= min(1, (1-s) g0 / l_p) =: lb_p.  Pass 1 computes lb_p for every pair
-// (one distance each; pairs whose first step already passes t = 1, or that do
-// not move, are resolved exactly here).  Pass 2 works in rounds with a ceiling
-// h per member, starting at 4 L (L the smallest lb_p) and growing 4x: each
-// round iterates the pairs with lb_p <= h, stopping a pair when it finishes
-// (exact t_p) or when its iterate reaches h or the member's current minimum;
-// a stopped pair keeps its iterate as its new lb_p.  After a round every
-// unfinished pair has t_p >= lb_p >= min(h, m) with m the smallest exact t_p
-// found, so once m <= h (or h = 1) alpha = min(1, m) exactly.  A pair's
-// iteration always restarts from t = 0, so an exact t_p is the same number
-// as a single uninterrupted run.
+// iterating every pair in FP64.  The additive-CCD iterate t only grows, and
+// t_p >= min(1, (1-s) g0 / l_p).  Pass 1 bounds that first step per pair (FP32
+// bounds; one FP64 distance where they cannot decide) and lists the pairs it
+// leaves below 1.  Pass 2 brackets each listed pair's t_p in FP32
+// (accd32.cuh), keeping the smallest upper bound per member, and lists the
+// pairs whose lower bound is not above it.  Pass 3 runs the FP64 iteration on
+// those, dropping a pair once its iterate is above that bound or reaches the
+// smallest exact t_p found: every pair dropped has t_p no smaller, so alpha is
+// the minimum over all pairs of the full iteration's t_p, bit for bit.  Every
+// list length stays on the device: no host wait after the broad phase.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
 
-#include "bound32.cuh"
+#include "accd32.cuh"
 #include "geometry.cuh"
 #include "frest.cuh"
 #include "prims.cuh"
@@ -39,7 +37,7 @@ namespace {
 constexpr double ACCD_S = 0.1;
 constexpr double ACCD_C = 0.9;
 constexpr int ACCD_MAX_ITER = 10000;
-constexpr uint8_t EXACT = 0x80;   // class byte flag: t_p is exact (else a lower bound)
+constexpr uint8_t EXACT = CB_CCD_EXACT, ONE = CB_CCD_ONE;  // class byte flags (scene.cuh)
 
 struct CcdArgs {
   int64_t np;
@@ -63,13 +61,18 @@ struct CcdArgs {
   const double* __restrict__ p;
   double* __restrict__ t_out;
   uint8_t* __restrict__ cls_out;
-  unsigned long long* __restrict__ macc;     // per member: alpha bits, lb bits, status, band lo/hi
+  unsigned long long* __restrict__ macc;     // per member: alpha bits, status, smallest upper bound
+  int members;
   unsigned long long* __restrict__ status;
   unsigned long long* __restrict__ max_iters;
   const float4* __restrict__ xf;  // FP32 (x - member centre), one float4 per vertex
   const float4* __restrict__ pf;  // FP32 p, one float4 per vertex
-  uint32_t* __restrict__ ulist;   // pairs left unresolved by the first step (lb < 1)
+  uint32_t* __restrict__ ulist;   // pairs left unresolved by the first step (t_out, a lower bound, below 1)
   unsigned int* __restrict__ nu;
+  // pairs left for the FP64 iteration: point-triangle from the front (nlist[0] of them), edge-edge from the back
+  // (nlist[1]) of np entries: the distance routine branches on the kind, and a warp that mixes them runs both
+  uint32_t* __restrict__ list;
+  unsigned int* __restrict__ nlist;
 };
 
 __device__ __forceinline__ unsigned long long* macc_of(const CcdArgs& A, int m, int slot) {
@@ -154,21 +157,25 @@ __device__ __forceinline__ cbb::f3 ldf(const float4* __restrict__ a, int n, int 
   return cbb::f3{q.x, q.y, q.z};
 }
 
-// Minimum of non-negative doubles per member (compared as bit patterns): one
-// atomicMin per warp when the warp holds one member, per lane otherwise;
-// 2.0 marks "no value".
-__device__ __forceinline__ void member_min_atomic(const CcdArgs& A, double v, int mem, int slot) {
-  unsigned long long b = (unsigned long long)__double_as_longlong(v);
-  const int m0 = __shfl_sync(0xffffffffu, mem, 0);
-  if (__all_sync(0xffffffffu, mem == m0 || mem < 0)) {
+// FP32 motion of a stencil in its local frame: positions relative to the
+// first vertex, displacements relative to their mean, subtracted in FP64
+__device__ __forceinline__ void pair_motion32(const double* __restrict__ x, const double* __restrict__ p, int n,
+                                              const int (&v)[4], cbb::Motion32& M) {
+  const d3 X0 = ld(x, n, v[0]);
+  d3 P[4];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long u = __shfl_xor_sync(0xffffffffu, b, o);
-      b = u < b ? u : b;
-    }
-    if ((threadIdx.x & 31) == 0 && m0 >= 0 && b < 0x4000000000000000ull) atomicMin(macc_of(A, m0, slot), b);
-  } else if (mem >= 0 && b < 0x4000000000000000ull) {
-    atomicMin(macc_of(A, mem, slot), b);
+  for (int k = 0; k < 4; ++k) {
+    const d3 Y = sub3(ld(x, n, v[k]), X0);
+    M.Y[k] = cbb::f3{(float)Y.x, (float)Y.y, (float)Y.z};
+    P[k] = ld(p, n, v[k]);
+  }
+  const d3 pb = mk3(xmul(xadd(xadd(xadd(P[0].x, P[1].x), P[2].x), P[3].x), 0.25),
+                    xmul(xadd(xadd(xadd(P[0].y, P[1].y), P[2].y), P[3].y), 0.25),
+                    xmul(xadd(xadd(xadd(P[0].z, P[1].z), P[2].z), P[3].z), 0.25));
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const d3 Q = sub3(P[k], pb);
+    M.Q[k] = cbb::f3{(float)Q.x, (float)Q.y, (float)Q.z};
   }
 }
 
@@ -183,6 +190,18 @@ __device__ __forceinline__ void warp_append(bool flag, uint32_t value, uint32_t*
   base = __shfl_sync(0xffffffffu, base, leader);
   if (flag) list[base + __popc(m & ((1u << lane) - 1u))] = value;
 }
+// ... from the end of a list of cap entries backwards
+__device__ __forceinline__ void warp_append_back(bool flag, uint32_t value, uint32_t* __restrict__ list, int64_t cap,
+                                                 unsigned int* __restrict__ count) {
+  const unsigned m = __ballot_sync(0xffffffffu, flag);
+  if (!m) return;
+  const unsigned lane = threadIdx.x & 31;
+  const int leader = __ffs(m) - 1;
+  unsigned base = 0;
+  if ((int)lane == leader) base = atomicAdd(count, (unsigned)__popc(m));
+  base = __shfl_sync(0xffffffffu, base, leader);
+  if (flag) list[cap - 1 - (int64_t)(base + __popc(m & ((1u << lane) - 1u)))] = value;
+}
 
 // pass 1a: an FP32 lower bound of the distance and an FP32 upper bound of
 // l_p give a lower bound of the first step.  A pair whose class is certain and
@@ -193,12 +212,10 @@ __device__ __forceinline__ void warp_append(bool flag, uint32_t value, uint32_t*
 // 1 - 2^-23, so it stays below the first step as FP64 evaluates it; the
 // thresholds are the members' FP32 copies rounded up.  (FP64 would put ~25
 // operations per candidate on the FP64 pipe, which issues 1/64 as fast.)
-__global__ void __launch_bounds__(128) k_ccd_screen(CcdArgs A, double* __restrict__ lb_out,
-                                                    uint32_t* __restrict__ list, unsigned int* __restrict__ nlist) {
+__global__ void __launch_bounds__(128) k_ccd_screen(CcdArgs A, uint32_t* __restrict__ list,
+                                                    unsigned int* __restrict__ nlist) {
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   bool need = false, unres = false;
-  double m_exact = 2.0, m_lb = 2.0;  // this lane's contributions to the two minima
-  int mem = -1;
   if (q < A.np) {
     const uint64_t key = A.keys[q];
     const uint32_t ty = cb_key_type(key), ki = cb_key_i(key), kj = cb_key_j(key);
@@ -217,7 +234,7 @@ __global__ void __launch_bounds__(128) k_ccd_screen(CcdArgs A, double* __restric
       v[3] = A.ev1[kj];
       ee = true;
     }
-    mem = A.vsc[v[0]];
+    const int mem = A.vsc[v[0]];
     const MemberParams& M = A.mp[mem];
     const bool filt = is_filtered(A, M, key, ki, kj);
     need = true;
@@ -226,9 +243,7 @@ __global__ void __launch_bounds__(128) k_ccd_screen(CcdArgs A, double* __restric
     const bool culled = M.cull_radius > 0 && A.comp[A.ev0[ki]] == A.comp[A.ev0[kj]] &&
                         rod_gap(A.rloop, ki, kj) <= M.cull_radius;
     if (culled) {
-      A.t_out[q] = 1.0;
-      A.cls_out[q] = (uint8_t)3 | EXACT;
-      m_exact = 1.0;
+      A.cls_out[q] = (uint8_t)3 | EXACT | ONE;
       need = false;
     } else {
       const double Xd = A.cx[4 * mem + 3];
@@ -253,104 +268,109 @@ __global__ void __launch_bounds__(128) k_ccd_screen(CcdArgs A, double* __restric
         if (lp32 > 1e-30f && g_lb > 0.f) {
           // (1 - s) g / l_p; 0.9f rounds below 0.9 = 1 - s
           const float tl_lb = __fmul_rd(__fdiv_rd(__fmul_rd(0.9f, g_lb), lp_ub), 0.99999988f);
-          const bool exact = tl_lb > 1.f;
-          const double t = exact ? 1.0 : (double)tl_lb;
-          A.t_out[q] = t;
-          if (!exact) lb_out[q] = t;
-          A.cls_out[q] = (uint8_t)cls | (exact ? EXACT : 0);
-          if (exact) m_exact = t;
-          else m_lb = t;
-          unres = !exact;
+          unres = !(tl_lb > 1.f);
+          if (unres) A.t_out[q] = (double)tl_lb;
+          A.cls_out[q] = (uint8_t)cls | (unres ? 0 : EXACT | ONE);
           need = false;
         }
       }
     }
   }
-  member_min_atomic(A, m_exact, mem, MACC_ALPHA);
-  member_min_atomic(A, m_lb, mem, MACC_LB);
   warp_append(need, (uint32_t)q, list, nlist);
   warp_append(unres, (uint32_t)q, A.ulist, A.nu);
 }
 
 // pass 1b: exact FP64 first step of the queued pairs
-__global__ void __launch_bounds__(128) k_ccd_bound(CcdArgs A, double* __restrict__ lb_out,
-                                                   const uint32_t* __restrict__ list,
+__global__ void __launch_bounds__(128) k_ccd_bound(CcdArgs A, const uint32_t* __restrict__ list,
                                                    const unsigned int* __restrict__ nlist) {
   const unsigned m = *nlist;
-  // uniform trip count per block so that every lane reaches the warp minima
+  // uniform trip count per block so that every lane reaches the append
   for (unsigned w0 = blockIdx.x * blockDim.x; w0 < m; w0 += gridDim.x * blockDim.x) {
     const unsigned w = w0 + threadIdx.x;
-    double m_exact = 2.0, m_lb = 2.0;
-    int mem = -1;
     bool unres = false;
     uint32_t qq = 0;
     if (w < m) {
       const int64_t q = list[w];
       const AccdStart S = accd_start(A, q);
-      mem = S.mem;
-      double t;
-      bool exact = true;
-      if (S.lp == 0.0) {
-        t = 1.0;
-      } else if (S.g0 <= 0.0) {
-        t = 0.0;
+      const double tl = S.lp == 0.0 ? 2.0 : xdiv(xmul(xsub(1.0, ACCD_S), S.g0), S.lp);
+      uint8_t flags = EXACT | ONE;  // no motion, or the first step already passes t_c = 1
+      if (S.lp != 0.0 && S.g0 <= 0.0) {
+        flags = EXACT;
+        A.t_out[q] = 0.0;
         atomicOr(A.status, (unsigned long long)CB_DEV_PENETRATION);
-        atomicOr(macc_of(A, mem, MACC_STATUS), (unsigned long long)CB_DEV_PENETRATION);
-      } else {
-        const double tl = xdiv(xmul(xsub(1.0, ACCD_S), S.g0), S.lp);
-        if (tl > 1.0) {
-          t = 1.0;  // the first step already passes t_c = 1: no contact within the step
-        } else {
-          t = tl;
-          exact = false;
-        }
+        atomicOr(macc_of(A, S.mem, MACC_STATUS), (unsigned long long)CB_DEV_PENETRATION);
+        atomicMin(macc_of(A, S.mem, MACC_ALPHA), 0ull);
+      } else if (!(tl > 1.0)) {
+        flags = 0;
+        A.t_out[q] = tl;
+        unres = true;
       }
-      A.t_out[q] = t;
-      if (!exact) lb_out[q] = t;
-      A.cls_out[q] = (uint8_t)S.cls | (exact ? EXACT : 0);
-      if (exact) m_exact = t;
-      else m_lb = t;
-      unres = !exact;
+      A.cls_out[q] = (uint8_t)S.cls | flags;
       qq = (uint32_t)q;
     }
-    member_min_atomic(A, m_exact, mem, MACC_ALPHA);
-    member_min_atomic(A, m_lb, mem, MACC_LB);
     warp_append(unres, qq, A.ulist, A.nu);
   }
 }
 
-// select the listed pairs with lb <= hi of their member: flag[w] for pair
-// ulist[w], counted by kind (point-triangle in the low 32 bits, edge-edge in
-// the high ones) so that the list puts each kind together: the distance
-// routine branches on the kind, and a warp that mixes them runs both
-__global__ void k_ccd_select_u(int64_t nu, const uint32_t* __restrict__ ulist, const uint64_t* __restrict__ keys,
-                               const int32_t* __restrict__ ev0, const int32_t* __restrict__ vsc,
-                               const double* __restrict__ lb, const unsigned long long* __restrict__ macc,
-                               unsigned long long* __restrict__ flag) {
-  const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (w >= nu) return;
-  const uint32_t q = ulist[w];
-  const uint64_t key = keys[q];
-  const bool pt = cb_key_type(key) == CB_KEY_PT;
-  const int v0 = pt ? (int)cb_key_i(key) : ev0[cb_key_i(key)];
-  const int mem = vsc[v0];
-  const double hi = __longlong_as_double(macc[(size_t)mem * MACC_STRIDE + MACC_HI]);
-  flag[w] = lb[q] <= hi ? (pt ? 1ull : 1ull << 32) : 0ull;
+// an upper bound of the member's smallest t_p: FP32 brackets and exact values so far (rounded up)
+__device__ __forceinline__ float member_cap(const CcdArgs& A, int mem) {
+  const double a = __longlong_as_double(*(volatile unsigned long long*)macc_of(A, mem, MACC_ALPHA));
+  const double h = __longlong_as_double(*(volatile unsigned long long*)macc_of(A, mem, MACC_HI));
+  return __double2float_ru(fmin(a, h));
 }
 
-// the selected pairs, point-triangle ones first (npt of them, the low half of
-// the scan's total), each kind in list order
-__global__ void k_list_u(int64_t nu, const uint32_t* __restrict__ ulist, const unsigned long long* __restrict__ flag,
-                         const unsigned long long* __restrict__ pos, const unsigned long long* __restrict__ total,
-                         uint32_t* __restrict__ list) {
-  const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (w >= nu || !flag[w]) return;
-  const unsigned long long p = pos[w];
-  const uint64_t at = (flag[w] & 0xffffffffull) ? (p & 0xffffffffull) : (*total & 0xffffffffull) + (p >> 32);
-  if (at < (uint64_t)nu) list[at] = ulist[w];  // always: at most nu pairs are selected
+// pass 2: FP32 brackets of the unresolved pairs (grid-stride; the trip count
+// is uniform over a warp so that every lane reaches the appends)
+__global__ void __launch_bounds__(128) k_ccd_refine(CcdArgs A) {
+  const int64_t nu = min((int64_t)*A.nu, A.np);
+  for (int64_t w0 = (int64_t)blockIdx.x * blockDim.x; w0 < nu; w0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t w = w0 + threadIdx.x;
+    bool keep = false, ee = false;
+    uint32_t q = 0;
+    if (w < nu) {
+      q = A.ulist[w];
+      const uint64_t key = A.keys[q];
+      const uint32_t ki = cb_key_i(key), kj = cb_key_j(key);
+      ee = cb_key_type(key) != CB_KEY_PT;
+      const int v0 = ee ? A.ev0[ki] : (int)ki;
+      const int mem = A.members > 1 ? A.vsc[v0] : 0;
+      const double lb = A.t_out[q];
+      if (__double2float_rd(lb) <= member_cap(A, mem)) {
+        int v[4] = {v0, 0, 0, 0};
+        if (ee) {
+          v[1] = A.ev1[ki];
+          v[2] = A.ev0[kj];
+          v[3] = A.ev1[kj];
+        } else {
+#pragma unroll
+          for (int k = 0; k < 3; ++k) v[1 + k] = A.tv[(size_t)k * A.T + kj];
+        }
+        cbb::Motion32 M;
+        M.ee = ee;
+        const uint8_t cls = A.cls_out[q];
+        const MemberParams& MP = A.mp[mem];
+        const double off = (cls == 0 && !MP.single) ? MP.xi : 0.0;
+        M.off_dn = __double2float_rd(off);
+        M.off_up = __double2float_ru(off);
+        pair_motion32(A.x, A.p, A.n, v, M);
+        float lo = 0.f, hi = 1.f;
+        const int r = cbb::motion_slopes(M) ? cbb::accd_bounds32(M, [&] { return member_cap(A, mem); }, lo, hi) : -1;
+        if (r == 1) {
+          A.cls_out[q] = cls | EXACT | ONE;
+        } else {
+          if (r == 0 && (double)lo > lb) A.t_out[q] = (double)lo;
+          if (r == 0 && hi < 1.f) atomicMin(macc_of(A, mem, MACC_HI), (unsigned long long)__double_as_longlong((double)hi));
+          keep = r < 0 || lo <= member_cap(A, mem);
+        }
+      }
+    }
+    warp_append(keep && !ee, q, A.list, &A.nlist[0]);
+    warp_append_back(keep && ee, q, A.list, A.np, &A.nlist[1]);
+  }
 }
 
-// pass 2: additive CCD of the selected pairs, each up to its member's ceiling.
+// pass 3: additive CCD of the pairs left by pass 2 whose lower bound is still
+// not above the member's bound.
 // Pairs need very different numbers of steps, and an FP64 warp instruction
 // costs a warp the same whether one lane or 32 use it, so the warps are
 // persistent and hand idle lanes new pairs -- but only once EXACT_REFILL of
@@ -366,24 +386,16 @@ struct ExactLane {
   int it;
 };
 
-// finish a pair: exact t_p (lower-bound flag clear) or a lower bound
-__device__ __forceinline__ void exact_finish(const CcdArgs& A, const ExactLane& L, double* __restrict__ lb_out,
-                                             bool stopped, double t) {
+// finish a pair: exact t_p, or (stopped) a lower bound
+__device__ __forceinline__ void exact_finish(const CcdArgs& A, const ExactLane& L, bool stopped, double t) {
   A.t_out[L.q] = t;
-  if (stopped) {
-    A.cls_out[L.q] = (uint8_t)L.S.cls;
-    lb_out[L.q] = t;
-    return;
-  }
-  A.cls_out[L.q] = (uint8_t)L.S.cls | EXACT;
-  lb_out[L.q] = 2.0;
-  atomicMin(macc_of(A, L.S.mem, MACC_ALPHA), (unsigned long long)__double_as_longlong(t));
+  A.cls_out[L.q] = (uint8_t)L.S.cls | (stopped ? 0 : EXACT);
+  if (!stopped) atomicMin(macc_of(A, L.S.mem, MACC_ALPHA), (unsigned long long)__double_as_longlong(t));
 }
 
 // fetch: a zeroed counter of the pairs handed out
-__global__ void __launch_bounds__(128) k_ccd_exact(CcdArgs A, int64_t m, const uint32_t* __restrict__ list,
-                                                   double* __restrict__ lb_out,
-                                                   unsigned long long* __restrict__ fetch) {
+__global__ void __launch_bounds__(128) k_ccd_exact(CcdArgs A, unsigned long long* __restrict__ fetch) {
+  const int64_t mf = min((int64_t)A.nlist[0], A.np), m = min(mf + (int64_t)A.nlist[1], A.np);
   const unsigned lane = threadIdx.x & 31u;
   const unsigned below = (1u << lane) - 1u;
   ExactLane L;
@@ -399,19 +411,25 @@ __global__ void __launch_bounds__(128) k_ccd_exact(CcdArgs A, int64_t m, const u
       b = __shfl_sync(0xffffffffu, b, 0);
       if ((int64_t)b + nidle >= m) drained = true;  // nothing left after this group
       const int64_t w = (int64_t)b + __popc(idle & below);
-      if (!have && w < m) {
-        L.q = list[w];
+      bool take = !have && w < m;
+      if (take) {
+        L.q = w < mf ? A.list[w] : A.list[A.np - 1 - (w - mf)];
+        const uint64_t key = A.keys[L.q];
+        const int v0 = cb_key_type(key) == CB_KEY_PT ? (int)cb_key_i(key) : A.ev0[cb_key_i(key)];
+        take = __double2float_rd(A.t_out[L.q]) <= member_cap(A, A.members > 1 ? A.vsc[v0] : 0);
+      }
+      if (take) {
         L.S = accd_start(A, L.q);
         if (L.S.lp == 0.0 || L.S.g0 <= 0.0) {  // only reachable through an FP32 bound below 1
           if (L.S.lp != 0.0) {
             atomicOr(A.status, (unsigned long long)CB_DEV_PENETRATION);
             atomicOr(macc_of(A, L.S.mem, MACC_STATUS), (unsigned long long)CB_DEV_PENETRATION);
           }
-          exact_finish(A, L, lb_out, false, L.S.lp == 0.0 ? 1.0 : 0.0);
+          exact_finish(A, L, false, L.S.lp == 0.0 ? 1.0 : 0.0);
         } else {
-          // ceiling: the band's upper end, lowered to the member's minimum as it falls
+          // dropped above the member's bound (pass 2 is over: it no longer moves), or on reaching its minimum so far
           L.hi = __longlong_as_double(*macc_of(A, L.S.mem, MACC_HI));
-          L.cap = fmin(L.hi, __longlong_as_double(*(volatile unsigned long long*)macc_of(A, L.S.mem, MACC_ALPHA)));
+          L.cap = __longlong_as_double(*(volatile unsigned long long*)macc_of(A, L.S.mem, MACC_ALPHA));
           L.g = xmul(ACCD_S, L.S.g0);
           L.t = 0.0;
           L.tl = xdiv(xmul(xsub(1.0, ACCD_S), L.S.g0), L.S.lp);
@@ -435,22 +453,22 @@ __global__ void __launch_bounds__(128) k_ccd_exact(CcdArgs A, int64_t m, const u
       cbg::stencil_distance(S.ee, S.Y0, S.Y1, S.Y2, S.Y3, d);
       const int it = L.it++;
       if (L.t > 0.0 && xsub(d, S.off) < L.g) {
-        exact_finish(A, L, lb_out, false, L.t);
+        exact_finish(A, L, false, L.t);
         have = false;
       } else {
         L.t = xadd(L.t, L.tl);
         if (L.t > 1.0) {
-          exact_finish(A, L, lb_out, false, 1.0);
+          exact_finish(A, L, false, 1.0);
           have = false;
         } else {
           if ((it & 7) == 7)
-            L.cap = fmin(L.hi, __longlong_as_double(*(volatile unsigned long long*)macc_of(A, S.mem, MACC_ALPHA)));
-          if (L.cap < 1.0 && L.t >= L.cap) {  // t_p >= t >= cap: this pair cannot lower the minimum now
-            exact_finish(A, L, lb_out, true, L.t);
+            L.cap = __longlong_as_double(*(volatile unsigned long long*)macc_of(A, S.mem, MACC_ALPHA));
+          if ((L.cap < 1.0 && L.t >= L.cap) || L.t > L.hi) {  // t_p >= t: this pair cannot lower the minimum
+            exact_finish(A, L, true, L.t);
             have = false;
           } else if (it + 1 >= ACCD_MAX_ITER) {
             atomicOr(A.status, (unsigned long long)CB_DEV_ITER_LIMIT);
-            exact_finish(A, L, lb_out, false, L.t);
+            exact_finish(A, L, false, L.t);
             have = false;
           } else {
             L.tl = xdiv(xmul(ACCD_C, xsub(d, S.off)), S.lp);
@@ -468,10 +486,16 @@ __global__ void k_alpha_final(int count, const unsigned long long* __restrict__ 
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m < count) out[m] = __longlong_as_double(macc[(size_t)m * MACC_STRIDE + MACC_ALPHA]);
 }
-__global__ void k_set(unsigned long long* p, unsigned long long v) { *p = v; }
-__global__ void k_macc_set(int count, unsigned long long* __restrict__ macc, int slot, unsigned long long v) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m < count) macc[(size_t)m * MACC_STRIDE + slot] = v;
+// One launch for the resets at the start of a step bound: its counters and
+// every member's minimum, bound and status.
+__global__ void k_ccd_reset(unsigned long long* __restrict__ sc, int count, unsigned long long* __restrict__ macc) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) sc[SC_ITERS] = sc[SC_NLIST] = sc[SC_NU] = sc[SC_NX] = sc[SC_FETCH] = 0ull;
+  if (i < count) {
+    unsigned long long* m = macc + (size_t)i * MACC_STRIDE;
+    m[MACC_ALPHA] = m[MACC_HI] = 0x3ff0000000000000ull;  // 1.0
+    m[MACC_STATUS] = 0ull;
+  }
 }
 
 }  // namespace
@@ -482,19 +506,14 @@ cb_status ccd_run(cb_scene* s, const double* x, const double* p, double* alpha, 
   const int M = s->count;
   unsigned long long* macc = bp<unsigned long long>(s->macc);
   unsigned long long* mi = (unsigned long long*)(sc + SC_ITERS);
-  k_macc_set<<<cb_grid(M), CB_THREADS, 0, cb_count(st)>>>(M, macc, MACC_ALPHA, 0x3ff0000000000000ull);  // 1.0
-  k_macc_set<<<cb_grid(M), CB_THREADS, 0, cb_count(st)>>>(M, macc, MACC_LB, 0x4000000000000000ull);     // 2.0
-  k_macc_set<<<cb_grid(M), CB_THREADS, 0, cb_count(st)>>>(M, macc, MACC_STATUS, 0ull);
-  k_set<<<1, 1, 0, cb_count(st)>>>(mi, 0ull);
+  k_ccd_reset<<<cb_grid(M), CB_THREADS, 0, cb_count(st)>>>((unsigned long long*)sc, M, macc);
   const int64_t np = s->n_ccd;
   if (np > 0) {
     CB_TRY(buf_ensure(s->ccd_t, sizeof(double) * (size_t)np, st));
     CB_TRY(buf_ensure(s->ccd_cls, (size_t)np, st));
-    CB_TRY(buf_ensure(s->ccd_lb, sizeof(double) * (size_t)np, st));
-    CB_TRY(buf_ensure(s->ccd_flag, sizeof(unsigned long long) * (size_t)np, st));
-    CB_TRY(buf_ensure(s->ccd_pos, sizeof(unsigned long long) * ((size_t)np + 1), st));
     CB_TRY(buf_ensure(s->ccd_list, sizeof(uint32_t) * (size_t)np, st));
-    CB_TRY(buf_ensure(s->scan_tmp, sizeof(uint64_t) * (size_t)(cbp::scan_tmp_elems(np) + 8), st));
+    CB_TRY(buf_ensure(s->ccd_ulist, sizeof(uint32_t) * (size_t)np, st));
+    CB_TRY(buf_ensure(s->dlist, sizeof(uint32_t) * (size_t)np, st));
     CcdArgs A;
     A.np = np;
     A.keys = bp<uint64_t>(s->ccd_keys);
@@ -520,115 +539,26 @@ cb_status ccd_run(cb_scene* s, const double* x, const double* p, double* alpha, 
     A.t_out = bp<double>(s->ccd_t);
     A.cls_out = bp<uint8_t>(s->ccd_cls);
     A.macc = macc;
+    A.members = M;
     A.status = (unsigned long long*)(sc + SC_STATUS);
     A.max_iters = mi;
     CB_TRY(to_f32(s, x, bp<double>(s->bwc.cx), s->xf, st));
     CB_TRY(to_f32(s, p, nullptr, s->pf, st));
     A.xf = bp<float4>(s->xf);
     A.pf = bp<float4>(s->pf);
-    CB_TRY(buf_ensure(s->dlist, sizeof(uint32_t) * (size_t)np, st));
-    CB_TRY(buf_ensure(s->ccd_ulist, sizeof(uint32_t) * (size_t)np, st));
     unsigned int* nl = (unsigned int*)(sc + SC_NLIST);
-    k_set<<<1, 1, 0, cb_count(st)>>>((unsigned long long*)(sc + SC_NLIST), 0ull);
-    k_set<<<1, 1, 0, cb_count(st)>>>((unsigned long long*)(sc + SC_NU), 0ull);
     A.ulist = bp<uint32_t>(s->ccd_ulist);
     A.nu = (unsigned int*)(sc + SC_NU);
-    k_ccd_screen<<<cb_grid(np, 128), 128, 0, cb_count(st)>>>(A, bp<double>(s->ccd_lb), bp<uint32_t>(s->dlist), nl);
+    A.list = bp<uint32_t>(s->ccd_list);
+    A.nlist = (unsigned int*)(sc + SC_NX);
+    k_ccd_screen<<<cb_grid(np, 128), 128, 0, cb_count(st)>>>(A, bp<uint32_t>(s->dlist), nl);
     k_ccd_bound<<<std::min<int64_t>(cb_grid(np, 128), (int64_t)s->n_sms * 16), 128, 0, cb_count(st)>>>(
-        A, bp<double>(s->ccd_lb), bp<uint32_t>(s->dlist), nl);
+        A, bp<uint32_t>(s->dlist), nl);
+    k_ccd_refine<<<std::min<int64_t>(cb_grid(np, 128), (int64_t)s->n_sms * 8), 128, 0, cb_count(st)>>>(A);
+    // persistent warps: at most three 128-thread blocks per SM (the kernel's registers)
+    k_ccd_exact<<<std::min<int64_t>(cb_grid(np, 128), (int64_t)s->n_sms * 3), 128, 0, cb_count(st)>>>(
+        A, (unsigned long long*)(sc + SC_FETCH));
     CB_CUDA(cudaGetLastError());
-    // Per member: the pairs left unresolved by pass 1 (lb < 1, listed by the
-    // pass-1 kernels themselves) go through rounds with ceiling
-    // h = 4 L, 16 L, ... (capped at 1) until the member's minimum is <= h.
-    // Members whose minimum is already below every remaining bound are done
-    // after pass 1.
-    std::vector<unsigned long long> hm((size_t)M * MACC_STRIDE);
-    auto read_macc = [&]() -> cb_status {
-      CB_CUDA(cudaMemcpyAsync(s->hstage_host, macc, sizeof(unsigned long long) * MACC_STRIDE * M,
-                              cudaMemcpyDeviceToHost, st));
-      CB_CUDA(cudaStreamSynchronize(st));
-      memcpy(hm.data(), s->hstage_host, sizeof(unsigned long long) * MACC_STRIDE * M);
-      return CB_OK;
-    };
-    auto upload_band = [&](const std::vector<double>& lo, const std::vector<double>& hi) -> cb_status {
-      // hm holds the device values read just before, and no kernel runs in between
-      for (int m = 0; m < M; ++m) {
-        memcpy(&hm[(size_t)m * MACC_STRIDE + MACC_LO], &lo[m], 8);
-        memcpy(&hm[(size_t)m * MACC_STRIDE + MACC_HI], &hi[m], 8);
-      }
-      memcpy(s->hstage_host, hm.data(), sizeof(unsigned long long) * MACC_STRIDE * M);
-      CB_CUDA(cudaMemcpyAsync(macc, s->hstage_host, sizeof(unsigned long long) * MACC_STRIDE * M,
-                              cudaMemcpyHostToDevice, st));
-      return CB_OK;
-    };
-    auto dbl = [](unsigned long long b) {
-      double d;
-      memcpy(&d, &b, 8);
-      return d;
-    };
-    CB_TRY(read_macc());
-    std::vector<double> lo(M, 3.0), hi(M, -1.0);
-    std::vector<char> done(M, 1);
-    bool any = false;
-    for (int m = 0; m < M; ++m) {
-      const double L = dbl(hm[(size_t)m * MACC_STRIDE + MACC_LB]);
-      const double mm = dbl(hm[(size_t)m * MACC_STRIDE + MACC_ALPHA]);
-      if (!(L > 1.0 || mm <= L)) {
-        done[m] = 0;
-        lo[m] = -1.0;
-        hi[m] = 1.0;
-        any = true;
-      }
-    }
-    uint32_t* tot = (uint32_t*)(sc + SC_COUNT1);
-    int64_t nu = 0;
-    if (any) {
-      uint64_t hn;
-      CB_TRY(read_scalars(s, SC_NU, 1, &hn, st));
-      nu = (int64_t)(uint32_t)hn;
-      for (int m = 0; m < M; ++m)
-        if (!done[m]) hi[m] = std::min(1.0, 4.0 * dbl(hm[(size_t)m * MACC_STRIDE + MACC_LB]));
-      any = nu > 0;
-    }
-    while (any) {
-      CB_TRY(upload_band(lo, hi));
-      unsigned long long* flag64 = bp<unsigned long long>(s->ccd_flag);
-      unsigned long long* pos64 = bp<unsigned long long>(s->ccd_pos);
-      unsigned long long* tot64 = (unsigned long long*)tot;
-      k_ccd_select_u<<<cb_grid(nu), CB_THREADS, 0, cb_count(st)>>>(
-          nu, bp<uint32_t>(s->ccd_ulist), bp<uint64_t>(s->ccd_keys), bp<int32_t>(s->ev0), bp<int32_t>(s->vsc),
-          bp<double>(s->ccd_lb), macc, flag64);
-      cbp::exclusive_scan<unsigned long long, unsigned long long>(flag64, pos64, nu,
-                                                                  bp<unsigned long long>(s->scan_tmp), tot64, st);
-      k_list_u<<<cb_grid(nu), CB_THREADS, 0, cb_count(st)>>>(nu, bp<uint32_t>(s->ccd_ulist), flag64, pos64, tot64,
-                                                             bp<uint32_t>(s->ccd_list));
-      uint64_t hmsel;
-      CB_TRY(read_scalars(s, SC_COUNT1, 1, &hmsel, st));
-      const int64_t msel = (int64_t)(hmsel & 0xffffffffull) + (int64_t)(hmsel >> 32);
-      if (msel > 0) {
-        // persistent warps: at most three 128-thread blocks per SM (the
-        // kernel's registers), fewer when the list is short
-        unsigned long long* fetch = (unsigned long long*)(sc + SC_FETCH);
-        CB_CUDA(cudaMemsetAsync(fetch, 0, sizeof(unsigned long long), st));
-        const int64_t g = std::min<int64_t>(cb_grid(msel, 128), (int64_t)s->n_sms * 3);
-        k_ccd_exact<<<(int)g, 128, 0, cb_count(st)>>>(A, msel, bp<uint32_t>(s->ccd_list), bp<double>(s->ccd_lb),
-                                                      fetch);
-      }
-      CB_CUDA(cudaGetLastError());
-      CB_TRY(read_macc());
-      any = false;
-      for (int m = 0; m < M; ++m) {
-        if (done[m]) continue;
-        const double mm = dbl(hm[(size_t)m * MACC_STRIDE + MACC_ALPHA]);
-        if (mm <= hi[m] || hi[m] >= 1.0) {
-          done[m] = 1;  // every unfinished pair has t_p >= lb_p >= min(h, m)
-          hi[m] = -1.0;
-        } else {
-          hi[m] = std::min(1.0, 4.0 * hi[m]);
-          any = true;
-        }
-      }
-    }
   }
   if (alpha) k_alpha_final<<<cb_grid(M), CB_THREADS, 0, cb_count(st)>>>(M, macc, alpha);
   CB_CUDA(cudaGetLastError());
@@ -649,14 +579,15 @@ cb_status ccd_run(cb_scene* s, const double* x, const double* p, double* alpha, 
 // by every call on a device: calls that overlap in time on one device (two
 // streams, two host threads) race and give wrong results.
 //
-// Layout (64-bit words): NA_SLOTS accumulator words (alpha bits, smallest
-// lower bound bits, condition flags), then one lower bound per stencil.
+// Layout: NA_SLOTS 64-bit accumulator words (alpha bits, smallest upper bound
+// bits, condition flags, list lengths), then per stencil an FP32 lower bound
+// and a list entry (the stencils left for the FP64 iteration: point-triangle
+// from the front, edge-edge from the back).
 
 namespace {
 constexpr int NA_SLOTS = 32;  // 256 bytes: keeps the per-stencil part 256-byte aligned
-constexpr int NA_ALPHA = 0, NA_LB = 1, NA_FLAGS = 2;
+constexpr int NA_ALPHA = 0, NA_HI = 1, NA_FLAGS = 2, NA_COUNT = 3;  // NA_COUNT: two uint32
 constexpr unsigned long long NA_ONE = 0x3ff0000000000000ull;  // 1.0
-constexpr unsigned long long NA_TWO = 0x4000000000000000ull;  // 2.0: "no value"
 }  // namespace
 
 static __device__ __align__(256) unsigned long long g_noalloc_scratch[NA_SLOTS + CB_NOALLOC_MAX_STENCILS];
@@ -671,8 +602,18 @@ struct NaArgs {
   const double* __restrict__ off;   // [ns] offset
   const double* __restrict__ x;
   const double* __restrict__ p;
-  unsigned long long* __restrict__ scr;
+  unsigned long long* scr;
 };
+
+__device__ __forceinline__ float* na_lb(const NaArgs& A) { return (float*)(A.scr + NA_SLOTS); }
+__device__ __forceinline__ uint32_t* na_list(const NaArgs& A) {
+  return (uint32_t*)(A.scr + NA_SLOTS) + CB_NOALLOC_MAX_STENCILS;
+}
+// an upper bound of the smallest t_p: FP32 brackets and exact values so far (rounded up)
+__device__ __forceinline__ float na_cap(const NaArgs& A) {
+  const volatile unsigned long long* s = A.scr;
+  return __double2float_ru(fmin(__longlong_as_double(s[NA_ALPHA]), __longlong_as_double(s[NA_HI])));
+}
 
 struct NaStart {
   bool ee;
@@ -717,64 +658,75 @@ __device__ __forceinline__ bool na_start(const NaArgs& A, int64_t q, NaStart& S)
   return isfinite(S.lp) && isfinite(S.g0);
 }
 
-// one atomicMin per warp of the lanes' non-negative values (2.0 = none)
-__device__ __forceinline__ void na_warp_min(unsigned long long* slot, double v) {
-  unsigned long long b = (unsigned long long)__double_as_longlong(v);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long u = __shfl_xor_sync(0xffffffffu, b, o);
-    b = u < b ? u : b;
-  }
-  if ((threadIdx.x & 31) == 0 && b < NA_TWO) atomicMin(slot, b);
-}
-
 __global__ void k_na_init(unsigned long long* __restrict__ scr) {
   if (threadIdx.x == 0) {
-    scr[NA_ALPHA] = NA_ONE;
-    scr[NA_LB] = NA_TWO;
-    scr[NA_FLAGS] = 0ull;
+    scr[NA_ALPHA] = scr[NA_HI] = NA_ONE;
+    scr[NA_FLAGS] = scr[NA_COUNT] = 0ull;
   }
 }
 
-// first step of every stencil: resolves t_p = 1 (no motion, or the first step
-// already passes 1) and t_p = 0 (at or inside the offset); otherwise stores
-// the lower bound (1-s) g0 / l_p of t_p
-__global__ void __launch_bounds__(128) k_na_first(NaArgs A) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  double m_exact = 2.0, m_lb = 2.0;
-  if (q < A.ns) {
-    NaStart S;
-    double lbq = 2.0;
-    if (!na_start(A, q, S)) {
-      atomicOr(&A.scr[NA_FLAGS], (unsigned long long)CB_NOALLOC_BAD_STENCIL);
-    } else if (S.lp == 0.0) {
-      m_exact = 1.0;
-    } else if (S.g0 <= 0.0) {
-      m_exact = 0.0;
-      atomicOr(&A.scr[NA_FLAGS], (unsigned long long)CB_DEV_PENETRATION);
-    } else {
-      const double tl = xdiv(xmul(xsub(1.0, ACCD_S), S.g0), S.lp);
-      if (tl > 1.0) {
-        m_exact = 1.0;
+// FP32 brackets of the stencils' t_p (accd32.cuh), in two launches: every
+// NA_SAMPLE-th stencil first, so that the rest meet an upper bound that already
+// drops most of them after their first step.  The stencils still below it are
+// listed.  Grid-stride; the trip count is uniform over a warp so that every
+// lane reaches the appends.
+constexpr int NA_SAMPLE = 16;
+
+__global__ void __launch_bounds__(128) k_na_refine(NaArgs A, int part) {
+  const int64_t ns = A.ns, head = (ns + NA_SAMPLE - 1) / NA_SAMPLE, m = part == 0 ? head : ns - head;
+  unsigned int* cnt = (unsigned int*)&A.scr[NA_COUNT];
+  for (int64_t w0 = (int64_t)blockIdx.x * blockDim.x; w0 < m; w0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t w = w0 + threadIdx.x;
+    bool keep = false, ee = false;
+    // part 1: the w-th stencil that is not a multiple of NA_SAMPLE
+    const int64_t q = part == 0 ? w * NA_SAMPLE : w + w / (NA_SAMPLE - 1) + 1;
+    if (w < m) {
+      int v[4];
+      bool ok = true;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        v[k] = A.st[4 * q + k];
+        ok = ok && v[k] >= 0 && v[k] < A.n;
+      }
+      const double off = A.off[q];
+      if (!ok || !(off >= 0.0) || !isfinite(off)) {
+        atomicOr(&A.scr[NA_FLAGS], (unsigned long long)CB_NOALLOC_BAD_STENCIL);
       } else {
-        lbq = tl;
-        m_lb = tl;
+        ee = A.ee[q] != 0;
+        cbb::Motion32 M;
+        M.ee = ee;
+        M.off_dn = __double2float_rd(off);
+        M.off_up = __double2float_ru(off);
+        pair_motion32(A.x, A.p, A.n, v, M);
+        float lo = 0.f, hi = 1.f;
+        const int r = cbb::motion_slopes(M) ? cbb::accd_bounds32(M, [&] { return na_cap(A); }, lo, hi) : -1;
+        if (r == 0 && hi < 1.f) atomicMin(&A.scr[NA_HI], (unsigned long long)__double_as_longlong((double)hi));
+        keep = r < 0 || (r == 0 && lo <= na_cap(A));
+        if (keep) na_lb(A)[q] = r < 0 ? 0.f : lo;
       }
     }
-    A.scr[NA_SLOTS + q] = (unsigned long long)__double_as_longlong(lbq);
+    warp_append(keep && !ee, (uint32_t)q, na_list(A), &cnt[0]);
+    warp_append_back(keep && ee, (uint32_t)q, na_list(A), ns, &cnt[1]);
   }
-  na_warp_min(&A.scr[NA_ALPHA], m_exact);
-  na_warp_min(&A.scr[NA_LB], m_lb);
 }
 
-// full additive CCD of stencil q (the iteration of k_ccd_exact)
+// full additive CCD of stencil q (the iteration of k_ccd_exact), dropped once
+// t is above the smallest upper bound or reaches the smallest exact t_p
 __device__ double na_iterate(const NaArgs& A, int64_t q) {
   NaStart S;
-  if (!na_start(A, q, S)) return 2.0;
+  if (!na_start(A, q, S)) {
+    atomicOr(&A.scr[NA_FLAGS], (unsigned long long)CB_NOALLOC_BAD_STENCIL);
+    return 1.0;
+  }
   if (S.lp == 0.0) return 1.0;
-  if (S.g0 <= 0.0) return 0.0;
+  if (S.g0 <= 0.0) {
+    atomicOr(&A.scr[NA_FLAGS], (unsigned long long)CB_DEV_PENETRATION);
+    return 0.0;
+  }
+  const volatile unsigned long long* scr = A.scr;
+  const double top = __longlong_as_double(scr[NA_HI]);  // no longer moves
   const double g = xmul(ACCD_S, S.g0);
-  double t = 0.0, d;
+  double t = 0.0, d, cap = __longlong_as_double(scr[NA_ALPHA]);
   double tl = xdiv(xmul(xsub(1.0, ACCD_S), S.g0), S.lp);
   for (int it = 0; it < ACCD_MAX_ITER; ++it) {
     S.Y0 = axpy3(S.Y0, tl, S.Q0);
@@ -785,48 +737,24 @@ __device__ double na_iterate(const NaArgs& A, int64_t q) {
     if (t > 0.0 && xsub(d, S.off) < g) return t;
     t = xadd(t, tl);
     if (t > 1.0) return 1.0;
+    if ((it & 7) == 7) cap = __longlong_as_double(scr[NA_ALPHA]);
+    if (t > top || (cap < 1.0 && t >= cap)) return 1.0;  // t_p >= t: cannot lower the minimum
     tl = xdiv(xmul(ACCD_C, xsub(d, S.off)), S.lp);
   }
   atomicOr(&A.scr[NA_FLAGS], (unsigned long long)CB_DEV_ITER_LIMIT);
   return t;
 }
 
-// Bands of lower bounds, as in ccd_run but decided on the device: band 0 is
-// (-1, min(1, 2L)] with L the smallest bound; band 1 is (hi0, min(1, m)] with
-// m the minimum after band 0.  Every stencil left after band 1 has
-// t_p >= lb_p > m, so alpha = min(1, m) exactly.  The minimum is read once per
-// block: a smaller value seen later only narrows the band to stencils that
-// still could lower it.
-__global__ void __launch_bounds__(128) k_na_band(NaArgs A, int band) {
-  __shared__ double s_lo, s_hi;
-  if (threadIdx.x == 0) {
-    const double L = __longlong_as_double(A.scr[NA_LB]);
-    const double m = __longlong_as_double(A.scr[NA_ALPHA]);
-    const double h0 = fmin(1.0, 2.0 * L);
-    double lo = 3.0, hi = 3.0;  // empty band
-    if (!(L > 1.0 || m <= L)) {
-      if (band == 0) {
-        lo = -1.0;
-        hi = h0;
-      } else if (!(m <= h0 || h0 >= 1.0)) {
-        lo = h0;
-        hi = fmin(1.0, m);
-      }
-    }
-    s_lo = lo;
-    s_hi = hi;
-  }
-  __syncthreads();
-  const double lo = s_lo, hi = s_hi;
-  if (lo >= 3.0) return;  // uniform over the block
-  for (int64_t w0 = (int64_t)blockIdx.x * blockDim.x; w0 < A.ns; w0 += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t q = w0 + threadIdx.x;
-    double t = 2.0;
-    if (q < A.ns) {
-      const double lbq = __longlong_as_double(A.scr[NA_SLOTS + q]);
-      if (lbq > lo && lbq <= hi) t = na_iterate(A, q);
-    }
-    na_warp_min(&A.scr[NA_ALPHA], t);
+// the listed stencils whose lower bound is still not above the bound; every
+// other stencil has t_p above it, so alpha = min(1, m) exactly
+__global__ void __launch_bounds__(128) k_na_exact(NaArgs A) {
+  const unsigned int* cnt = (const unsigned int*)&A.scr[NA_COUNT];
+  const int64_t mf = min((int64_t)cnt[0], A.ns), m = min(mf + (int64_t)cnt[1], A.ns);
+  for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < m; w += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t q = w < mf ? na_list(A)[w] : na_list(A)[A.ns - 1 - (w - mf)];
+    if (!(na_lb(A)[q] <= na_cap(A))) continue;
+    const double t = na_iterate(A, q);
+    if (t < 1.0) atomicMin(&A.scr[NA_ALPHA], (unsigned long long)__double_as_longlong(t));
   }
 }
 
@@ -914,11 +842,12 @@ cb_status ccd_step_noalloc(const double* x_dev, const double* p_dev, int32_t n_v
     A.x = x_dev;
     A.p = p_dev;
     A.scr = scr;
-    k_na_first<<<cb_grid(n_stencils, 128), 128, 0, cb_count(st)>>>(A);
-    // the band kernels stride over the list: up to 16 resident blocks of 128 threads per SM
-    const int gb = (int)std::min<int64_t>(cb_grid(n_stencils, 128), (int64_t)nsm * 16);
-    k_na_band<<<gb, 128, 0, cb_count(st)>>>(A, 0);
-    k_na_band<<<gb, 128, 0, cb_count(st)>>>(A, 1);
+    // grid-stride over the list: up to 8 (FP32) and 4 (FP64) resident blocks of 128 threads per SM
+    const int64_t g = cb_grid(n_stencils, 128);
+    const int g32 = (int)std::min<int64_t>(g, (int64_t)nsm * 8);
+    k_na_refine<<<g32, 128, 0, cb_count(st)>>>(A, 0);
+    k_na_refine<<<g32, 128, 0, cb_count(st)>>>(A, 1);
+    k_na_exact<<<(int)std::min<int64_t>(g, (int64_t)nsm * 4), 128, 0, cb_count(st)>>>(A);
   }
   k_na_final<<<1, 32, 0, cb_count(st)>>>(scr, alpha_dev, flags_dev);
   CB_CUDA(cudaGetLastError());

@@ -137,7 +137,7 @@ struct cb_scene {
   DevBuf vsc;           // int32 [n] member of each vertex
   std::vector<int64_t> voff, eoff, toff;  // member offsets of vertices, edges, triangles (count+1)
   int64_t n_frest_pt = 0;                 // shells: point-triangle keys at the head of frest
-  DevBuf macc;          // per member: double energy, u64 alpha bits, u64 lb bits, u64 status, double lo, hi
+  DevBuf macc;          // per member: double energy, u64 alpha bits, u64 status, double upper bound of alpha
   void* hstage_host = nullptr;  // pinned staging (the largest per-member record x members + 256)
   cudaStream_t last_stream = nullptr;
   int device = 0;
@@ -205,10 +205,9 @@ struct cb_scene {
   DevBuf xf, pf;         // float [3][n]: centred FP32 copies of x and of p
   DevBuf dlist;          // uint32: candidates / CCD pairs queued for the FP64 phase
   DevBuf ccd_keys;      // uint64 [nccd]
-  DevBuf ccd_t;         // double [nccd]
-  DevBuf ccd_cls;       // uint8 [nccd] class | 0x80 when t is exact
-  DevBuf ccd_lb;        // double [nccd] lower bound of t (2 when resolved)
-  DevBuf ccd_flag, ccd_pos, ccd_list;  // band selection: u64 kind counts (flag, scan), uint32 list
+  DevBuf ccd_t;         // double [nccd] t_p or a lower bound of it; not written where the class byte has CB_CCD_ONE
+  DevBuf ccd_cls;       // uint8 [nccd] class | CB_CCD_EXACT when t is exact | CB_CCD_ONE when it is 1
+  DevBuf ccd_list;      // uint32 pairs left for the FP64 iteration
   DevBuf ccd_ulist;     // uint32 pairs still unresolved after the first-step pass
   int64_t n_ccd = 0;
   // lagged friction (friction_lag / friction_eval / friction_spmv)
@@ -258,12 +257,13 @@ enum {
   SC_KSPLIT = 16,       // two uint32 counters: face / line-line pairs, the other active pairs
   SC_NOVF = 17,         // broad phase: entries whose pairs overflow the stage
   SC_NBK = 18,          // BSR pattern: keys left after the per-run sets of k_block_keys
-  SC_FETCH = 19,        // ccd_step, exact rounds: pairs of the list handed out so far
+  SC_FETCH = 19,        // ccd_step, FP64 iteration: pairs of the list handed out so far
   SC_NMOLL = 20,        // barrier_eval: mollified edge-edge pairs
   SC_GEO_COUNT = 21,    // geodesic rest filter: (edge, vertex) entries below the activation
   SC_GEO_ERR = 22,      // ... error bits of its sources (a fixed capacity exceeded)
   SC_NVLONG = 23,       // shell broad phase: entries of flat_vlong
-  SC_N = 24
+  SC_NX = 24,           // ccd_step: two uint32 counters, point-triangle and edge-edge pairs of the FP64 iteration
+  SC_N = 25
 };
 // read_scalars stages up to SC_N scalars through the pinned host scratch
 static_assert(SC_N <= 64, "the scalars must fit the pinned scratch");
@@ -271,7 +271,9 @@ static_assert(SC_N <= 64, "the scalars must fit the pinned scratch");
 static inline uint64_t* scalars(cb_scene* s) { return (uint64_t*)s->dev_scalars.p; }
 
 // per-member accumulator slots (uint64 / double each) inside macc
-enum { MACC_E = 0, MACC_ALPHA = 1, MACC_LB = 2, MACC_STATUS = 3, MACC_LO = 4, MACC_HI = 5, MACC_STRIDE = 6 };
+enum { MACC_E = 0, MACC_ALPHA = 1, MACC_STATUS = 2, MACC_HI = 3, MACC_STRIDE = 4 };
+// flags of a CCD pair's class byte: t_p is exact (else ccd_t holds a lower bound), and it is 1
+constexpr uint8_t CB_CCD_EXACT = 0x80, CB_CCD_ONE = 0x40;
 
 // read n uint64 device scalars into host (sync on stream)
 cb_status read_scalars(cb_scene* s, int first, int count, uint64_t* out, cudaStream_t st);
