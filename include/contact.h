@@ -173,9 +173,9 @@ typedef struct {
   int64_t n_hess_face;        /* last barrier_eval: active face / line-line pairs (9x9 projection) */
   int64_t n_hess_pe_frame;    /* ... point-edge pairs projected in their own frame (3x3 + 2x2) */
   int64_t n_hess_pe;          /* ... point-edge pairs on the generic 6x6 projection */
-  int64_t n_pair_overflow;    /* last broad phase of a rod scene (ccd_step's, once a pass ran it): entries
-                                 with more pairs than the 32 keys the count pass stages, re-tested by the fill
-                                 pass (shell scenes keep one hit bit per test and never re-test: 0) */
+  int64_t n_pair_overflow;    /* last broad phase of a rod scene (ccd_step's, once a pass ran it): crowded rows --
+                                 an edge against a cluster of 32 others with more than 16 of them its partners
+                                 (shell scenes: 0) */
   int64_t n_mollified;        /* last barrier_eval with CB_EE_MOLLIFIER: edge-edge pairs below their threshold */
   int64_t n_stencil_dropped;  /* last contact_filter with CB_PER_STENCIL: filtered broad-phase pairs outside
                                  their own width, removed from the candidates */
@@ -196,10 +196,10 @@ cb_status cb_scene_destroy(cb_scene* scene);
 
 /* (a) Broad phase, Sec. 3.3: every non-incident primitive pair (shells:
  * point-triangle and edge-edge; rods: edge-edge) whose FP64 bounding boxes of
- * x, each inflated by a/2, overlap (closed intervals).  Runs an FP32 spatial
- * hash with outward-rounded boxes (a provable superset) and decides ambiguous
- * pairs in FP64.  x_dev: DEVICE [3][n] FP64, read during the call's kernels.
- * Result (scene-owned, kept in hash-cell order; the getters return it sorted
+ * x, each inflated by a/2, overlap (closed intervals).  Tests FP32 boxes
+ * rounded outwards (a provable superset), cluster by cluster, and decides
+ * ambiguous pairs in FP64.  x_dev: DEVICE [3][n] FP64, read during the call's kernels.
+ * Result (scene-owned, kept in no particular order; the getters return it sorted
  * by key) is the input of the next three calls. */
 cb_status contact_build(cb_scene* scene, const double* x_dev, void* stream);
 
@@ -246,7 +246,7 @@ cb_status ccd_step(cb_scene* scene, const double* x_dev, const double* p_dev, do
 /* Batch: several scenes of one kind in one pass (one launch per stage for all
  * of them).  The batch concatenates the members' vertices, edges and
  * triangles in member order (offsets: cb_batch_offsets) and keeps each
- * member's parameters, filter tables, hash grid and results separate; pairs of
+ * member's parameters, filter tables, clusters and results separate; pairs of
  * different members are never formed.  It copies what it needs at creation:
  * members may be destroyed afterwards.  allocator: as for cb_scene_create (the
  * batch's own buffers; the members keep theirs).  Use it with the four pass calls: x, p
@@ -388,12 +388,12 @@ cb_status cb_get_stage_ms(cb_scene* scene, float* ms5);
  * candidates; entries past 7 are 0.  sync.  Errors: CB_ERR_ARG. */
 cb_status cb_get_stage_times(cb_scene* scene, float* ms, int32_t count);
 /* Tuning knobs of a broad phase (no counterpart in the paper; no result
- * depends on them, only speed).  phase 0: contact_build's broad phase, 1:
- * ccd_step's swept broad phase.  cell_factor in (0, 64]: hash cell edge =
- * factor x the members' mean primitive box extent (rounded to a quarter
- * octave; default 1).  pair_block: threads per block of the pair enumeration,
- * 64, 128 or 256 (default 256).  A batch starts from its first member's
- * settings.  Errors: CB_ERR_ARG. */
+ * depends on them).  phase 0: contact_build's broad phase, 1: ccd_step's swept
+ * broad phase.  cell_factor in (0, 64] (default 1) and pair_block 64, 128 or
+ * 256 (default 256) sized the cells and blocks of a cell hash; the cluster
+ * broad phase has neither, so they are checked, kept and returned but change
+ * nothing.  A batch starts from its first member's settings.  Errors:
+ * CB_ERR_ARG. */
 cb_status cb_set_tuning(cb_scene* scene, int32_t phase, float cell_factor, int32_t pair_block);
 cb_status cb_get_tuning(cb_scene* scene, int32_t phase, float* cell_factor, int32_t* pair_block);
 /* enable (1) / disable (0) the stage events; default off */

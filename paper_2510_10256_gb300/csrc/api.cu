@@ -84,7 +84,7 @@ static cb_status upload(DevBuf& b, const T* h, size_t count, cudaStream_t st) {
 
 static void scene_release(cb_scene* s) {
   cudaStream_t st = s->last_stream;
-  DevBuf* bufs[] = {&s->ev0, &s->ev1, &s->tv, &s->comp, &s->rest, &s->rod_ptr, &s->S, &s->win, &s->wst,
+  DevBuf* bufs[] = {&s->ev0, &s->ev1, &s->tv, &s->comp, &s->rest, &s->rod_ptr, &s->slots, &s->cinfo, &s->supers, &s->jobs, &s->S, &s->win, &s->wst,
                     &s->rloop, &s->rlast, &s->elen2, &s->hmoll, &s->mlist, &s->ruv, &s->frest,
                     &s->frest_dbar, &s->frest_j, &s->frow_pt, &s->frow_ee, &s->dbar_comp, &s->cand, &s->klass, &s->cand_alt, &s->klass_alt, &s->cd, &s->cflag, &s->cpos, &s->ctype, &s->ccls, &s->aidx,
                     &s->bkey[0], &s->bkey[1], &s->bflag, &s->bpos, &s->bsr_row, &s->bsr_col, &s->bsr_val,
@@ -92,11 +92,8 @@ static void scene_release(cb_scene* s) {
                     &s->fr_key, &s->fr_st, &s->fr_dat, &s->fr_hw, &s->dev_scalars};
   for (DevBuf* b : bufs) buf_free(*b, st);
   for (BroadWork* w : {&s->bw, &s->bwc}) {
-    DevBuf* wb[] = {&w->grids, &w->cx, &w->box32,   &w->box64,  &w->box_raw, &w->bounds,   &w->cell_cnt, &w->cell_off, &w->ekey[0], &w->ekey[1],
-                    &w->eval[0], &w->eval[1], &w->run_flag, &w->run_id,   &w->run_start, &w->pair_cnt,
-                    &w->pair_off, &w->ebox, &w->ckey[0], &w->ckey[1],  &w->stage, &w->ovl, &w->scan_tmp, &w->hist,
-                    &w->flat_len, &w->flat_off, &w->flat_j0, &w->flat_bits, &w->flat_slen, &w->flat_sbits,
-                    &w->flat_lflag, &w->flat_lpos, &w->flat_lidx, &w->flat_llen, &w->flat_vlong};
+    DevBuf* wb[] = {&w->cx, &w->box, &w->cbox, &w->sbox, &w->box_raw, &w->bounds, &w->tiles,
+                    &w->ckey[0], &w->ckey[1], &w->scan_tmp, &w->hist};
     for (DevBuf* b : wb) buf_free(*b, st);
   }
   cudaStreamSynchronize(st);
@@ -418,7 +415,8 @@ cb_status cb_scene_create(const cb_scene_desc* d, const cb_allocator* allocator,
   if (d->kind == CB_SHELL && (rc = buf_ensure(s->rloop, 16, st)) != CB_OK) return fail(rc);
   for (auto& e : s->ev)
     if (cudaEventCreate(&e) != cudaSuccess) return fail(CB_ERR_CUDA);
-  // the rest broad phase reads the member parameters (box inflation, primitive count)
+  if ((rc = clusters_build(s, d->rest_xyz, st)) != CB_OK) return fail(rc);
+  // the rest broad phase reads the member parameters (box inflation)
   if ((rc = upload_members(s, st)) != CB_OK) return fail(rc);
   if ((rc = filter_precompute(s, st)) != CB_OK) return fail(rc);
   // the adjacency served the geodesic rest filter only
@@ -568,6 +566,7 @@ cb_status cb_batch_create(cb_scene* const* members, int32_t count, const cb_allo
       wee += nee;
     }
   }
+  if ((rc = clusters_concat(b, members, st)) != CB_OK) return fail(rc);
   if (cudaGetLastError() != cudaSuccess) return fail(CB_ERR_CUDA);
   b->n_frest = b->kind == CB_SHELL ? nf : 0;
   b->n_frest_pt = nf_pt;
@@ -724,7 +723,7 @@ cb_status cb_get_stage_times(cb_scene* s, float* ms, int32_t count) {
 }
 
 // Ascending order of 64-bit keys on the host (the pass keeps its pair lists
-// in hash-cell order; the getters return them sorted): LSD radix sort of
+// in tile order; the getters return them sorted): LSD radix sort of
 // (key, original index) with 16-bit digits, skipping digits that are equal
 // in every key.  idx (optional) receives the original positions.
 static void sort_keys(std::vector<uint64_t>& keys, std::vector<uint32_t>* idx) {

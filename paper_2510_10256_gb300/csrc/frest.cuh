@@ -4,7 +4,7 @@
 // table is sorted by key (type, i, j), so the keys with one first primitive i
 // form a contiguous row; per-row offsets (by vertex for point-triangle keys,
 // by edge for edge-edge keys) bound the search to that row, a few dozen keys
-// that consecutive candidates (in hash-cell order, grouped by i) share.
+// that consecutive candidates (of one tile of primitives) share.
 #pragma once
 #include <cstdint>
 

@@ -429,7 +429,7 @@ __global__ void k_active_compact(int64_t nc, const uint32_t* __restrict__ flag, 
 // 16 (row, col) block keys of each active stencil
 // BSR pattern keys (row << bits_n | col) of the 16 blocks of every active
 // stencil, made distinct within each run of BK_PAIRS active pairs (in
-// candidate order, i.e. hash-cell order, a run shares most of its vertices:
+// candidate order, i.e. tile by tile, a run shares most of its vertices:
 // its 16 x 256 keys hold about a fifth as many distinct ones) through an
 // open-addressing set in shared memory (linear probing, at most half full,
 // each probe sequence bounded by the table size).  The distinct keys of each

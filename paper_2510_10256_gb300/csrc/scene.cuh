@@ -70,47 +70,18 @@ struct MemberParams {
   int32_t per_stencil;    // CB_PER_STENCIL: class-F candidates outside their own width are dropped
 };
 
-// Spatial-hash grid of one member.
-struct Grid {
-  float ox, oy, oz, inv;
-  int dx, dy, dz, pad;
-};
-
 // Workspace of one broad phase (static or swept) -- reused between calls.
 struct BroadWork {
-  float cell_factor = 1.0f;  // hash cell edge = factor x mean primitive box extent (tuning knob)
-  int pair_block = CB_THREADS;  // threads per block of the pair enumeration (tuning knob)
-  DevBuf box32;       // float4 lo, float4 hi per primitive
-  DevBuf box64;       // double lo[3], hi[3] per primitive
+  // cb_set_tuning's knobs: kept and returned; the cluster broad phase has no cells to size
+  float cell_factor = 1.0f;
+  int pair_block = CB_THREADS;
+  DevBuf box;         // float4 lo, float4 hi per slot (inflated, rounded outwards)
+  DevBuf cbox, sbox;  // ... per cluster and per supercluster
   DevBuf box_raw;     // per-stencil activation (static phase): double lo[3], hi[3] per primitive, not inflated
-  DevBuf bounds;      // per member: 6 x uint32 ordered-float min/max, 2 pad, double extent sum
-  DevBuf grids;       // Grid per member
+  DevBuf bounds;      // per member: 6 x uint32 ordered-float min/max
   DevBuf cx;          // per member: double centre[3], X (max |coordinate - centre|)
-  DevBuf cell_cnt;    // uint32 per primitive
-  DevBuf cell_off;    // uint32 per primitive (+1)
-  DevBuf ekey[2];     // uint64 (member << 30 | Morton cell) per entry (ping-pong); shells: shifted up by
-                      // 12 bits above the entry's type group and x level in the cell
-  DevBuf eval[2];     // uint32 primitive per entry
-  DevBuf run_flag;    // uint32 per entry
-  DevBuf run_id;      // uint32 per entry
-  DevBuf run_start;   // uint32 per run (+1)
-  DevBuf pair_cnt;    // uint32 per entry
-  DevBuf pair_off;    // uint32 per entry (+1)
-  DevBuf ebox;        // float4 lo, float4 hi per entry (boxes gathered into entry order)
-  DevBuf ckey[2];     // uint64 compact candidate keys (ping-pong)
-  DevBuf stage;       // uint64 [PAIR_STAGE][entries]: the count pass's first pairs of each entry
-  DevBuf ovl;         // uint32 entries with more pairs than the stage holds
-  DevBuf flat_len;    // shells: uint32 per entry, the length of a long swept partner range
-  DevBuf flat_lflag;  // shells: uint32 per entry (+1), 1 for a long range
-  DevBuf flat_lpos;   // shells: uint32 per entry (+1), its place among the long entries (scan of flat_lflag)
-  DevBuf flat_lidx;   // shells: uint32 per long entry, the entry
-  DevBuf flat_llen;   // shells: uint32 per long entry (+1), its range length
-  DevBuf flat_vlong;  // shells: uint32, the long entries with ranges of FLAT_EMIT_WARP slots or more (any order)
-  DevBuf flat_off;    // shells: uint64 per long entry (+1), its first test slot (scan of flat_llen)
-  DevBuf flat_j0;     // shells: uint32 per entry, its first partner
-  DevBuf flat_bits;   // shells: one hit bit per test slot
-  DevBuf flat_slen;   // shells: uint8 per entry, the length of a short range (tested per entry)
-  DevBuf flat_sbits;  // shells: uint32 per entry, the hits of a short range
+  DevBuf tiles;       // uint2 pairs of overlapping clusters
+  DevBuf ckey[2];     // uint64 compact candidate keys (ping-pong; sorted lists only)
   DevBuf scan_tmp;
   DevBuf hist;
 };
@@ -150,6 +121,12 @@ struct cb_scene {
   DevBuf comp;          // int32 [n]
   DevBuf rest;          // double [3][n]
   DevBuf rod_ptr;       // int32 [n_rods+1] (rods)
+  // clusters of 32 primitives and superclusters of 32 clusters (broad.cu), fixed at creation
+  int n_clusters = 0, n_supers = 0, n_jobs = 0;
+  DevBuf slots;         // int4 [n_clusters][32]: a primitive's vertices (-1: none) and its index within its kind (-1: pad)
+  DevBuf cinfo;         // uint32 [n_clusters] member << 2 | kind (0 vertex, 1 triangle, 2 edge)
+  DevBuf supers;        // int4: first cluster, count, member, kind
+  DevBuf jobs;          // int4: row supercluster, first and end column supercluster (at most 32)
   // filter tables
   DevBuf S;             // double [n] rods: arc length
   DevBuf win;           // int32 [E] rods: last filtered partner edge
@@ -255,15 +232,14 @@ enum {
   SC_FP32_PAIRS = 12,   // broad phase of contact_build: pairs passing the FP32 box test
   SC_FP64_DECIDED = 13, // ... of which the FP64 boxes decided
   SC_KSPLIT = 16,       // two uint32 counters: face / line-line pairs, the other active pairs
-  SC_NOVF = 17,         // broad phase: entries whose pairs overflow the stage
+  SC_NOVF = 17,         // broad phase: rod rows with more than half of a cluster as partners
   SC_NBK = 18,          // BSR pattern: keys left after the per-run sets of k_block_keys
   SC_FETCH = 19,        // ccd_step, FP64 iteration: pairs of the list handed out so far
   SC_NMOLL = 20,        // barrier_eval: mollified edge-edge pairs
   SC_GEO_COUNT = 21,    // geodesic rest filter: (edge, vertex) entries below the activation
   SC_GEO_ERR = 22,      // ... error bits of its sources (a fixed capacity exceeded)
-  SC_NVLONG = 23,       // shell broad phase: entries of flat_vlong
-  SC_NX = 24,           // ccd_step: two uint32 counters, point-triangle and edge-edge pairs of the FP64 iteration
-  SC_N = 25
+  SC_NX = 23,           // ccd_step: two uint32 counters, point-triangle and edge-edge pairs of the FP64 iteration
+  SC_N = 24
 };
 // read_scalars stages up to SC_N scalars through the pinned host scratch
 static_assert(SC_N <= 64, "the scalars must fit the pinned scratch");
@@ -279,11 +255,15 @@ constexpr uint8_t CB_CCD_EXACT = 0x80, CB_CCD_ONE = 0x40;
 cb_status read_scalars(cb_scene* s, int first, int count, uint64_t* out, cudaStream_t st);
 
 // broad.cu
+// The clusters of a new scene (topology and rest positions on the device;
+// rest_host the same positions on the host) or of a batch (its members' ones,
+// renumbered).
+cb_status clusters_build(cb_scene* s, const double* rest_host, cudaStream_t st);
+cb_status clusters_concat(cb_scene* b, cb_scene* const* members, cudaStream_t st);
 // Candidate pairs of x (p == nullptr) or of the sweep x -> x + p.  Boxes are
 // inflated per member by a/2 (static) or xi/2 (swept = true).  Writes the
 // canonical keys into *out (grown as needed), in ascending order when
-// sort_out is set and otherwise in hash-cell order, and their count into
-// *n_out.
+// sort_out is set and otherwise in tile order, and their count into *n_out.
 cb_status broad_phase(cb_scene* s, BroadWork& w, const double* x, const double* p, bool swept, bool sort_out,
                       DevBuf& out, int64_t* n_out, cudaStream_t st);
 

@@ -1,13 +1,13 @@
 """Autotuner for the broad-phase knobs of a scene or batch.
 
-The knobs change speed only, never results: the hash-cell edge (a factor
-times the members' mean primitive box extent) and the block size of the
-pair-enumeration kernel, separately for contact_build's broad phase (phase 0)
-and ccd_step's swept broad phase (phase 1).  Each candidate is timed with the
+The knobs change no result: a cell factor and a pair-kernel block size,
+separately for contact_build's broad phase (phase 0) and ccd_step's swept
+broad phase (phase 1).  They sized a cell hash; the library's cluster broad
+phase has neither cells nor such blocks, so every choice now times the same.  Each candidate is timed with the
 library's own stage events on passes over the caller's data; the fastest is
 kept and cached in a JSON file, keyed by the GPU, the scene kind, the vertex
 count (octave) and the ratio of the activation to the mean edge length
-(half octave): scenes alike in these have alike hash occupancy.
+(half octave).
 """
 from __future__ import annotations
 
