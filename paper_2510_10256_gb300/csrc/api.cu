@@ -7,6 +7,7 @@
 #include <numeric>
 #include <vector>
 
+#include "pairs.cuh"
 #include "scene.cuh"
 
 #include <atomic>
@@ -85,10 +86,10 @@ static cb_status upload(DevBuf& b, const T* h, size_t count, cudaStream_t st) {
 static void scene_release(cb_scene* s) {
   cudaStream_t st = s->last_stream;
   DevBuf* bufs[] = {&s->ev0, &s->ev1, &s->tv, &s->comp, &s->rest, &s->rod_ptr, &s->slots, &s->cinfo, &s->supers, &s->jobs, &s->S, &s->win, &s->wst,
-                    &s->rloop, &s->rlast, &s->elen2, &s->hmoll, &s->mlist, &s->ruv, &s->frest,
-                    &s->frest_dbar, &s->frest_j, &s->frow_pt, &s->frow_ee, &s->dbar_comp, &s->cand, &s->klass, &s->cand_alt, &s->klass_alt, &s->cd, &s->cflag, &s->cpos, &s->ctype, &s->ccls, &s->aidx,
-                    &s->bkey[0], &s->bkey[1], &s->bflag, &s->bpos, &s->bsr_row, &s->bsr_col, &s->bsr_val,
-                    &s->row_cnt, &s->hB9, &s->horder, &s->xf, &s->pf, &s->dlist, &s->mp, &s->vsc, &s->macc, &s->ccd_keys, &s->ccd_t, &s->ccd_cls, &s->ccd_list, &s->ccd_ulist, &s->scan_tmp, &s->hist,
+                    &s->rloop, &s->rlast, &s->elen2, &s->mlist, &s->ruv, &s->frest,
+                    &s->frest_dbar, &s->frest_j, &s->frow_pt, &s->frow_ee, &s->dbar_comp, &s->cand, &s->klass, &s->cand_alt, &s->klass_alt, &s->cd, &s->cflag, &s->cpos, &s->ctype, &s->ccls, &s->clist, &s->aidx,
+                    &s->bkey, &s->rcol, &s->bsr_row, &s->bsr_col, &s->bsr_val,
+                    &s->row_cnt, &s->hB9, &s->xf, &s->pf, &s->dlist, &s->mp, &s->vsc, &s->macc, &s->ccd_keys, &s->ccd_t, &s->ccd_cls, &s->ccd_list, &s->ccd_ulist, &s->scan_tmp,
                     &s->fr_key, &s->fr_st, &s->fr_dat, &s->fr_hw, &s->dev_scalars};
   for (DevBuf* b : bufs) buf_free(*b, st);
   for (BroadWork* w : {&s->bw, &s->bwc}) {
@@ -178,6 +179,19 @@ template <typename T>
 static cb_status dl(std::vector<T>& h, const DevBuf& b, int64_t count, cudaStream_t st) {
   h.resize((size_t)count);
   if (count) CB_CUDA(cudaMemcpyAsync(h.data(), b.p, sizeof(T) * (size_t)count, cudaMemcpyDeviceToHost, st));
+  return CB_OK;
+}
+
+// the active candidates (pairs.cuh, ActiveList): the list's two ends
+static cb_status dl_active(std::vector<uint32_t>& h, const cb_scene* s, cudaStream_t st) {
+  h.resize((size_t)s->n_active);
+  const int64_t n1 = s->n_active - s->n_plane;
+  const uint32_t* p = bp<uint32_t>(s->aidx);
+  if (s->n_active > 0 && s->n_plane > 0)
+    CB_CUDA(cudaMemcpyAsync(h.data(), p, sizeof(uint32_t) * (size_t)s->n_plane, cudaMemcpyDeviceToHost, st));
+  if (n1 > 0)
+    CB_CUDA(cudaMemcpyAsync(h.data() + s->n_plane, p + (s->act_cap - n1), sizeof(uint32_t) * (size_t)n1,
+                            cudaMemcpyDeviceToHost, st));
   return CB_OK;
 }
 
@@ -624,7 +638,8 @@ cb_status contact_build(cb_scene* s, const double* x, void* stream) {
   stage_begin(s, 0, st);
   cb_status r = broad_phase(s, s->bw, x, nullptr, false, false, s->cand, &s->n_cand, st);
   stage_end(s, 0, st);
-  s->n_active = 0;
+  s->n_active = s->n_plane = 0;
+  s->core_valid = false;
   return r;
 }
 
@@ -775,15 +790,18 @@ cb_status cb_get_pairs(cb_scene* s, int32_t which, uint64_t* keys, int64_t cap, 
         if (c[i] == 1) res.push_back(k[i]);
       break;
     case CB_PAIRS_CORE:
-      CB_TRY(dl(k, s->cand, s->n_cand, st));
-      CB_TRY(dl(c, s->ccls, s->n_cand, st));
-      CB_CUDA(cudaStreamSynchronize(st));
-      for (size_t i = 0; i < k.size(); ++i)
-        if (c[i] == 2) res.push_back(k[i]);
+      if (s->core_valid) {
+        uint64_t nc = 0;
+        CB_TRY(read_scalars(s, SC_NCORE, 1, &nc, st));
+        CB_TRY(dl(k, s->cand, s->n_cand, st));
+        CB_TRY(dl(ai, s->clist, (int64_t)(uint32_t)nc, st));
+        CB_CUDA(cudaStreamSynchronize(st));
+        for (uint32_t i : ai) res.push_back(k[i]);
+      }
       break;
     case CB_PAIRS_ACTIVE:
       CB_TRY(dl(k, s->cand, s->n_cand, st));
-      CB_TRY(dl(ai, s->aidx, s->n_active, st));
+      CB_TRY(dl_active(ai, s, st));
       CB_CUDA(cudaStreamSynchronize(st));
       for (uint32_t a : ai) res.push_back(k[a]);
       break;
@@ -828,7 +846,7 @@ cb_status cb_get_active(cb_scene* s, uint64_t* keys, double* dd, uint8_t* klass,
   std::vector<uint8_t> c;
   std::vector<int8_t> t;
   CB_TRY(dl(k, s->cand, s->n_cand, st));
-  CB_TRY(dl(ai, s->aidx, s->n_active, st));
+  CB_TRY(dl_active(ai, s, st));
   CB_TRY(dl(d, s->cd, s->n_cand, st));
   CB_TRY(dl(c, s->ccls, s->n_cand, st));
   CB_TRY(dl(t, s->ctype, s->n_cand, st));
@@ -841,7 +859,7 @@ cb_status cb_get_active(cb_scene* s, uint64_t* keys, double* dd, uint8_t* klass,
     const uint32_t src = ai[order[q]];
     if (keys) keys[q] = ak[q];
     if (dd) dd[q] = d[src];
-    if (klass) klass[q] = c[src];
+    if (klass) klass[q] = (uint8_t)(c[src] & ~CB_CLS_MOLLIFIED);
     if (dtype) dtype[q] = t[src];
   }
   return CB_OK;

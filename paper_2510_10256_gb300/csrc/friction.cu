@@ -83,7 +83,7 @@ __device__ void closest_weights(bool ee, int ty, const d3 (&R)[4], double (&b)[4
 
 struct FricLagArgs {
   int64_t na;
-  const uint32_t* __restrict__ aidx;
+  ActiveList act;
   const uint64_t* __restrict__ cand;
   const int8_t* __restrict__ ctype;
   const uint8_t* __restrict__ ccls;
@@ -106,12 +106,12 @@ struct FricLagArgs {
 __global__ void k_fric_lag(FricLagArgs A) {
   const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (a >= A.na) return;
-  const uint32_t c = A.aidx[a];
+  const uint32_t c = A.act.at(a);
   const uint64_t key = A.cand[c];
   const Stencil s = stencil_of(key, A.ev0, A.ev1, A.tv, A.T);
   const PassParams P = member_pass(A.mp[A.vsc[s.v[0]]]);
   double xi_p, dh_p;
-  pair_params(P, A.ccls[c], f_width(P, A.dbar_comp, A.comp, s.v[0]), xi_p, dh_p);
+  pair_params(P, A.ccls[c] & ~CB_CLS_MOLLIFIED, f_width(P, A.dbar_comp, A.comp, s.v[0]), xi_p, dh_p);
   double b, b1, b2;
   barrier_b012(A.cd[c] - xi_p, dh_p, b, b1, b2);
   const double lam = -P.kappa * b1;
@@ -252,7 +252,7 @@ extern "C" cb_status friction_lag(cb_scene* s, const double* x_lag, double mu, d
   CB_TRY(buf_ensure(s->fr_hw, sizeof(double) * 6 * (size_t)na, st));
   FricLagArgs A;
   A.na = na;
-  A.aidx = bp<uint32_t>(s->aidx);
+  A.act = active_list(s);
   A.cand = bp<uint64_t>(s->cand);
   A.ctype = bp<int8_t>(s->ctype);
   A.ccls = bp<uint8_t>(s->ccls);

@@ -293,7 +293,8 @@ __device__ __forceinline__ void warp_append_back(bool flag, uint32_t value, uint
 
 // Per candidate, phase 1: an FP32 lower bound of the distance.  Candidates it
 // places beyond every threshold of their class (U: a, which is above xi; F:
-// dbar_min) are inactive and not class C.  The rest are queued for the exact
+// dbar_min) are inactive and not class C, and nothing is written for them.
+// The rest are queued for the exact
 // FP64 phase, so that no warp pays for FP64 on behalf of a few lanes:
 // point-triangle pairs from the start of the list (count nlist[0]), edge-edge
 // pairs from its end backwards (count nlist[1]), so that the exact kernel's
@@ -303,9 +304,7 @@ __global__ void k_distance_screen(int64_t nc, const uint64_t* __restrict__ cand,
                                   const int32_t* __restrict__ ev1, const int32_t* __restrict__ tv, int T,
                                   const float4* __restrict__ xf, const double* __restrict__ cx,
                                   const int32_t* __restrict__ vsc, const MemberParams* __restrict__ mp, int n,
-                                  double* __restrict__ dout, int8_t* __restrict__ tout, uint8_t* __restrict__ cls,
-                                  uint32_t* __restrict__ flag, uint32_t* __restrict__ list,
-                                  unsigned int* __restrict__ nlist) {
+                                  uint32_t* __restrict__ list, unsigned int* __restrict__ nlist) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   bool exact = false, ee = false;
   if (c < nc) {
@@ -314,13 +313,7 @@ __global__ void k_distance_screen(int64_t nc, const uint64_t* __restrict__ cand,
     const int k = klass_in[c];
     const int mem = vsc[s.v[0]];
     const MemberParams& M = mp[mem];
-    if (k == 3) {  // culled (Kaldor mode): no barrier, no distance needed
-      dout[c] = __longlong_as_double(0x7ff0000000000000LL);
-      tout[c] = -1;
-      cls[c] = 3;
-      flag[c] = 0;
-      ee = false;
-    } else {
+    if (k != 3) {  // (3: culled in Kaldor mode, no barrier)
       // thresholds beyond which a pair is surely inactive and not class C (the
       // 1e-9 margins cover the rounding of the FP64 decision; FP32 copies
       // rounded up, so the FP32 comparison is as safe)
@@ -329,14 +322,7 @@ __global__ void k_distance_screen(int64_t nc, const uint64_t* __restrict__ cand,
       const float4 q0 = xf[s.v[0]], q1 = xf[s.v[1]], q2 = xf[s.v[2]], q3 = xf[s.v[3]];
       const float lb = cbb::lower_bound(s.ee, cbb::f3{q0.x, q0.y, q0.z}, cbb::f3{q1.x, q1.y, q1.z},
                                         cbb::f3{q2.x, q2.y, q2.z}, cbb::f3{q3.x, q3.y, q3.z}, X);
-      if (lb >= thr) {
-        dout[c] = __longlong_as_double(0x7ff0000000000000LL);
-        tout[c] = -1;
-        cls[c] = (uint8_t)k;
-        flag[c] = 0;
-      } else {
-        exact = true;
-      }
+      exact = !(lb >= thr);
     }
   }
   warp_append(exact && !ee, (uint32_t)c, list, &nlist[0]);
@@ -344,9 +330,15 @@ __global__ void k_distance_screen(int64_t nc, const uint64_t* __restrict__ cand,
 }
 
 // phase 2: exact FP64 distance, class C and activity of the queued candidates
-// (list entries [0, nlist[0]) and [cap - nlist[1], cap)).  With energy set
-// (the energy-only pass), every active pair also adds kappa b(y) to its
-// member's energy.
+// (list entries [0, nlist[0]) and [cap - nlist[1], cap)).  Class-C candidates
+// are listed in clist.  With ENERGY (the energy-only pass) every active pair
+// adds kappa b(y) to its member's energy; otherwise the active candidates are
+// listed in aidx: face / line-line pairs (the branch of k_pair_hess with the
+// most FP64 work) from the front, the others from the back, so that a warp of
+// that kernel runs one branch.  Appends are warp-aggregated, so the lists keep
+// the candidates' order but for the arrival of warps.  (Flags, a scan and a
+// compaction over all candidates made these lists before: 0.35 ms of a
+// pleated 256x256 pass, 14 bytes written per candidate.)
 template <bool ENERGY>
 __global__ void k_distance_exact(const uint32_t* __restrict__ list, int64_t cap, const unsigned int* __restrict__ nlist,
                                  const uint64_t* __restrict__ cand, const uint8_t* __restrict__ klass_in,
@@ -354,18 +346,21 @@ __global__ void k_distance_exact(const uint32_t* __restrict__ list, int64_t cap,
                                  const int32_t* __restrict__ tv, int T, const double* __restrict__ x, int n,
                                  const int32_t* __restrict__ vsc, const MemberParams* __restrict__ mp,
                                  double* __restrict__ dout, int8_t* __restrict__ tout,
-                                 uint8_t* __restrict__ cls, uint32_t* __restrict__ flag,
+                                 uint8_t* __restrict__ cls, uint32_t* __restrict__ clist, uint32_t* __restrict__ aidx,
+                                 unsigned* __restrict__ nsplit, uint32_t* __restrict__ mlist,
+                                 unsigned* __restrict__ nmoll,
                                  unsigned long long* __restrict__ status, unsigned long long* __restrict__ ncore,
                                  unsigned long long* __restrict__ macc, const int32_t* __restrict__ comp,
                                  const unsigned long long* __restrict__ dbar_comp, const double* __restrict__ elen2) {
   constexpr bool energy = ENERGY;  // energy only (barrier_energy): add kappa b per active pair
   const unsigned m0 = nlist[0], m = m0 + nlist[1];
   for (unsigned w = blockIdx.x * blockDim.x + threadIdx.x; w - threadIdx.x < m; w += gridDim.x * blockDim.x) {
-    uint32_t is_core = 0;
+    bool is_core = false, active = false, plane = false, moll = false;
+    uint32_t c = 0;
     double e_local = 0.0;
     int e_mem = -1;
     if (w < m) {
-      const uint32_t c = w < m0 ? list[w] : list[cap - 1 - (int64_t)(w - m0)];
+      c = w < m0 ? list[w] : list[cap - 1 - (int64_t)(w - m0)];
       Stencil s = stencil_of(cand[c], ev0, ev1, tv, T);
       int k = klass_in[c];
       const int mem = vsc[s.v[0]];
@@ -377,16 +372,25 @@ __global__ void k_distance_exact(const uint32_t* __restrict__ list, int64_t cap,
       double xi_p, dh_p;
       pair_params(P, k, f_width(P, dbar_comp, comp, s.v[0]), xi_p, dh_p);
       const double y = xsub(d, xi_p);
-      const uint32_t act = (y < dh_p) ? 1u : 0u;
+      const bool act = y < dh_p;
       if (act && y <= 0.0) {
         atomicOr(status, (unsigned long long)CB_DEV_PENETRATION);
         atomicOr(&macc[(size_t)mem * MACC_STRIDE + MACC_STATUS], (unsigned long long)CB_DEV_PENETRATION);
       }
-      dout[c] = d;
-      tout[c] = (int8_t)ty;
-      cls[c] = (uint8_t)k;
-      flag[c] = act;
       is_core = (k == 2);
+      if (!energy && act) {
+        active = true;
+        plane = ty == (s.ee ? 8 : 6);
+        // an edge-edge pair below its mollifier's threshold: its energy, gradient and 9x9 matrix come from
+        // k_moll_hess instead of k_pair_hess
+        if (P.mollify && s.ee) {
+          const double c2 = ee_cross2(load3(x, n, s.v[0]), load3(x, n, s.v[1]), load3(x, n, s.v[2]), load3(x, n, s.v[3]));
+          moll = c2 < 1e-3 * elen2[cb_key_i(cand[c])] * elen2[cb_key_j(cand[c])];
+        }
+        dout[c] = d;
+        tout[c] = (int8_t)ty;
+        cls[c] = (uint8_t)k | (moll ? CB_CLS_MOLLIFIED : 0);
+      }
       if (energy && act && y > 0.0) {
         double mf = 1.0;
         if (P.mollify && s.ee) {  // IPC's edge-edge mollifier
@@ -400,9 +404,14 @@ __global__ void k_distance_exact(const uint32_t* __restrict__ list, int64_t cap,
         e_mem = mem;
       }
     }
-    if (energy) member_energy_add(macc, e_mem, e_local);
-    const uint32_t b = __ballot_sync(0xffffffffu, is_core);
-    if ((threadIdx.x & 31) == 0 && b) atomicAdd(ncore, (unsigned long long)__popc(b));
+    warp_append(is_core, c, clist, (unsigned*)ncore);
+    if (energy) {
+      member_energy_add(macc, e_mem, e_local);
+    } else {
+      warp_append(active && plane, c, aidx, &nsplit[0]);
+      warp_append_back(active && !plane, c, aidx, cap, &nsplit[1]);
+      if (mlist) warp_append(moll, c, mlist, nmoll);
+    }
   }
 }
 
@@ -418,63 +427,100 @@ __global__ void k_to_f32(int n, const double* __restrict__ v, const double* __re
                        (float)(v[2 * (size_t)n + i] - (c ? c[2] : 0.0)), 0.f);
 }
 
-__global__ void k_active_compact(int64_t nc, const uint32_t* __restrict__ flag, const uint32_t* __restrict__ pos,
-                                 uint32_t* __restrict__ aidx) {
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c < nc && flag[c]) aidx[pos[c]] = (uint32_t)c;
-}
-
 // ------------------------------------------------------------------ (d) ----
 
-// 16 (row, col) block keys of each active stencil
-// BSR pattern keys (row << bits_n | col) of the 16 blocks of every active
-// stencil, made distinct within each run of BK_PAIRS active pairs (in
-// candidate order, i.e. tile by tile, a run shares most of its vertices:
-// its 16 x 256 keys hold about a fifth as many distinct ones) through an
-// open-addressing set in shared memory (linear probing, at most half full,
-// each probe sequence bounded by the table size).  The distinct keys of each
-// run are appended to bkey in no particular order -- the radix sort and the
-// unique pass that follow make the pattern -- and their count to *m_out.
+// The BSR pattern: the distinct (row, column) of the 16 blocks of every active
+// stencil, columns ascending in each row, without sorting the keys: each run of
+// BK_PAIRS active pairs makes its blocks distinct in shared memory
+// (k_block_keys), the survivors are bucketed by row (counts, scan, k_row_fill),
+// and each row's short bucket is sorted and made distinct by a warp
+// (k_row_unique; a block for buckets past ROW_MAX, k_row_unique_long).  On a
+// pleated 256x256 pass (862k active pairs, 1.7M blocks) the keys take 0.11 ms,
+// fill, unique and write 0.38; a set of 4,096 keys per run and a radix sort of
+// the survivors (five digits) with its flags and scans took 0.18 and 0.75 (the
+// whole barrier pass 2.79 -> 2.38 ms; 64 rod scenes 3.40 -> 3.06, a chain of
+// 2,000 loops 0.68 -> 0.54, a woven patch 0.28 -> 0.20).
+//
+// A run of active pairs (in candidate order, i.e. tile by tile) shares most of
+// its vertices, so its 4 x BK_PAIRS vertices become few local numbers through
+// an open-addressing set (linear probing, at most half full) and the blocks
+// bits of a local adjacency matrix.  A run with more than BK_VERTS vertices
+// appends all its blocks as they are: the rows' unique pass removes the rest.
 constexpr int BK_PAIRS = 256;
-constexpr int BK_SLOTS = 8192;  // 2 x 16 keys x BK_PAIRS
+constexpr int BK_SLOTS = 2048;  // 2 x 4 vertices x BK_PAIRS
+constexpr int BK_VERTS = 512;
+constexpr int BK_WORDS = BK_VERTS / 32;
+constexpr int BK_SMEM = (BK_SLOTS + BK_VERTS + BK_VERTS * BK_WORDS) * 4 + BK_SLOTS * 2;
 
-__global__ void __launch_bounds__(BK_PAIRS) k_block_keys(int64_t na, const uint32_t* __restrict__ aidx,
-                                                         const uint64_t* __restrict__ cand,
+__global__ void __launch_bounds__(BK_PAIRS) k_block_keys(ActiveList act, const uint64_t* __restrict__ cand,
                                                          const int32_t* __restrict__ ev0,
                                                          const int32_t* __restrict__ ev1,
-                                                         const int32_t* __restrict__ tv, int T, int bits_n,
-                                                         uint64_t* __restrict__ bkey, unsigned int* __restrict__ m_out) {
-  extern __shared__ unsigned long long tab[];  // BK_SLOTS
-  __shared__ unsigned int wsum[BK_PAIRS / 32];
-  __shared__ unsigned int base;
-  constexpr unsigned long long EMPTY = ~0ull;  // no key: rows and columns are below 2^31
+                                                         const int32_t* __restrict__ tv, int T,
+                                                         uint2* __restrict__ bkey, unsigned int* __restrict__ m_out,
+                                                         uint32_t* __restrict__ row_cnt) {
+  extern __shared__ int bk_smem[];
+  int* key = bk_smem;                               // [BK_SLOTS] vertex (-1: empty)
+  int* vert = key + BK_SLOTS;                       // [BK_VERTS] vertex of each local number
+  uint32_t* adj = (uint32_t*)(vert + BK_VERTS);     // [BK_VERTS][BK_WORDS]
+  uint16_t* loc = (uint16_t*)(adj + BK_VERTS * BK_WORDS);  // [BK_SLOTS] local number
+  __shared__ unsigned nv_s, wsum[BK_PAIRS / 32], base_s;
   const int tid = threadIdx.x;
-  for (int k = tid; k < BK_SLOTS; k += BK_PAIRS) tab[k] = EMPTY;
-  __syncthreads();
   const int64_t a = (int64_t)blockIdx.x * BK_PAIRS + tid;
-  if (a < na) {
-    const Stencil s = stencil_of(cand[aidx[a]], ev0, ev1, tv, T);
+  for (int k = tid; k < BK_SLOTS; k += BK_PAIRS) key[k] = -1;
+  if (tid == 0) nv_s = 0;
+  __syncthreads();
+  Stencil s;
+  int slot[4];
+  if (a < act.n) {
+    s = stencil_of(cand[act.at(a)], ev0, ev1, tv, T);
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const unsigned long long key = ((unsigned long long)s.v[i] << bits_n) | (unsigned long long)s.v[j];
-        // Fibonacci hashing (multiplicative, Knuth): the top bits of key x 2^64/phi
-        unsigned h = (unsigned)((key * 0x9E3779B97F4A7C15ull) >> 51);
-        for (int probe = 0; probe < BK_SLOTS; ++probe) {
-          const unsigned long long prev = atomicCAS(&tab[h], EMPTY, key);
-          if (prev == EMPTY || prev == key) break;
-          h = (h + 1) & (BK_SLOTS - 1);
-        }
+    for (int i = 0; i < 4; ++i) {
+      // Fibonacci hashing (multiplicative, Knuth): the top bits of v x 2^32/phi
+      unsigned h = ((unsigned)s.v[i] * 0x9E3779B1u) >> 21;
+      for (int probe = 0; probe < BK_SLOTS; ++probe) {
+        const int prev = atomicCAS(&key[h], -1, s.v[i]);
+        if (prev == -1 || prev == s.v[i]) break;
+        h = (h + 1) & (BK_SLOTS - 1);
       }
+      slot[i] = (int)h;
+    }
   }
   __syncthreads();
-  // compaction: thread tid owns slots [tid * 32, tid * 32 + 32)
-  constexpr int PER = BK_SLOTS / BK_PAIRS;
-  unsigned c = 0;
-#pragma unroll
-  for (int k = 0; k < PER; ++k) c += tab[tid * PER + k] != EMPTY;
+  for (int k = tid; k < BK_SLOTS; k += BK_PAIRS)
+    if (key[k] >= 0) {
+      const unsigned id = atomicAdd(&nv_s, 1u);
+      loc[k] = (uint16_t)id;
+      if (id < BK_VERTS) vert[id] = key[k];
+    }
+  __syncthreads();
+  const unsigned nv = nv_s;
   const unsigned lane = tid & 31, wid = tid >> 5;
+  const bool raw = nv > BK_VERTS;
+  const unsigned words = (nv + 31) / 32;
+  if (!raw) {
+    for (unsigned k = tid; k < nv * BK_WORDS; k += BK_PAIRS) adj[k] = 0u;
+    __syncthreads();
+    if (a < act.n) {
+      unsigned l[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) l[i] = loc[slot[i]];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) atomicOr(&adj[l[i] * BK_WORDS + (l[j] >> 5)], 1u << (l[j] & 31));
+    }
+    __syncthreads();
+  }
+  // this thread's blocks: local rows 2 tid and 2 tid + 1, or its stencil's 16
+  unsigned c = raw ? (a < act.n ? 16u : 0u) : 0u, cr[2] = {0u, 0u};
+  if (!raw)
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const unsigned r = 2 * tid + q;
+      if (r >= nv) continue;
+      for (unsigned w = 0; w < words; ++w) cr[q] += (unsigned)__popc(adj[r * BK_WORDS + w]);
+      c += cr[q];
+    }
   unsigned incl = c;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -489,29 +535,158 @@ __global__ void __launch_bounds__(BK_PAIRS) k_block_keys(int64_t na, const uint3
     woff += (w < (int)wid) ? wsum[w] : 0u;
     tot += wsum[w];
   }
-  if (tid == 0) base = tot ? atomicAdd(m_out, tot) : 0u;
+  if (tid == 0) base_s = tot ? atomicAdd(m_out, tot) : 0u;
   __syncthreads();
-  size_t pos = (size_t)base + woff + incl - c;
+  size_t pos = (size_t)base_s + woff + incl - c;
+  if (raw) {
+    if (a < act.n) {
 #pragma unroll
-  for (int k = 0; k < PER; ++k) {
-    const unsigned long long key = tab[tid * PER + k];
-    if (key != EMPTY) bkey[pos++] = key;
+      for (int i = 0; i < 4; ++i) {
+        atomicAdd(&row_cnt[s.v[i]], 4u);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) bkey[pos++] = make_uint2((uint32_t)s.v[i], (uint32_t)s.v[j]);
+      }
+    }
+    return;
+  }
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const unsigned r = 2 * tid + q;
+    if (r >= nv) continue;
+    const uint32_t row = (uint32_t)vert[r];
+    atomicAdd(&row_cnt[row], cr[q]);
+    for (unsigned w = 0; w < words; ++w)
+      for (uint32_t bits = adj[r * BK_WORDS + w]; bits; bits &= bits - 1u)
+        bkey[pos++] = make_uint2(row, (uint32_t)vert[32 * w + __ffs((int)bits) - 1]);
   }
 }
 
-__global__ void k_unique_flag(int64_t m, const uint64_t* __restrict__ k, uint32_t* __restrict__ flag) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < m) flag[i] = (i == 0 || k[i] != k[i - 1]) ? 1u : 0u;
+// the columns of the keys into their rows' buckets
+__global__ void k_row_fill(const uint2* __restrict__ bkey, const unsigned int* __restrict__ m_in,
+                           const uint32_t* __restrict__ off, uint32_t* __restrict__ cursor, uint32_t* __restrict__ rcol) {
+  const int64_t m = *m_in;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+    const uint2 k = bkey[i];
+    rcol[off[k.x] + atomicAdd(&cursor[k.x], 1u)] = k.y;
+  }
 }
 
-__global__ void k_unique_write(int64_t m, const uint64_t* __restrict__ k, const uint32_t* __restrict__ flag,
-                               const uint32_t* __restrict__ pos, int bits_n, int32_t* __restrict__ col,
-                               uint32_t* __restrict__ row_cnt) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m || !flag[i]) return;
-  const uint64_t key = k[i];
-  col[pos[i]] = (int32_t)(key & ((1ull << bits_n) - 1ull));
-  atomicAdd(&row_cnt[key >> bits_n], 1u);
+// Ascending bitonic sort of len values at p by `threads` threads of one warp or
+// block (sync() between steps): each merge starts by comparing mirrored pairs,
+// so every exchange puts the smaller value first and values past the end (as
+// if infinite) never move.
+template <typename Sync>
+__device__ __forceinline__ void sort_segment(uint32_t* p, unsigned len, unsigned tid, unsigned threads, Sync sync) {
+  unsigned size = 2;
+  for (;; size <<= 1) {
+    for (unsigned half = size >> 1, first = 1; half > 0; half >>= 1, first = 0) {
+      // pair t of this step: the t-th index whose bit `half` is clear, and its partner
+      const unsigned pairs = (len + 2 * half - 1) / (2 * half) * half;
+      for (unsigned t = tid; t < pairs; t += threads) {
+        const unsigned lo = (t / half) * 2 * half + (t & (half - 1));
+        const unsigned hi = first ? (lo ^ (size - 1)) : lo + half;
+        if (hi < len) {
+          const uint32_t x = p[lo], y = p[hi];
+          if (x > y) {
+            p[lo] = y;
+            p[hi] = x;
+          }
+        }
+      }
+      sync();
+    }
+    if (size >= len) break;
+  }
+}
+
+constexpr unsigned ROW_MAX = 512;  // bucket entries a warp sorts in shared memory
+constexpr int ROW_WARPS = 8;
+
+// a warp per row: its bucket sorted and made distinct in place, the count to
+// uniq; longer buckets are listed for k_row_unique_long
+__global__ void __launch_bounds__(32 * ROW_WARPS) k_row_unique(int n, const uint32_t* __restrict__ off,
+                                                               uint32_t* __restrict__ rcol, uint32_t* __restrict__ uniq,
+                                                               uint32_t* __restrict__ longs,
+                                                               unsigned int* __restrict__ nlong) {
+  __shared__ uint32_t buf[ROW_WARPS][ROW_MAX];
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int r = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  if (r >= n) return;
+  const uint32_t b = off[r], len = off[r + 1] - b;
+  if (len > ROW_MAX) {
+    if (lane == 0) longs[atomicAdd(nlong, 1u)] = (uint32_t)r;
+    return;
+  }
+  if (len <= 32) {
+    uint32_t v = lane < (int)len ? rcol[b + lane] : full;
+#pragma unroll
+    for (int size = 2; size <= 32; size <<= 1)
+#pragma unroll
+      for (int half = size >> 1; half > 0; half >>= 1) {
+        const int o = half == size >> 1 ? size - 1 : half;
+        const uint32_t u = __shfl_xor_sync(full, v, o);
+        v = (lane & half) ? max(u, v) : min(u, v);
+      }
+    const uint32_t before = __shfl_up_sync(full, v, 1);
+    const bool keep = lane < (int)len && (lane == 0 || v != before);
+    const unsigned m = __ballot_sync(full, keep);
+    if (keep) rcol[b + __popc(m & ((1u << lane) - 1u))] = v;
+    if (lane == 0) uniq[r] = (uint32_t)__popc(m);
+    return;
+  }
+  uint32_t* p = buf[threadIdx.x >> 5];
+  for (unsigned i = lane; i < len; i += 32) p[i] = rcol[b + i];
+  __syncwarp();
+  sort_segment(p, len, lane, 32, [] { __syncwarp(); });
+  unsigned at = 0;
+  for (unsigned i0 = 0; i0 < len; i0 += 32) {
+    const unsigned i = i0 + lane;
+    const bool keep = i < len && (i == 0 || p[i] != p[i - 1]);
+    const unsigned m = __ballot_sync(full, keep);
+    if (keep) rcol[b + at + __popc(m & ((1u << lane) - 1u))] = p[i];
+    at += (unsigned)__popc(m);
+  }
+  if (lane == 0) uniq[r] = at;
+}
+
+// ... a block per long bucket, in global memory
+__global__ void __launch_bounds__(cbp::SCAN_T) k_row_unique_long(const uint32_t* __restrict__ off, uint32_t* rcol,
+                                                                 uint32_t* __restrict__ uniq,
+                                                                 const uint32_t* __restrict__ longs,
+                                                                 const unsigned int* __restrict__ nlong) {
+  __shared__ unsigned tot;
+  __shared__ uint32_t last;
+  for (unsigned q = blockIdx.x; q < *nlong; q += gridDim.x) {
+    const uint32_t r = longs[q], b = off[r], len = off[r + 1] - b;
+    uint32_t* p = rcol + b;
+    sort_segment(p, len, threadIdx.x, blockDim.x, [] { __syncthreads(); });
+    unsigned at = 0;
+    for (unsigned i0 = 0; i0 < len; i0 += blockDim.x) {
+      const unsigned i = i0 + threadIdx.x;
+      const uint32_t v = i < len ? p[i] : 0u;
+      // the entry before the chunk may have been overwritten already: it is carried in `last`
+      const uint32_t u = i < len && threadIdx.x > 0 ? p[i - 1] : (i0 > 0 ? last : 0u);
+      const bool keep = i < len && (i == 0 || v != u);
+      const unsigned pos = cbp::block_excl_scan<unsigned>(keep ? 1u : 0u, &tot);
+      if (i < len && threadIdx.x == blockDim.x - 1) last = v;  // every read of this chunk is over
+      if (keep) p[at + pos] = v;
+      at += tot;
+      __syncthreads();
+    }
+    if (threadIdx.x == 0) uniq[r] = at;
+    __syncthreads();
+  }
+}
+
+// the rows' distinct columns to their place
+__global__ void k_row_write(int n, const uint32_t* __restrict__ off, const uint32_t* __restrict__ rcol,
+                            const int32_t* __restrict__ row_ptr, int32_t* __restrict__ col) {
+  const int r = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  if (r >= n) return;
+  const uint32_t b = off[r];
+  const int o = row_ptr[r], c = row_ptr[r + 1] - o;
+  for (int i = threadIdx.x & 31; i < c; i += 32) col[o + i] = (int32_t)rcol[b + i];
 }
 
 // Distance types as difference vectors z_m = sum_i C[m][i] x_i (m <= kind):
@@ -563,9 +738,7 @@ __device__ __forceinline__ int64_t find_block(const int32_t* __restrict__ row_pt
 }
 
 struct HessArgs {
-  int64_t na;
-  const uint32_t* __restrict__ order;  // thread -> active pair index
-  const uint32_t* __restrict__ aidx;
+  ActiveList act;
   const uint64_t* __restrict__ cand;
   const double* __restrict__ cd;
   const int8_t* __restrict__ ctype;
@@ -593,8 +766,7 @@ struct HessArgs {
   // ([e * cap + slot], slot = the pair's place in mlist)
   double* __restrict__ B9;
   int64_t cap;
-  // CB_EE_MOLLIFIER: pairs handled by k_moll_hess (hmoll null: none)
-  const uint8_t* __restrict__ hmoll;
+  // CB_EE_MOLLIFIER: candidates handled by k_moll_hess
   const uint32_t* __restrict__ mlist;
   const unsigned* __restrict__ nmoll;
   const double* __restrict__ elen2;
@@ -638,64 +810,6 @@ __device__ __forceinline__ void add_block(const HessArgs& A, int64_t bi, const d
     for (int j = 0; j < 3; ++j) atomicAdd(&dst[3 * i + j], tr ? blk[3 * j + i] : blk[3 * i + j]);
 }
 
-// Active pairs in the order k_pair_hess takes them: face / line-line pairs
-// (the branch with the most FP64 work) first, the other pairs from the end
-// backwards, so that a warp of that kernel runs one branch rather than
-// both with few lanes each.  Warp-aggregated appends; inside each group the
-// order follows warp arrival.
-struct MollArgs {                   // CB_EE_MOLLIFIER scenes only (mp null: no mollifier)
-  const double* __restrict__ x;
-  int n;
-  const int32_t* __restrict__ ev0;
-  const int32_t* __restrict__ ev1;
-  const int32_t* __restrict__ vsc;
-  const MemberParams* __restrict__ mp;
-  const double* __restrict__ elen2;
-  uint8_t* __restrict__ hmoll;       // [na] 1: mollified edge-edge pair
-  uint32_t* __restrict__ mlist;      // their active indices
-  unsigned* __restrict__ nmoll;
-};
-
-__global__ void k_kind_split(int64_t na, const uint32_t* __restrict__ aidx, const uint64_t* __restrict__ cand,
-                             const int8_t* __restrict__ ctype, uint32_t* __restrict__ order,
-                             unsigned* __restrict__ cnt, MollArgs MA) {
-  const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  bool plane = false, moll = false;
-  if (a < na) {
-    const uint32_t c = aidx[a];
-    const int ty = ctype[c];
-    const uint64_t key = cand[c];
-    plane = (cb_key_type(key) == CB_KEY_PT ? c_pt_types[ty] : c_ee_types[ty]).kind == 2;
-    if (MA.mp && cb_key_type(key) != CB_KEY_PT) {
-      // edge-edge pair below its mollifier threshold: its energy, gradient
-      // and 9x9 matrix come from k_moll_hess instead of k_pair_hess
-      const uint32_t i = cb_key_i(key), j = cb_key_j(key);
-      const int a0 = MA.ev0[i], a1 = MA.ev1[i], b0 = MA.ev0[j], b1 = MA.ev1[j];
-      if (MA.mp[MA.vsc[a0]].mollify) {
-        const double c2 = ee_cross2(load3(MA.x, MA.n, a0), load3(MA.x, MA.n, a1), load3(MA.x, MA.n, b0),
-                                    load3(MA.x, MA.n, b1));
-        moll = c2 < 1e-3 * MA.elen2[i] * MA.elen2[j];
-      }
-    }
-    if (MA.mp) MA.hmoll[a] = moll ? 1 : 0;
-  }
-  if (MA.mp) warp_append(moll, (uint32_t)a, MA.mlist, MA.nmoll);
-  const unsigned lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
-  const unsigned mp = __ballot_sync(0xffffffffu, a < na && plane);
-  const unsigned mr = __ballot_sync(0xffffffffu, a < na && !plane);
-  unsigned bp = 0, br = 0;
-  if (lane == 0) {
-    if (mp) bp = atomicAdd(&cnt[0], (unsigned)__popc(mp));
-    if (mr) br = atomicAdd(&cnt[1], (unsigned)__popc(mr));
-  }
-  bp = __shfl_sync(0xffffffffu, bp, 0);
-  br = __shfl_sync(0xffffffffu, br, 0);
-  if (a < na) {
-    if (plane) order[bp + __popc(mp & lt)] = (uint32_t)a;
-    else order[na - 1 - (int64_t)(br + __popc(mr & lt))] = (uint32_t)a;
-  }
-}
-
 // Stage (d), one thread per active pair: barrier value and derivatives,
 // energy, gradient scatter, the PSD-projected Hessian in closed form
 // (pairhess.cuh) and its scatter into the BSR values.  PAIR_T threads a block:
@@ -711,12 +825,11 @@ __device__ __forceinline__ int pick(const int (&v)[4], int i) {
 
 __global__ void __launch_bounds__(PAIR_T) k_pair_hess(HessArgs A) {
   const int64_t t = (int64_t)blockIdx.x * PAIR_T + threadIdx.x;
-  int64_t a = t < A.na ? (int64_t)A.order[t] : A.na;
-  if (A.hmoll && a < A.na && A.hmoll[a]) a = A.na;  // mollified edge-edge pair: k_moll_hess
+  const uint32_t c = t < A.act.n ? A.act.at(t) : 0u;
+  const uint8_t cls = t < A.act.n ? A.ccls[c] : CB_CLS_MOLLIFIED;
   double e_local = 0.0;
   int mem = -1, counted = 0;  // 9, 6, 4: the statistics' kinds
-  if (a < A.na) {
-    const uint32_t c = A.aidx[a];
+  if (!(cls & CB_CLS_MOLLIFIED)) {  // (mollified: k_moll_hess)
     const Stencil s = stencil_of(A.cand[c], A.ev0, A.ev1, A.tv, A.T);
     const int ty = A.ctype[c];
     const TypeInfo& TI = s.ee ? c_ee_types[ty] : c_pt_types[ty];
@@ -728,7 +841,7 @@ __global__ void __launch_bounds__(PAIR_T) k_pair_hess(HessArgs A) {
     mem = A.vsc[s.v[0]];
     const PassParams P = member_pass(A.mp[mem]);
     double xi_p, dh_p;
-    pair_params(P, A.ccls[c], f_width(P, A.dbar_comp, A.comp, s.v[0]), xi_p, dh_p);
+    pair_params(P, cls, f_width(P, A.dbar_comp, A.comp, s.v[0]), xi_p, dh_p);
     const double y = d - xi_p;
     double b, b1, b2;
     barrier_b012(y, dh_p, b, b1, b2);
@@ -1065,21 +1178,20 @@ __device__ void ee_distance_derivs(int ty, const d3 (&X)[4], double d, LocalDeri
                         0.75 * g * r5 * Nd.g[i] * Nd.g[j]);
 }
 
-// one thread per mollified pair (listed by k_kind_split)
+// one thread per mollified pair (listed by k_distance_exact)
 __global__ void __launch_bounds__(128) k_moll_hess(HessArgs A) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   double e_local = 0.0;
   int mem = -1;
   if (t < (int64_t)*A.nmoll) {
-    const uint32_t a = A.mlist[t];
-    const uint32_t c = A.aidx[a];
+    const uint32_t c = A.mlist[t];
     const uint64_t key = A.cand[c];
     const Stencil s = stencil_of(key, A.ev0, A.ev1, A.tv, A.T);
     const int ty = A.ctype[c];
     mem = A.vsc[s.v[0]];
     const PassParams P = member_pass(A.mp[mem]);
     double xi_p, dh_p;
-    pair_params(P, A.ccls[c], f_width(P, A.dbar_comp, A.comp, s.v[0]), xi_p, dh_p);
+    pair_params(P, A.ccls[c] & ~CB_CLS_MOLLIFIED, f_width(P, A.dbar_comp, A.comp, s.v[0]), xi_p, dh_p);
     const double d = A.cd[c];
     double b, b1, b2;
     barrier_b012(d - xi_p, dh_p, b, b1, b2);
@@ -1405,7 +1517,7 @@ __global__ void __launch_bounds__(S) k_hess_proj(HessArgs A) {
     float* V32 = (float*)smem + tid;                    // FP32 V, same indexing, inside the V region
     float* A32 = (float*)(smem + D * D * S) + tid;      // FP32 A, same indexing, inside the A region
     const bool act = w < m;                             // no early exit before the last barrier
-    const uint32_t a = act ? A.mlist[w] : 0u;
+    const uint32_t c = act ? A.mlist[w] : 0u;
     // B stays in registers until B+ is formed
     double Br[NP];
     double mx = 0.0;
@@ -1520,7 +1632,6 @@ __global__ void __launch_bounds__(S) k_hess_proj(HessArgs A) {
         for (int jj = i; jj < D; ++jj) Bs[tri_idx(i, jj, D) * S] += wi * v[jj];
       }
     }
-    const uint32_t c = A.aidx[a];
     const Stencil st = stencil_of(A.cand[c], A.ev0, A.ev1, A.tv, A.T);
     hadamard_scatter(A, st, Bs, S);
   }
@@ -1644,7 +1755,7 @@ __global__ void __launch_bounds__(PL_THREADS) k_hess_proj_lanes(HessArgs A) {
   float* A32 = (float*)(Vs + 81);
   float* X32 = A32 + 81;
   float* V32 = X32 + 81;
-  const uint32_t a = A.mlist[w];
+  const uint32_t ci = A.mlist[w];
   double Br[9];  // row r of B
   double mx = 0.0;
 #pragma unroll
@@ -1774,7 +1885,6 @@ __global__ void __launch_bounds__(PL_THREADS) k_hess_proj_lanes(HessArgs A) {
   // over the row points, and the sixteen blocks' entries of that row
   if (lane < 12) {
     const int q1 = lane / 3, i = lane % 3;
-    const uint32_t ci = A.aidx[a];
     const Stencil st = stencil_of(A.cand[ci], A.ev0, A.ev1, A.tv, A.T);
     const int rv = st.v[q1];
 #pragma unroll
@@ -2031,12 +2141,6 @@ cb_status to_f32(cb_scene* s, const double* v, const double* cx, DevBuf& out, cu
   return CB_OK;
 }
 
-static int bits_for(int64_t v) {
-  int b = 1;
-  while ((1ll << b) <= v) ++b;
-  return b;
-}
-
 cb_status barrier_run(cb_scene* s, const double* x, double* energy, double* grad, bool energy_only,
                       cudaStream_t st) {
   const int64_t nc = s->n_cand;
@@ -2045,16 +2149,19 @@ cb_status barrier_run(cb_scene* s, const double* x, double* energy, double* grad
   unsigned long long* ncore = (unsigned long long*)(sc + SC_NCORE);
   unsigned long long* macc = bp<unsigned long long>(s->macc);
   const int M = s->count;
+  bool mollify = false;
+  for (const MemberParams& m : s->hmp) mollify |= m.mollify != 0;
   s->cd_split = false;
+  s->core_valid = true;
   // the pass's counters (the queue lengths stay readable until the next pass)
   {
     const uint32_t scm = (1u << SC_NCORE) | (1u << SC_NLIST) | (1u << SC_KSPLIT) | (1u << SC_NMOLL) |
-                         (1u << SC_N9) | (1u << SC_N6) | (1u << SC_N4);
+                         (1u << SC_N9) | (1u << SC_N6) | (1u << SC_N4) | (1u << SC_NBK) | (1u << SC_NLONG);
     k_pass_reset<<<cb_grid(std::max(M, (int)SC_N)), CB_THREADS, 0, cb_count(st)>>>(
         (unsigned long long*)sc, scm, M, macc, (1u << MACC_E) | (1u << MACC_STATUS));
   }
   if (grad) CB_CUDA(cudaMemsetAsync(grad, 0, sizeof(double) * 3 * (size_t)s->n, st));
-  s->n_active = 0;
+  s->n_active = s->n_plane = 0;
   s->nnzb = 0;
   CB_TRY(buf_ensure(s->bsr_row, sizeof(int32_t) * ((size_t)s->n + 1), st));
   CB_CUDA(cudaMemsetAsync(s->bsr_row.p, 0, sizeof(int32_t) * ((size_t)s->n + 1), st));
@@ -2062,105 +2169,79 @@ cb_status barrier_run(cb_scene* s, const double* x, double* energy, double* grad
     CB_TRY(buf_ensure(s->cd, sizeof(double) * (size_t)nc, st));
     CB_TRY(buf_ensure(s->ctype, (size_t)nc, st));
     CB_TRY(buf_ensure(s->ccls, (size_t)nc, st));
-    CB_TRY(buf_ensure(s->cflag, sizeof(uint32_t) * (size_t)nc, st));
-    CB_TRY(buf_ensure(s->cpos, sizeof(uint32_t) * ((size_t)nc + 1), st));
-    CB_TRY(buf_ensure(s->scan_tmp, sizeof(uint64_t) * (size_t)(cbp::scan_tmp_elems(nc) + 8), st));
+    CB_TRY(buf_ensure(s->clist, sizeof(uint32_t) * (size_t)nc, st));
+    CB_TRY(buf_ensure(s->aidx, sizeof(uint32_t) * (size_t)nc, st));
+    if (mollify) CB_TRY(buf_ensure(s->mlist, sizeof(uint32_t) * (size_t)nc, st));
     CB_TRY(to_f32(s, x, bp<double>(s->bw.cx), s->xf, st));
     CB_TRY(buf_ensure(s->dlist, sizeof(uint32_t) * (size_t)nc, st));
     unsigned int* nl = (unsigned int*)(sc + SC_NLIST);
     k_distance_screen<<<cb_grid(nc), CB_THREADS, 0, cb_count(st)>>>(
         nc, bp<uint64_t>(s->cand), bp<uint8_t>(s->klass), bp<int32_t>(s->ev0), bp<int32_t>(s->ev1),
         bp<int32_t>(s->tv), s->T, bp<float4>(s->xf), bp<double>(s->bw.cx), bp<int32_t>(s->vsc),
-        bp<MemberParams>(s->mp), s->n, bp<double>(s->cd),
-        bp<int8_t>(s->ctype), bp<uint8_t>(s->ccls), bp<uint32_t>(s->cflag), bp<uint32_t>(s->dlist), nl);
+        bp<MemberParams>(s->mp), s->n, bp<uint32_t>(s->dlist), nl);
     (energy_only ? k_distance_exact<true> : k_distance_exact<false>)<<<std::min<int64_t>(cb_grid(nc), (int64_t)s->n_sms * 16), CB_THREADS, 0, cb_count(st)>>>(
         bp<uint32_t>(s->dlist), nc, nl, bp<uint64_t>(s->cand), bp<uint8_t>(s->klass), bp<int32_t>(s->ev0),
         bp<int32_t>(s->ev1), bp<int32_t>(s->tv), s->T, x, s->n, bp<int32_t>(s->vsc), bp<MemberParams>(s->mp),
-        bp<double>(s->cd), bp<int8_t>(s->ctype), bp<uint8_t>(s->ccls), bp<uint32_t>(s->cflag), status, ncore,
+        bp<double>(s->cd), bp<int8_t>(s->ctype), bp<uint8_t>(s->ccls), bp<uint32_t>(s->clist), bp<uint32_t>(s->aidx),
+        (unsigned*)(sc + SC_KSPLIT), mollify ? bp<uint32_t>(s->mlist) : nullptr, (unsigned*)(sc + SC_NMOLL), status, ncore,
         macc, bp<int32_t>(s->comp), bp<unsigned long long>(s->dbar_comp), bp<double>(s->elen2));
     if (energy_only) {
       if (energy) k_energy_final<<<cb_grid(M), CB_THREADS, 0, cb_count(st)>>>(M, macc, energy);
       CB_CUDA(cudaGetLastError());
       return CB_OK;
     }
-    uint32_t* tot = (uint32_t*)(sc + SC_COUNT1);
-    cbp::exclusive_scan<uint32_t, uint32_t>(bp<uint32_t>(s->cflag), bp<uint32_t>(s->cpos), nc,
-                                            bp<uint32_t>(s->scan_tmp), tot, st);
     CB_CUDA(cudaGetLastError());
     uint64_t h;
-    CB_TRY(read_scalars(s, SC_COUNT1, 1, &h, st));
-    s->n_active = (int64_t)(uint32_t)h;
+    CB_TRY(read_scalars(s, SC_KSPLIT, 1, &h, st));
+    s->n_plane = (int64_t)(uint32_t)h;
+    s->n_active = s->n_plane + (int64_t)(h >> 32);
+    s->act_cap = nc;
     // end of stage (c): distances, classes and the active set
     if (s->timing) cudaEventRecord(s->ev[12], st);
     s->cd_split = true;
   }
   const int64_t na = s->n_active;
   if (na > 0) {
-    CB_TRY(buf_ensure(s->aidx, sizeof(uint32_t) * (size_t)na, st));
-    k_active_compact<<<cb_grid(nc), CB_THREADS, 0, cb_count(st)>>>(nc, bp<uint32_t>(s->cflag), bp<uint32_t>(s->cpos),
-                                                         bp<uint32_t>(s->aidx));
-    // BSR pattern: sorted unique (row, col) of the 16 blocks of every active stencil
-    int64_t m = 16 * na;  // capacity; the keys actually sorted are counted by k_block_keys
-    const int bn = bits_for(s->n);
-    for (int b = 0; b < 2; ++b) CB_TRY(buf_ensure(s->bkey[b], sizeof(uint64_t) * (size_t)m, st));
-    CB_TRY(buf_ensure(s->bflag, sizeof(uint32_t) * (size_t)m, st));
-    CB_TRY(buf_ensure(s->bpos, sizeof(uint32_t) * ((size_t)m + 1), st));
-    CB_TRY(buf_ensure(s->hist, sizeof(uint32_t) * (size_t)cbp::radix_hist_elems(m), st));
-    CB_TRY(buf_ensure(s->scan_tmp, sizeof(uint64_t) * (size_t)(cbp::scan_tmp_elems(cbp::radix_hist_elems(m)) +
-                                                                cbp::scan_tmp_elems(m) + 8),
-                      st));
+    const ActiveList act = active_list(s);
+    // BSR pattern: distinct (row, col) of the 16 blocks of every active stencil
+    const int n = s->n;
+    const size_t m = 16 * (size_t)na;  // capacity; the keys are counted by k_block_keys
+    CB_TRY(buf_ensure(s->bkey, sizeof(uint2) * m, st));
+    CB_TRY(buf_ensure(s->rcol, sizeof(uint32_t) * m, st));
+    // row counts, fill cursors, distinct counts (cleared together), bucket offsets, long buckets
+    CB_TRY(buf_ensure(s->row_cnt, sizeof(uint32_t) * 5 * ((size_t)n + 1), st));
+    CB_TRY(buf_ensure(s->scan_tmp, sizeof(uint64_t) * (size_t)(cbp::scan_tmp_elems(n + 1) + 8), st));
+    uint32_t* cnt = bp<uint32_t>(s->row_cnt);
+    uint32_t *cursor = cnt + (n + 1), *uniq = cursor + (n + 1), *off = uniq + (n + 1), *longs = off + (n + 1);
+    CB_CUDA(cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * 3 * ((size_t)n + 1), st));
     unsigned int* nbk = (unsigned int*)(sc + SC_NBK);
-    CB_CUDA(cudaMemsetAsync(nbk, 0, sizeof(unsigned int), st));
-    {
-      const int smem = BK_SLOTS * (int)sizeof(unsigned long long);
-      CB_CUDA(cudaFuncSetAttribute(k_block_keys, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-      k_block_keys<<<(int)((na + BK_PAIRS - 1) / BK_PAIRS), BK_PAIRS, smem, cb_count(st)>>>(
-          na, bp<uint32_t>(s->aidx), bp<uint64_t>(s->cand), bp<int32_t>(s->ev0), bp<int32_t>(s->ev1),
-          bp<int32_t>(s->tv), s->T, bn, bp<uint64_t>(s->bkey[0]), nbk);
-      CB_CUDA(cudaGetLastError());
-    }
-    uint64_t hm;
-    CB_TRY(read_scalars(s, SC_NBK, 1, &hm, st));
-    m = (int64_t)(uint32_t)hm;  // keys left after the per-run sets (at most 16 na)
-    int r = cbp::radix_sort<uint64_t, uint32_t, false>(bp<uint64_t>(s->bkey[0]), nullptr, bp<uint64_t>(s->bkey[1]),
-                                                       nullptr, m, 0, 2 * bn, bp<uint32_t>(s->hist),
-                                                       bp<uint32_t>(s->scan_tmp), st);
-    const uint64_t* bk = bp<uint64_t>(s->bkey[r]);
-    k_unique_flag<<<cb_grid(m), CB_THREADS, 0, cb_count(st)>>>(m, bk, bp<uint32_t>(s->bflag));
+    unsigned int* nlong = (unsigned int*)(sc + SC_NLONG);
+    CB_CUDA(cudaFuncSetAttribute(k_block_keys, cudaFuncAttributeMaxDynamicSharedMemorySize, BK_SMEM));
+    k_block_keys<<<(int)((na + BK_PAIRS - 1) / BK_PAIRS), BK_PAIRS, BK_SMEM, cb_count(st)>>>(
+        act, bp<uint64_t>(s->cand), bp<int32_t>(s->ev0), bp<int32_t>(s->ev1), bp<int32_t>(s->tv), s->T,
+        bp<uint2>(s->bkey), nbk, cnt);
+    cbp::exclusive_scan<uint32_t, uint32_t>(cnt, off, (int64_t)n + 1, bp<uint32_t>(s->scan_tmp), (uint32_t*)nullptr, st);
+    k_row_fill<<<(int)std::min<int64_t>(cb_grid((int64_t)m), (int64_t)s->n_sms * 16), CB_THREADS, 0, cb_count(st)>>>(
+        bp<uint2>(s->bkey), nbk, off, cursor, bp<uint32_t>(s->rcol));
+    k_row_unique<<<cb_grid((int64_t)n * 32, 32 * ROW_WARPS), 32 * ROW_WARPS, 0, cb_count(st)>>>(
+        n, off, bp<uint32_t>(s->rcol), uniq, longs, nlong);
+    k_row_unique_long<<<s->n_sms, cbp::SCAN_T, 0, cb_count(st)>>>(off, bp<uint32_t>(s->rcol), uniq, longs, nlong);
+    // uniq[n] = 0: the scan's last entry is the block count
     uint32_t* tot = (uint32_t*)(sc + SC_COUNT1);
-    cbp::exclusive_scan<uint32_t, uint32_t>(bp<uint32_t>(s->bflag), bp<uint32_t>(s->bpos), m,
-                                            bp<uint32_t>(s->scan_tmp), tot, st);
+    cbp::exclusive_scan<uint32_t, int32_t>(uniq, bp<int32_t>(s->bsr_row), (int64_t)n + 1,
+                                           (int32_t*)bp<uint32_t>(s->scan_tmp), (int32_t*)tot, st);
     CB_CUDA(cudaGetLastError());
     uint64_t h;
     CB_TRY(read_scalars(s, SC_COUNT1, 1, &h, st));
     s->nnzb = (int64_t)(uint32_t)h;
     CB_TRY(buf_ensure(s->bsr_col, sizeof(int32_t) * (size_t)s->nnzb, st));
     CB_TRY(buf_ensure(s->bsr_val, sizeof(double) * 9 * (size_t)s->nnzb, st));
-    CB_TRY(buf_ensure(s->row_cnt, sizeof(uint32_t) * ((size_t)s->n + 1), st));
-    CB_CUDA(cudaMemsetAsync(s->row_cnt.p, 0, sizeof(uint32_t) * ((size_t)s->n + 1), st));
     CB_CUDA(cudaMemsetAsync(s->bsr_val.p, 0, sizeof(double) * 9 * (size_t)s->nnzb, st));
-    k_unique_write<<<cb_grid(m), CB_THREADS, 0, cb_count(st)>>>(m, bk, bp<uint32_t>(s->bflag), bp<uint32_t>(s->bpos), bn,
-                                                      bp<int32_t>(s->bsr_col), bp<uint32_t>(s->row_cnt));
-    cbp::exclusive_scan<uint32_t, int32_t>(bp<uint32_t>(s->row_cnt), bp<int32_t>(s->bsr_row), (int64_t)s->n + 1,
-                                           (int32_t*)bp<uint32_t>(s->scan_tmp), (int32_t*)nullptr, st);
-    CB_TRY(buf_ensure(s->horder, sizeof(uint32_t) * (size_t)na, st));
-    bool mollify = false;
-    for (const MemberParams& mpm : s->hmp) mollify |= mpm.mollify != 0;
-    MollArgs MA{};
-    if (mollify) {
-      CB_TRY(buf_ensure(s->hmoll, (size_t)na, st));
-      CB_TRY(buf_ensure(s->mlist, sizeof(uint32_t) * (size_t)na, st));
-      MA = MollArgs{x, s->n, bp<int32_t>(s->ev0), bp<int32_t>(s->ev1), bp<int32_t>(s->vsc),
-                    bp<MemberParams>(s->mp), bp<double>(s->elen2), bp<uint8_t>(s->hmoll),
-                    bp<uint32_t>(s->mlist), (unsigned*)(sc + SC_NMOLL)};
-    }
-    k_kind_split<<<cb_grid(na), CB_THREADS, 0, cb_count(st)>>>(na, bp<uint32_t>(s->aidx), bp<uint64_t>(s->cand),
-                                                             bp<int8_t>(s->ctype), bp<uint32_t>(s->horder),
-                                                             (unsigned*)(sc + SC_KSPLIT), MA);
+    k_row_write<<<cb_grid((int64_t)n * 32), CB_THREADS, 0, cb_count(st)>>>(n, off, bp<uint32_t>(s->rcol),
+                                                                          bp<int32_t>(s->bsr_row),
+                                                                          bp<int32_t>(s->bsr_col));
     HessArgs A;
-    A.na = na;
-    A.order = bp<uint32_t>(s->horder);
-    A.aidx = bp<uint32_t>(s->aidx);
+    A.act = act;
     A.cand = bp<uint64_t>(s->cand);
     A.cd = bp<double>(s->cd);
     A.ctype = bp<int8_t>(s->ctype);
@@ -2187,7 +2268,6 @@ cb_status barrier_run(cb_scene* s, const double* x, double* energy, double* grad
     A.n6 = (unsigned int*)(sc + SC_N6);
     A.n4 = (unsigned int*)(sc + SC_N4);
     A.cap = na;
-    A.hmoll = mollify ? bp<uint8_t>(s->hmoll) : nullptr;
     A.mlist = bp<uint32_t>(s->mlist);
     A.nmoll = (const unsigned*)(sc + SC_NMOLL);
     A.elen2 = bp<double>(s->elen2);

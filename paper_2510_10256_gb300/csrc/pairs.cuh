@@ -37,6 +37,21 @@ __device__ __forceinline__ d3 load3(const double* __restrict__ x, int n, int v) 
   return mk3(x[v], x[(size_t)n + v], x[2 * (size_t)n + v]);
 }
 
+// class byte flag of an active candidate: a mollified edge-edge pair
+constexpr uint8_t CB_CLS_MOLLIFIED = 0x40;
+
+// The active candidates of the last barrier pass, two-ended: n0 face /
+// line-line pairs from the front of idx, the others from the back of its cap
+// entries.
+struct ActiveList {
+  int64_t n, n0, cap;
+  const uint32_t* __restrict__ idx;
+  __device__ __forceinline__ uint32_t at(int64_t a) const { return a < n0 ? idx[a] : idx[cap - 1 - (a - n0)]; }
+};
+inline ActiveList active_list(const cb_scene* s) {
+  return ActiveList{s->n_active, s->n_plane, s->act_cap, (const uint32_t*)s->aidx.p};
+}
+
 struct PassParams {
   double xi, dhat, a, dbar_min, kappa;
   int single, core_temp, per_comp, mollify;

@@ -162,22 +162,23 @@ struct cb_scene {
     return false;
   }
   DevBuf cd;            // double [nc] distance
-  DevBuf cflag;         // uint32 [nc] active flag
-  DevBuf cpos;          // uint32 [nc+1] scan of flags
+  DevBuf cflag, cpos;   // per-stencil activation: uint32 keep flags of the candidates and their scan
+  // ... of the active candidates only: distance (cd), type and final class (with C; | CB_CLS_MOLLIFIED)
   DevBuf ctype;         // int8 [nc]
-  DevBuf ccls;          // uint8 [nc] final class (with C)
+  DevBuf ccls;          // uint8 [nc]
+  DevBuf clist;         // uint32 [nc] candidates of class C, SC_NCORE of them
+  bool core_valid = false;  // clist belongs to the current candidates
   int64_t n_active = 0;
-  DevBuf aidx;          // uint32 [na] candidate index of each active pair
-  DevBuf bkey[2];       // uint64 [16 na]
-  DevBuf bflag, bpos;   // uint32
+  DevBuf aidx;          // uint32 [nc] active candidates, two-ended (pairs.cuh, ActiveList)
+  int64_t n_plane = 0, act_cap = 0;
+  DevBuf bkey;          // uint2 [16 na] (row, column) of the active stencils' blocks, distinct within a run
+  DevBuf rcol;          // uint32 [16 na] their columns, bucketed by row
   DevBuf bsr_row;       // int32 [n+1]
   DevBuf bsr_col;       // int32 [nnzb]
   DevBuf bsr_val;       // double [nnzb][9]
-  DevBuf row_cnt;       // uint32 [n+1]
+  DevBuf row_cnt;       // uint32 [5][n+1]: keys, fill cursor, distinct columns and bucket offset of each row; long rows
   int64_t nnzb = 0;
-  DevBuf horder;        // uint32 active pair indices in prep order (face / line-line pairs first)
-  DevBuf hmoll;         // uint8 [na] mollified edge-edge pair (CB_EE_MOLLIFIER), handled by k_moll_hess
-  DevBuf mlist;         // uint32 active indices of the mollified pairs
+  DevBuf mlist;         // uint32 [nc] active candidates with a mollifier below 1 (CB_EE_MOLLIFIER)
   DevBuf hB9;           // CB_EE_MOLLIFIER: queued reduced Hessians (packed, element-major)
   DevBuf xf, pf;         // float [3][n]: centred FP32 copies of x and of p
   DevBuf dlist;          // uint32: candidates / CCD pairs queued for the FP64 phase
@@ -196,7 +197,6 @@ struct cb_scene {
   double fr_mu = 0.0, fr_eps = 0.0;
   bool fr_lagged = false, fr_hw_valid = false;
   DevBuf scan_tmp;
-  DevBuf hist;
   DevBuf dev_scalars;   // misc device scalars (counters, energy, alpha bits, status)
 
   uint64_t* h_pinned = nullptr;  // pinned host scratch (64 slots)
@@ -233,13 +233,14 @@ enum {
   SC_FP64_DECIDED = 13, // ... of which the FP64 boxes decided
   SC_KSPLIT = 16,       // two uint32 counters: face / line-line pairs, the other active pairs
   SC_NOVF = 17,         // broad phase: rod rows with more than half of a cluster as partners
-  SC_NBK = 18,          // BSR pattern: keys left after the per-run sets of k_block_keys
+  SC_NBK = 18,          // BSR pattern: keys left by the runs of k_block_keys
   SC_FETCH = 19,        // ccd_step, FP64 iteration: pairs of the list handed out so far
   SC_NMOLL = 20,        // barrier_eval: mollified edge-edge pairs
   SC_GEO_COUNT = 21,    // geodesic rest filter: (edge, vertex) entries below the activation
   SC_GEO_ERR = 22,      // ... error bits of its sources (a fixed capacity exceeded)
   SC_NX = 23,           // ccd_step: two uint32 counters, point-triangle and edge-edge pairs of the FP64 iteration
-  SC_N = 24
+  SC_NLONG = 24,        // barrier_eval: rows of the pattern with buckets past a warp's
+  SC_N = 25
 };
 // read_scalars stages up to SC_N scalars through the pinned host scratch
 static_assert(SC_N <= 64, "the scalars must fit the pinned scratch");

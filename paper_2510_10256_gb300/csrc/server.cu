@@ -178,17 +178,15 @@ cb_status cb_scene_reserve(cb_scene* s, int64_t n_candidates, int64_t n_ccd, int
   CB_TRY(buf_ensure(s->cd, sizeof(double) * nc, st));
   CB_TRY(buf_ensure(s->ctype, nc, st));
   CB_TRY(buf_ensure(s->ccls, nc, st));
-  CB_TRY(buf_ensure(s->cflag, sizeof(uint32_t) * nc, st));
-  CB_TRY(buf_ensure(s->cpos, sizeof(uint32_t) * (nc + 1), st));
+  CB_TRY(buf_ensure(s->clist, sizeof(uint32_t) * nc, st));
   CB_TRY(buf_ensure(s->dlist, sizeof(uint32_t) * std::max(nc, nq), st));
   // active pairs (stage d): compaction, BSR pattern keys, Hessian queues
-  CB_TRY(buf_ensure(s->aidx, sizeof(uint32_t) * na, st));
-  for (int k = 0; k < 2; ++k) CB_TRY(buf_ensure(s->bkey[k], sizeof(uint64_t) * 16 * na, st));
-  CB_TRY(buf_ensure(s->bflag, sizeof(uint32_t) * 16 * na, st));
-  CB_TRY(buf_ensure(s->bpos, sizeof(uint32_t) * (16 * na + 1), st));
-  CB_TRY(buf_ensure(s->horder, sizeof(uint32_t) * na, st));
+  CB_TRY(buf_ensure(s->aidx, sizeof(uint32_t) * nc, st));
+  CB_TRY(buf_ensure(s->bkey, sizeof(uint2) * 16 * na, st));
+  CB_TRY(buf_ensure(s->rcol, sizeof(uint32_t) * 16 * na, st));
   bool mollify = false;
   for (const MemberParams& m : s->hmp) mollify |= m.mollify != 0;
+  if (mollify) CB_TRY(buf_ensure(s->mlist, sizeof(uint32_t) * nc, st));
   if (mollify) CB_TRY(buf_ensure(s->hB9, sizeof(double) * 45 * na, st));
   // CCD candidates (stage e)
   CB_TRY(buf_ensure(s->ccd_keys, sizeof(uint64_t) * nq, st));
