@@ -87,7 +87,7 @@ static void scene_release(cb_scene* s) {
   cudaStream_t st = s->last_stream;
   DevBuf* bufs[] = {&s->ev0, &s->ev1, &s->tv, &s->comp, &s->rest, &s->rod_ptr, &s->slots, &s->cinfo, &s->supers, &s->jobs, &s->S, &s->win, &s->wst,
                     &s->rloop, &s->rlast, &s->elen2, &s->mlist, &s->ruv, &s->frest,
-                    &s->frest_dbar, &s->frest_j, &s->frow_pt, &s->frow_ee, &s->dbar_comp, &s->cand, &s->klass, &s->cand_alt, &s->klass_alt, &s->cd, &s->cflag, &s->cpos, &s->ctype, &s->ccls, &s->clist, &s->aidx,
+                    &s->frest_dbar, &s->fmask_key, &s->fmask_bits, &s->dbar_comp, &s->cand, &s->klass, &s->cand_alt, &s->klass_alt, &s->cd, &s->cflag, &s->cpos, &s->ctype, &s->ccls, &s->clist, &s->aidx,
                     &s->bkey, &s->rcol, &s->bsr_row, &s->bsr_col, &s->bsr_val,
                     &s->row_cnt, &s->hB9, &s->xf, &s->pf, &s->dlist, &s->mp, &s->vsc, &s->macc, &s->ccd_keys, &s->ccd_t, &s->ccd_cls, &s->ccd_list, &s->ccd_ulist, &s->scan_tmp,
                     &s->fr_key, &s->fr_st, &s->fr_dat, &s->fr_hw, &s->dev_scalars};
@@ -448,7 +448,8 @@ cb_status cb_scene_create(const cb_scene_desc* d, const cb_allocator* allocator,
     if ((rc = read_scalars(s, SC_COUNT1, 1, &h, st)) != CB_OK) return fail(rc);
     s->n_frest_pt = (int64_t)h;
   }
-  if ((rc = frest_rows_build(s, st)) != CB_OK) return fail(rc);
+  // the filtered pairs lie in the tiles of the rest broad phase
+  if ((rc = filter_masks_build(s, s->bw.n_tiles, st)) != CB_OK) return fail(rc);
   if (cudaStreamSynchronize(st) != cudaSuccess) return fail(CB_ERR_CUDA);
   *out = s;
   return CB_OK;
@@ -596,7 +597,9 @@ cb_status cb_batch_create(cb_scene* const* members, int32_t count, const cb_allo
                                sizeof(unsigned long long) * cnt, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
       return fail(CB_ERR_CUDA);
   }
-  if ((rc = frest_rows_build(b, st)) != CB_OK) return fail(rc);
+  int64_t tiles = 0;
+  for (int m = 0; m < count; ++m) tiles += members[m]->n_fmask;
+  if ((rc = filter_masks_build(b, tiles, st)) != CB_OK) return fail(rc);
   for (auto& e : b->ev)
     if (cudaEventCreate(&e) != cudaSuccess) return fail(CB_ERR_CUDA);
   if ((rc = upload_members(b, st)) != CB_OK) return fail(rc);
@@ -636,7 +639,7 @@ cb_status contact_build(cb_scene* s, const double* x, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   s->last_stream = st;
   stage_begin(s, 0, st);
-  cb_status r = broad_phase(s, s->bw, x, nullptr, false, false, s->cand, &s->n_cand, st);
+  cb_status r = broad_phase(s, s->bw, x, nullptr, false, false, s->cand, &s->klass, &s->n_cand, st);
   stage_end(s, 0, st);
   s->n_active = s->n_plane = 0;
   s->core_valid = false;

@@ -28,7 +28,6 @@
 
 #include "accd32.cuh"
 #include "geometry.cuh"
-#include "frest.cuh"
 #include "prims.cuh"
 #include "scene.cuh"
 
@@ -45,22 +44,14 @@ struct CcdArgs {
   const int32_t* __restrict__ ev0;
   const int32_t* __restrict__ ev1;
   const int32_t* __restrict__ tv;
-  const int32_t* __restrict__ comp;
-  const int32_t* __restrict__ win;
-  const int32_t* __restrict__ wst;
-  const int32_t* __restrict__ rloop;
-  const uint32_t* __restrict__ frest_j;  // partner index j of the sorted rest-filtered keys
-  const uint32_t* __restrict__ frow_pt;  // ... their row offsets by vertex and by edge (frest.cuh)
-  const uint32_t* __restrict__ frow_ee;
-  int64_t nf;
-  int T, n, kind;
+  int T, n;
   const int32_t* __restrict__ vsc;           // member of each vertex
   const MemberParams* __restrict__ mp;
   const double* __restrict__ cx;             // per member: centre[3], X
   const double* __restrict__ x;
   const double* __restrict__ p;
   double* __restrict__ t_out;
-  uint8_t* __restrict__ cls_out;
+  uint8_t* __restrict__ cls_out;             // in: 1 filtered, 3 culled, else 0 (Sec. 3.2); out: class | flags
   unsigned long long* __restrict__ macc;     // per member: alpha bits, status, smallest upper bound
   int members;
   unsigned long long* __restrict__ status;
@@ -85,15 +76,6 @@ __device__ __forceinline__ d3 ld(const double* __restrict__ a, int n, int v) {
 __device__ __forceinline__ double norm3(d3 a) { return __dsqrt_rn(dot3(a, a)); }
 __device__ __forceinline__ d3 axpy3(d3 x, double t, d3 p) {
   return mk3(xadd(x.x, xmul(t, p.x)), xadd(x.y, xmul(t, p.y)), xadd(x.z, xmul(t, p.z)));
-}
-
-// filtered class of a pair (Sec. 3.2 tables built at scene creation)
-__device__ __forceinline__ bool is_filtered(const CcdArgs& A, const MemberParams& M, uint64_t key, uint32_t ki,
-                                            uint32_t kj) {
-  if (M.filter_off) return false;
-  if (A.kind == CB_ROD) return A.comp[A.ev0[ki]] == A.comp[A.ev0[kj]] && rod_filtered(A.win, A.wst, M.loops != 0, ki, kj);
-  if (A.nf <= 0) return false;
-  return frest_contains(A.frest_j, A.frow_pt, A.frow_ee, key);
 }
 
 // Everything additive CCD needs before its first step.
@@ -124,7 +106,7 @@ __device__ __forceinline__ AccdStart accd_start(const CcdArgs& A, int64_t q) {
   }
   S.mem = A.vsc[v[0]];
   const MemberParams& M = A.mp[S.mem];
-  const bool filt = is_filtered(A, M, key, ki, kj);
+  const bool filt = (A.cls_out[q] & 3u) == 1u;
   const d3 X0 = ld(A.x, A.n, v[0]), X1 = ld(A.x, A.n, v[1]), X2 = ld(A.x, A.n, v[2]), X3 = ld(A.x, A.n, v[3]);
   const d3 P0 = ld(A.p, A.n, v[0]), P1 = ld(A.p, A.n, v[1]), P2 = ld(A.p, A.n, v[2]), P3 = ld(A.p, A.n, v[3]);
   double d;
@@ -236,13 +218,10 @@ __global__ void __launch_bounds__(128) k_ccd_screen(CcdArgs A, uint32_t* __restr
     }
     const int mem = A.vsc[v[0]];
     const MemberParams& M = A.mp[mem];
-    const bool filt = is_filtered(A, M, key, ki, kj);
+    const uint8_t cls0 = A.cls_out[q];
+    const bool filt = cls0 == 1;
     need = true;
-    // Kaldor culling (rods: edges numbered along each polyline): the pair
-    // does not constrain the step
-    const bool culled = M.cull_radius > 0 && A.comp[A.ev0[ki]] == A.comp[A.ev0[kj]] &&
-                        rod_gap(A.rloop, ki, kj) <= M.cull_radius;
-    if (culled) {
+    if (cls0 == 3) {  // culled (Kaldor mode): the pair does not constrain the step
       A.cls_out[q] = (uint8_t)3 | EXACT | ONE;
       need = false;
     } else {
@@ -501,7 +480,7 @@ __global__ void k_ccd_reset(unsigned long long* __restrict__ sc, int count, unsi
 }  // namespace
 
 cb_status ccd_run(cb_scene* s, const double* x, const double* p, double* alpha, cudaStream_t st) {
-  CB_TRY(broad_phase(s, s->bwc, x, p, true, false, s->ccd_keys, &s->n_ccd, st));
+  CB_TRY(broad_phase(s, s->bwc, x, p, true, false, s->ccd_keys, &s->ccd_cls, &s->n_ccd, st));
   uint64_t* sc = scalars(s);
   const int M = s->count;
   unsigned long long* macc = bp<unsigned long long>(s->macc);
@@ -510,7 +489,6 @@ cb_status ccd_run(cb_scene* s, const double* x, const double* p, double* alpha, 
   const int64_t np = s->n_ccd;
   if (np > 0) {
     CB_TRY(buf_ensure(s->ccd_t, sizeof(double) * (size_t)np, st));
-    CB_TRY(buf_ensure(s->ccd_cls, (size_t)np, st));
     CB_TRY(buf_ensure(s->ccd_list, sizeof(uint32_t) * (size_t)np, st));
     CB_TRY(buf_ensure(s->ccd_ulist, sizeof(uint32_t) * (size_t)np, st));
     CB_TRY(buf_ensure(s->dlist, sizeof(uint32_t) * (size_t)np, st));
@@ -520,17 +498,8 @@ cb_status ccd_run(cb_scene* s, const double* x, const double* p, double* alpha, 
     A.ev0 = bp<int32_t>(s->ev0);
     A.ev1 = bp<int32_t>(s->ev1);
     A.tv = bp<int32_t>(s->tv);
-    A.comp = bp<int32_t>(s->comp);
-    A.win = bp<int32_t>(s->win);
-    A.wst = bp<int32_t>(s->wst);
-    A.rloop = bp<int32_t>(s->rloop);
-    A.frest_j = bp<uint32_t>(s->frest_j);
-    A.frow_pt = bp<uint32_t>(s->frow_pt);
-    A.frow_ee = bp<uint32_t>(s->frow_ee);
-    A.nf = s->n_frest;
     A.T = s->T;
     A.n = s->n;
-    A.kind = s->kind;
     A.vsc = bp<int32_t>(s->vsc);
     A.mp = bp<MemberParams>(s->mp);
     A.cx = bp<double>(s->bwc.cx);

@@ -1,31 +1,43 @@
-// frest.cuh -- filter membership (Sec. 3.2).  Shells: a candidate is
-// filtered iff its stencil is in the rest-filter table built at scene
-// creation.  Rods: through the per-edge arc-length windows (below).  The shell
-// table is sorted by key (type, i, j), so the keys with one first primitive i
-// form a contiguous row; per-row offsets (by vertex for point-triangle keys,
-// by edge for edge-edge keys) bound the search to that row, a few dozen keys
-// that consecutive candidates (of one tile of primitives) share.
+// frest.cuh -- filter membership (Sec. 3.2).  Shells: a pair is filtered iff
+// its stencil is one of the rest mesh's filtered pairs, kept as bit masks over
+// pairs of primitive clusters (broad.cu).  Rods: through the per-edge
+// arc-length windows.
 #pragma once
 #include <cstdint>
 
 #include "common.cuh"
 
-// A row holds the keys of one (type, i), so the search compares only their
-// partner index j: fj[k] is the j of frest[k] (32 bits), which halves the
-// bytes a search touches.
-__device__ __forceinline__ bool frest_contains(const uint32_t* __restrict__ fj, const uint32_t* __restrict__ row_pt,
-                                               const uint32_t* __restrict__ row_ee, uint64_t key) {
-  const uint32_t i = cb_key_i(key), j = cb_key_j(key);
-  const uint32_t* __restrict__ row = cb_key_type(key) == CB_KEY_PT ? row_pt : row_ee;
-  const int64_t end = row[i + 1];
-  int64_t lo = row[i], hi = end;
-  while (lo < hi) {
-    const int64_t mid = (lo + hi) >> 1;
-    if (fj[mid] < j) lo = mid + 1;
-    else hi = mid;
+// The filtered pairs of a shell's rest mesh as 32x32 bit masks over the pairs
+// of clusters that hold any: an open-addressing table (linear probing, at most
+// half full) of tile keys, and at the same place the mask, word r for row
+// primitive r.
+struct FilterMasks {
+  const unsigned long long* __restrict__ key;
+  const uint32_t* __restrict__ bits;
+  uint32_t mask;  // table size - 1 (0: no filtered pair)
+
+  static constexpr unsigned long long EMPTY = ~0ull;
+  __host__ __device__ static __forceinline__ unsigned long long tile_key(uint32_t row, uint32_t col) {
+    return ((unsigned long long)row << 32) | col;
   }
-  return lo < end && fj[lo] == j;
-}
+  // multiplicative (Fibonacci) hashing of the tile key, Knuth
+  __host__ __device__ static __forceinline__ uint32_t hash(unsigned long long k) {
+    return (uint32_t)((k * 0x9E3779B97F4A7C15ull) >> 32);
+  }
+  // word `lane` of the tile's mask (0 if it has none); every lane of the warp
+  // calls it with the same tile, and the lanes probe 32 places at once
+  __device__ __forceinline__ uint32_t row(uint32_t r, uint32_t c, int lane) const {
+    if (mask == 0u) return 0u;
+    const unsigned long long k = tile_key(r, c);
+    for (uint32_t h = hash(k);; h += 32u) {
+      const unsigned long long e = key[(h + (uint32_t)lane) & mask];
+      const unsigned hit = __ballot_sync(0xffffffffu, e == k), end = __ballot_sync(0xffffffffu, e == EMPTY);
+      const int at = __ffs((int)hit) - 1, stop = __ffs((int)end) - 1;
+      if (at >= 0 && (stop < 0 || at < stop)) return bits[(size_t)((h + (uint32_t)at) & mask) * 32 + lane];
+      if (stop >= 0) return 0u;  // (half of the table is empty: the loop ends)
+    }
+  }
+};
 
 // Rods: edges ki < kj of one polyline are filtered when kj is within the
 // forward window of ki (kj <= win[ki]) or, on a closed loop, within its

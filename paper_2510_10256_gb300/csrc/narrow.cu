@@ -6,7 +6,6 @@
 
 #include "bound32.cuh"
 #include "geometry.cuh"
-#include "frest.cuh"
 #include "pairhess.cuh"
 #include "pairs.cuh"
 #include "prims.cuh"
@@ -162,74 +161,31 @@ __device__ __forceinline__ double member_f_width(const MemberParams& M, const un
 // class byte of a filtered candidate dropped by the per-stencil activation
 constexpr uint8_t KL_DROPPED = 0xFE;
 
-struct StencilArgs {
-  const double* __restrict__ box_raw;            // null unless a member uses per-stencil activation
-  const unsigned long long* __restrict__ dbar_comp;
-  const int32_t* __restrict__ comp;
-  unsigned long long* __restrict__ ndrop;
-};
-
-__global__ void k_filter_rod(int64_t nc, const uint64_t* __restrict__ cand, const int32_t* __restrict__ ev0,
-                             const int32_t* __restrict__ comp, const int32_t* __restrict__ win,
-                             const int32_t* __restrict__ wst, const int32_t* __restrict__ rloop,
-                             const int32_t* __restrict__ vsc, const MemberParams* __restrict__ mp,
-                             uint8_t* __restrict__ klass, unsigned long long* __restrict__ nfilt, StencilArgs SA) {
+// Per-stencil activation: the class-F candidates outside their own width take
+// class KL_DROPPED (counted in ndrop); the rest are counted in nfilt.
+__global__ void k_own_width(int64_t nc, const uint64_t* __restrict__ cand, const double* __restrict__ box_raw,
+                            const int32_t* __restrict__ ev0, const int32_t* __restrict__ vsc,
+                            const MemberParams* __restrict__ mp, const unsigned long long* __restrict__ dbar_comp,
+                            const int32_t* __restrict__ comp, bool rod, int n, int T, uint8_t* __restrict__ klass,
+                            unsigned long long* __restrict__ nfilt, unsigned long long* __restrict__ ndrop) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  uint32_t f = 0, dropped = 0;
-  if (c < nc) {
-    const uint64_t key = cand[c];
-    const uint32_t k = cb_key_i(key), l = cb_key_j(key);
-    const int v0 = ev0[k];
-    const MemberParams& M = mp[vsc[v0]];
-    const bool same = comp[v0] == comp[ev0[l]];
-    f = (!M.filter_off && same && rod_filtered(win, wst, M.loops != 0, k, l)) ? 1u : 0u;
-    // Kaldor culling: edges are numbered along each polyline, so the gap is
-    // l - k (the shorter way round on a closed loop)
-    uint8_t kl = (M.cull_radius > 0 && same && rod_gap(rloop, k, l) <= M.cull_radius) ? (uint8_t)3 : (uint8_t)f;
-    if (kl == 1 && M.per_stencil &&
-        !within_own_width(SA.box_raw, k, l, member_f_width(M, SA.dbar_comp, SA.comp, v0))) {
-      kl = KL_DROPPED;
-      f = 0;
-      dropped = 1;
-    }
-    klass[c] = kl;
-  }
-  uint32_t b = __ballot_sync(0xffffffffu, f);
-  if ((threadIdx.x & 31) == 0 && b) atomicAdd(nfilt, (unsigned long long)__popc(b));
-  b = __ballot_sync(0xffffffffu, dropped);
-  if ((threadIdx.x & 31) == 0 && b) atomicAdd(SA.ndrop, (unsigned long long)__popc(b));
-}
-
-__global__ void k_filter_shell(int64_t nc, const uint64_t* __restrict__ cand, const uint32_t* __restrict__ frest_j,
-                               const uint32_t* __restrict__ row_pt, const uint32_t* __restrict__ row_ee, int64_t nf,
-                               const int32_t* __restrict__ ev0, const int32_t* __restrict__ vsc,
-                               const MemberParams* __restrict__ mp, uint8_t* __restrict__ klass,
-                               unsigned long long* __restrict__ nfilt, int n, int T, StencilArgs SA) {
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  uint32_t f = 0, dropped = 0;
-  if (c < nc) {
+  bool f = false, dropped = false;
+  if (c < nc && klass[c] == 1) {
     const uint64_t key = cand[c];
     const bool pt = cb_key_type(key) == CB_KEY_PT;
-    const int v0 = pt ? (int)cb_key_i(key) : ev0[cb_key_i(key)];
+    const int64_t i = cb_key_i(key), j = cb_key_j(key);
+    const int v0 = pt ? (int)i : ev0[i];
     const MemberParams& M = mp[vsc[v0]];
-    if (!M.filter_off && nf > 0) f = frest_contains(frest_j, row_pt, row_ee, key) ? 1u : 0u;
-    uint8_t kl = (uint8_t)f;
-    if (f && M.per_stencil) {
-      // broad-phase primitive ids: vertices, then triangles, then edges
-      const int64_t p1 = pt ? (int64_t)cb_key_i(key) : (int64_t)n + T + cb_key_i(key);
-      const int64_t p2 = pt ? (int64_t)n + cb_key_j(key) : (int64_t)n + T + cb_key_j(key);
-      if (!within_own_width(SA.box_raw, p1, p2, member_f_width(M, SA.dbar_comp, SA.comp, v0))) {
-        kl = KL_DROPPED;
-        f = 0;
-        dropped = 1;
-      }
-    }
-    klass[c] = kl;
+    // broad-phase primitive ids: vertices, then triangles, then edges (rods: edges)
+    const int64_t p1 = pt || rod ? i : (int64_t)n + T + i, p2 = rod ? j : (pt ? (int64_t)n + j : (int64_t)n + T + j);
+    dropped = M.per_stencil && !within_own_width(box_raw, p1, p2, member_f_width(M, dbar_comp, comp, v0));
+    f = !dropped;
+    if (dropped) klass[c] = KL_DROPPED;
   }
   uint32_t b = __ballot_sync(0xffffffffu, f);
   if ((threadIdx.x & 31) == 0 && b) atomicAdd(nfilt, (unsigned long long)__popc(b));
   b = __ballot_sync(0xffffffffu, dropped);
-  if ((threadIdx.x & 31) == 0 && b) atomicAdd(SA.ndrop, (unsigned long long)__popc(b));
+  if ((threadIdx.x & 31) == 0 && b) atomicAdd(ndrop, (unsigned long long)__popc(b));
 }
 
 // per-stencil activation: keep flags of the candidates, then the kept ones
@@ -1991,7 +1947,7 @@ cb_status filter_precompute(cb_scene* s, cudaStream_t st) {
     DevBuf& rc = rcs.b;
     // positions of the reference distances: the flat pattern when given, else the rest shape
     const double* rf = s->ruv.p ? bp<double>(s->ruv) : bp<double>(s->rest);
-    CB_TRY(broad_phase(s, s->bw, rf, nullptr, false, true, rc, &nr, st));
+    CB_TRY(broad_phase(s, s->bw, rf, nullptr, false, true, rc, nullptr, &nr, st));
     if (nr > 0) {
       ScopedBuf flags(st), poss(st), dbars(st);
       DevBuf &flag = flags.b, &pos = poss.b, &dbar = dbars.b;
@@ -2047,70 +2003,29 @@ cb_status filter_precompute(cb_scene* s, cudaStream_t st) {
   return CB_OK;
 }
 
-// Row offsets of the sorted rest-filter table: row[r] = first index whose key
-// is at or above (type, r, 0), for r = 0..nrows (row[nrows] ends the type).
-__global__ void k_frest_rows(int64_t nrows, uint32_t type, const uint64_t* __restrict__ frest, int64_t nf,
-                             uint32_t* __restrict__ row) {
-  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r > nrows) return;
-  const uint64_t bound = ((uint64_t)type << 62) | ((uint64_t)r << 31);
-  int64_t lo = 0, hi = nf;
-  while (lo < hi) {
-    const int64_t mid = (lo + hi) >> 1;
-    if (frest[mid] < bound) lo = mid + 1;
-    else hi = mid;
-  }
-  row[r] = (uint32_t)lo;
-}
-
-// the partner index j of every rest-filtered key (the low 31 bits)
-__global__ void k_frest_j(int64_t nf, const uint64_t* __restrict__ frest, uint32_t* __restrict__ fj) {
-  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < nf) fj[k] = cb_key_j(frest[k]);
-}
-
-cb_status frest_rows_build(cb_scene* s, cudaStream_t st) {
-  if (s->kind != CB_SHELL || s->n_frest <= 0) return CB_OK;
-  CB_TRY(buf_ensure(s->frest_j, sizeof(uint32_t) * (size_t)s->n_frest, st));
-  k_frest_j<<<cb_grid(s->n_frest), CB_THREADS, 0, cb_count(st)>>>(s->n_frest, bp<uint64_t>(s->frest),
-                                                                  bp<uint32_t>(s->frest_j));
-  CB_TRY(buf_ensure(s->frow_pt, sizeof(uint32_t) * ((size_t)s->n + 1), st));
-  CB_TRY(buf_ensure(s->frow_ee, sizeof(uint32_t) * ((size_t)s->E + 1), st));
-  k_frest_rows<<<cb_grid((int64_t)s->n + 1), CB_THREADS, 0, cb_count(st)>>>(s->n, CB_KEY_PT, bp<uint64_t>(s->frest),
-                                                                           s->n_frest, bp<uint32_t>(s->frow_pt));
-  k_frest_rows<<<cb_grid((int64_t)s->E + 1), CB_THREADS, 0, cb_count(st)>>>(s->E, CB_KEY_EE, bp<uint64_t>(s->frest),
-                                                                           s->n_frest, bp<uint32_t>(s->frow_ee));
-  CB_CUDA(cudaGetLastError());
-  return CB_OK;
-}
-
+// The candidates' classes come with them from contact_build (broad.cu); what
+// is left here is their count and the per-stencil activation.
 cb_status filter_apply(cb_scene* s, cudaStream_t st) {
   const int64_t nc = s->n_cand;
-  CB_TRY(buf_ensure(s->klass, (size_t)std::max<int64_t>(1, nc), st));
-  unsigned long long* nf = (unsigned long long*)(scalars(s) + SC_NFILT);
-  k_set_u64<<<1, 1, 0, cb_count(st)>>>(nf, 0ull);
+  uint64_t* sc = scalars(s);
+  unsigned long long* nf = (unsigned long long*)(sc + SC_NFILT);
   s->n_dropped = 0;
-  if (nc == 0) return CB_OK;
   const bool ps = s->per_stencil();
-  unsigned long long* ndrop = (unsigned long long*)(scalars(s) + SC_COUNT1);
-  if (ps) {
-    if (!s->bw.box_raw.p) return CB_ERR_ARG;  // the candidates came from before the mode was set
-    k_set_u64<<<1, 1, 0, cb_count(st)>>>(ndrop, 0ull);
+  if (nc == 0 || ps) {
+    CB_CUDA(cudaMemsetAsync(nf, 0, sizeof(unsigned long long), st));
+    if (nc == 0) return CB_OK;
+  } else {
+    CB_CUDA(cudaMemcpyAsync(nf, sc + SC_NFB, sizeof(unsigned long long), cudaMemcpyDeviceToDevice, st));
+    return CB_OK;
   }
-  const StencilArgs SA{ps ? bp<double>(s->bw.box_raw) : nullptr, bp<unsigned long long>(s->dbar_comp),
-                       bp<int32_t>(s->comp), ndrop};
-  if (s->kind == CB_ROD)
-    k_filter_rod<<<cb_grid(nc), CB_THREADS, 0, cb_count(st)>>>(
-        nc, bp<uint64_t>(s->cand), bp<int32_t>(s->ev0), bp<int32_t>(s->comp), bp<int32_t>(s->win),
-        bp<int32_t>(s->wst), bp<int32_t>(s->rloop), bp<int32_t>(s->vsc), bp<MemberParams>(s->mp),
-        bp<uint8_t>(s->klass), nf, SA);
-  else
-    k_filter_shell<<<cb_grid(nc), CB_THREADS, 0, cb_count(st)>>>(
-        nc, bp<uint64_t>(s->cand), bp<uint32_t>(s->frest_j), bp<uint32_t>(s->frow_pt), bp<uint32_t>(s->frow_ee),
-        s->n_frest, bp<int32_t>(s->ev0), bp<int32_t>(s->vsc), bp<MemberParams>(s->mp), bp<uint8_t>(s->klass), nf,
-        s->n, s->T, SA);
+  if (!s->bw.box_raw.p) return CB_ERR_ARG;  // the candidates came from before the mode was set
+  unsigned long long* ndrop = (unsigned long long*)(sc + SC_COUNT1);
+  k_set_u64<<<1, 1, 0, cb_count(st)>>>(ndrop, 0ull);
+  k_own_width<<<cb_grid(nc), CB_THREADS, 0, cb_count(st)>>>(
+      nc, bp<uint64_t>(s->cand), bp<double>(s->bw.box_raw), bp<int32_t>(s->ev0), bp<int32_t>(s->vsc),
+      bp<MemberParams>(s->mp), bp<unsigned long long>(s->dbar_comp), bp<int32_t>(s->comp), s->kind == CB_ROD, s->n,
+      s->T, bp<uint8_t>(s->klass), nf, ndrop);
   CB_CUDA(cudaGetLastError());
-  if (!ps) return CB_OK;
   // per-stencil activation: drop the class-F candidates outside their own width
   uint64_t hd;
   CB_TRY(read_scalars(s, SC_COUNT1, 1, &hd, st));

@@ -81,6 +81,7 @@ struct BroadWork {
   DevBuf bounds;      // per member: 6 x uint32 ordered-float min/max
   DevBuf cx;          // per member: double centre[3], X (max |coordinate - centre|)
   DevBuf tiles;       // uint2 pairs of overlapping clusters
+  int64_t n_tiles = 0;  // of the last call
   DevBuf ckey[2];     // uint64 compact candidate keys (ping-pong; sorted lists only)
   DevBuf scan_tmp;
   DevBuf hist;
@@ -141,12 +142,14 @@ struct cb_scene {
   std::vector<int32_t> geo_te, geo_ef, geo_vfp, geo_vf;
   DevBuf frest;         // uint64 shells: sorted rest-filtered keys
   DevBuf frest_dbar;    // double
-  DevBuf frest_j;       // uint32 shells: the partner index j of each frest key (the rows' search keys)
   DevBuf dbar_comp;     // uint64 bits of the per-component dbar_min, by component label (n entries)
   double dbar_fmax = 0.0;  // largest per-component dbar_min (finite), or dbar_min
   int64_t n_frest = 0;
-  DevBuf frow_pt;       // uint32 shells: row offsets of frest by vertex (point-triangle keys), n + 1
-  DevBuf frow_ee;       // uint32 shells: row offsets of frest by edge (edge-edge keys), E + 1
+  // shells: frest as bit masks over pairs of clusters (frest.cuh, FilterMasks)
+  DevBuf fmask_key;     // uint64 [fmask_cap]
+  DevBuf fmask_bits;    // uint32 [fmask_cap][32]
+  uint32_t fmask_cap = 0;
+  int64_t n_fmask = 0;  // pairs of clusters with filtered pairs
 
   // pass state
   BroadWork bw;         // static broad phase
@@ -240,10 +243,11 @@ enum {
   SC_GEO_ERR = 22,      // ... error bits of its sources (a fixed capacity exceeded)
   SC_NX = 23,           // ccd_step: two uint32 counters, point-triangle and edge-edge pairs of the FP64 iteration
   SC_NLONG = 24,        // barrier_eval: rows of the pattern with buckets past a warp's
-  SC_N = 25
+  SC_NFB = 25,          // contact_build: filtered pairs among the candidates
+  SC_N = 26
 };
 // read_scalars stages up to SC_N scalars through the pinned host scratch
-static_assert(SC_N <= 64, "the scalars must fit the pinned scratch");
+static_assert(SC_N <= 32, "the scalars must fit the pinned scratch and a 32-bit mask");
 
 static inline uint64_t* scalars(cb_scene* s) { return (uint64_t*)s->dev_scalars.p; }
 
@@ -264,9 +268,12 @@ cb_status clusters_concat(cb_scene* b, cb_scene* const* members, cudaStream_t st
 // Candidate pairs of x (p == nullptr) or of the sweep x -> x + p.  Boxes are
 // inflated per member by a/2 (static) or xi/2 (swept = true).  Writes the
 // canonical keys into *out (grown as needed), in ascending order when
-// sort_out is set and otherwise in tile order, and their count into *n_out.
+// sort_out is set and otherwise in tile order, their classes (1 filtered,
+// 3 culled, else 0) into *cls unless null, and their count into *n_out.
 cb_status broad_phase(cb_scene* s, BroadWork& w, const double* x, const double* p, bool swept, bool sort_out,
-                      DevBuf& out, int64_t* n_out, cudaStream_t st);
+                      DevBuf& out, DevBuf* cls, int64_t* n_out, cudaStream_t st);
+// the bit masks of the filtered pairs s->frest, which lie in at most max_tiles pairs of clusters
+cb_status filter_masks_build(cb_scene* s, int64_t max_tiles, cudaStream_t st);
 
 // narrow.cu
 cb_status filter_precompute(cb_scene* s, cudaStream_t st);
@@ -275,7 +282,6 @@ cb_status filter_precompute(cb_scene* s, cudaStream_t st);
 cb_status geo_rest_dbar(cb_scene* s, const uint64_t* cand, int64_t nc, uint32_t* flag, double* dbar,
                         unsigned long long* dmin, unsigned long long* dcomp, cudaStream_t st);
 cb_status filter_apply(cb_scene* s, cudaStream_t st);
-cb_status frest_rows_build(cb_scene* s, cudaStream_t st);
 // energy_only: distances and energy (no active list, gradient, Hessian or BSR)
 cb_status barrier_run(cb_scene* s, const double* x, double* energy, double* grad, bool energy_only,
                       cudaStream_t st);
