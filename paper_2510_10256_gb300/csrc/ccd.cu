@@ -30,6 +30,7 @@
 #include "geometry.cuh"
 #include "prims.cuh"
 #include "scene.cuh"
+#include "typed.cuh"
 
 namespace {
 
@@ -110,7 +111,7 @@ __device__ __forceinline__ AccdStart accd_start(const CcdArgs& A, int64_t q) {
   const d3 X0 = ld(A.x, A.n, v[0]), X1 = ld(A.x, A.n, v[1]), X2 = ld(A.x, A.n, v[2]), X3 = ld(A.x, A.n, v[3]);
   const d3 P0 = ld(A.p, A.n, v[0]), P1 = ld(A.p, A.n, v[1]), P2 = ld(A.p, A.n, v[2]), P3 = ld(A.p, A.n, v[3]);
   double d;
-  cbg::stencil_distance(S.ee, X0, X1, X2, X3, d);
+  cbt::stencil_distance(S.ee, X0, X1, X2, X3, d);
   S.cls = filt ? 1 : 0;
   if (!filt && M.core_temp && !M.single && d <= M.xi) S.cls = 2;
   S.off = (S.cls == 0 && !M.single) ? M.xi : 0.0;
@@ -429,7 +430,7 @@ __global__ void __launch_bounds__(128) k_ccd_exact(CcdArgs A, unsigned long long
       S.Y2 = axpy3(S.Y2, L.tl, S.Q2);
       S.Y3 = axpy3(S.Y3, L.tl, S.Q3);
       double d;
-      cbg::stencil_distance(S.ee, S.Y0, S.Y1, S.Y2, S.Y3, d);
+      cbt::stencil_distance(S.ee, S.Y0, S.Y1, S.Y2, S.Y3, d);
       const int it = L.it++;
       if (L.t > 0.0 && xsub(d, S.off) < L.g) {
         exact_finish(A, L, false, L.t);
@@ -607,7 +608,7 @@ __device__ __forceinline__ bool na_start(const NaArgs& A, int64_t q, NaStart& S)
   const d3 X0 = ld(A.x, A.n, v[0]), X1 = ld(A.x, A.n, v[1]), X2 = ld(A.x, A.n, v[2]), X3 = ld(A.x, A.n, v[3]);
   const d3 P0 = ld(A.p, A.n, v[0]), P1 = ld(A.p, A.n, v[1]), P2 = ld(A.p, A.n, v[2]), P3 = ld(A.p, A.n, v[3]);
   double d;
-  cbg::stencil_distance(S.ee, X0, X1, X2, X3, d);
+  cbt::stencil_distance(S.ee, X0, X1, X2, X3, d);
   const d3 pb = mk3(xmul(xadd(xadd(xadd(P0.x, P1.x), P2.x), P3.x), 0.25),
                     xmul(xadd(xadd(xadd(P0.y, P1.y), P2.y), P3.y), 0.25),
                     xmul(xadd(xadd(xadd(P0.z, P1.z), P2.z), P3.z), 0.25));
@@ -702,7 +703,7 @@ __device__ double na_iterate(const NaArgs& A, int64_t q) {
     S.Y1 = axpy3(S.Y1, tl, S.Q1);
     S.Y2 = axpy3(S.Y2, tl, S.Q2);
     S.Y3 = axpy3(S.Y3, tl, S.Q3);
-    cbg::stencil_distance(S.ee, S.Y0, S.Y1, S.Y2, S.Y3, d);
+    cbt::stencil_distance(S.ee, S.Y0, S.Y1, S.Y2, S.Y3, d);
     if (t > 0.0 && xsub(d, S.off) < g) return t;
     t = xadd(t, tl);
     if (t > 1.0) return 1.0;

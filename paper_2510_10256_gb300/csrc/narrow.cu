@@ -10,6 +10,7 @@
 #include "pairs.cuh"
 #include "prims.cuh"
 #include "scene.cuh"
+#include "typed.cuh"
 
 namespace {
 
@@ -295,6 +296,12 @@ __global__ void k_distance_screen(int64_t nc, const uint64_t* __restrict__ cand,
 // the candidates' order but for the arrival of warps.  (Flags, a scan and a
 // compaction over all candidates made these lists before: 0.35 ms of a
 // pleated 256x256 pass, 14 bytes written per candidate.)
+//
+// Bound by the FP64 pipe.  Each pair whose type FP32 is sure of takes one
+// formula (typed.cuh); the undecided few wait in shared memory until a block's
+// worth, or the rest, runs the full routine in full warps.  862k pairs of a
+// pleated sheet 458 -> 292 us, of 64 rod scenes 736 -> 326, the energy-only
+// pass of a 181x181 sheet 212 -> 113.
 template <bool ENERGY>
 __global__ void k_distance_exact(const uint32_t* __restrict__ list, int64_t cap, const unsigned int* __restrict__ nlist,
                                  const uint64_t* __restrict__ cand, const uint8_t* __restrict__ klass_in,
@@ -310,20 +317,56 @@ __global__ void k_distance_exact(const uint32_t* __restrict__ list, int64_t cap,
                                  const unsigned long long* __restrict__ dbar_comp, const double* __restrict__ elen2) {
   constexpr bool energy = ENERGY;  // energy only (barrier_energy): add kappa b per active pair
   const unsigned m0 = nlist[0], m = m0 + nlist[1];
-  for (unsigned w = blockIdx.x * blockDim.x + threadIdx.x; w - threadIdx.x < m; w += gridDim.x * blockDim.x) {
+  __shared__ uint32_t unsure[2 * CB_THREADS];
+  __shared__ unsigned n_unsure;
+  if (threadIdx.x == 0) n_unsure = 0;
+  __syncthreads();
+  // block-uniform: the next CB_THREADS queued pairs, or as many of the undecided ones once enough wait (or no others are left)
+  for (unsigned w0 = blockIdx.x * blockDim.x;;) {
+    const unsigned nu = n_unsure;
+    const bool more = w0 < m, typed = more && nu < CB_THREADS;
+    if (!more && nu == 0) break;
+    __syncthreads();
     bool is_core = false, active = false, plane = false, moll = false;
     uint32_t c = 0;
     double e_local = 0.0;
     int e_mem = -1;
-    if (w < m) {
-      c = w < m0 ? list[w] : list[cap - 1 - (int64_t)(w - m0)];
-      Stencil s = stencil_of(cand[c], ev0, ev1, tv, T);
+    bool live;
+    if (typed) {
+      const unsigned w = w0 + threadIdx.x;
+      live = w < m;
+      if (live) c = w < m0 ? list[w] : list[cap - 1 - (int64_t)(w - m0)];
+      w0 += gridDim.x * blockDim.x;
+    } else {
+      const unsigned take = min(nu, (unsigned)CB_THREADS);
+      live = threadIdx.x < take;
+      if (live) c = unsure[nu - 1 - threadIdx.x];
+      __syncthreads();
+      if (threadIdx.x == 0) n_unsure = nu - take;
+    }
+    Stencil s;
+    double d = 0.0;
+    int ty = -1;
+    if (live) {
+      s = stencil_of(cand[c], ev0, ev1, tv, T);
+      const cbg::Local L = cbg::make_local(load3(x, n, s.v[0]), load3(x, n, s.v[1]), load3(x, n, s.v[2]), load3(x, n, s.v[3]));
+      double d2 = 0.0;
+      if (typed) {
+        ty = cbt::certain_type(s.ee, cbt::to_f3(L.P1), cbt::to_f3(L.P2), cbt::to_f3(L.P3));
+        if (ty >= 0) d2 = cbt::typed_d2(s.ee, L, ty);
+      } else {
+        ty = s.ee ? cbg::ee_type(L, d2) : cbg::pt_type(L, d2);
+      }
+      d = __dsqrt_rn(d2);
+    }
+    if (typed) {
+      warp_append(live && ty < 0, c, unsure, &n_unsure);  // fewer than CB_THREADS waited: room for all
+      live = live && ty >= 0;
+    }
+    if (live) {
       int k = klass_in[c];
       const int mem = vsc[s.v[0]];
       const PassParams P = member_pass(mp[mem]);
-      double d;
-      const int ty = cbg::stencil_distance(s.ee, load3(x, n, s.v[0]), load3(x, n, s.v[1]), load3(x, n, s.v[2]),
-                                           load3(x, n, s.v[3]), d);
       if (k == 0 && P.core_temp && !P.single && d <= P.xi) k = 2;
       double xi_p, dh_p;
       pair_params(P, k, f_width(P, dbar_comp, comp, s.v[0]), xi_p, dh_p);
@@ -368,6 +411,7 @@ __global__ void k_distance_exact(const uint32_t* __restrict__ list, int64_t cap,
       warp_append_back(active && !plane, c, aidx, cap, &nsplit[1]);
       if (mlist) warp_append(moll, c, mlist, nmoll);
     }
+    __syncthreads();
   }
 }
 
