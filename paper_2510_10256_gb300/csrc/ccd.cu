@@ -26,6 +26,7 @@
 #include <cstring>
 #include <mutex>
 
+#include "accd16.cuh"
 #include "accd32.cuh"
 #include "geometry.cuh"
 #include "prims.cuh"
@@ -358,6 +359,12 @@ __global__ void __launch_bounds__(128) k_ccd_refine(CcdArgs A) {
 // runs once for a group of lanes instead of once per lane that finishes.
 // A pair's arithmetic is the same whichever lane runs it.
 constexpr int EXACT_REFILL = 8;
+// Pairs per 128-thread block (one per SM) up to which a half-warp takes each (accd16.cuh).  A half-warp's step costs
+// its warp 25 FP64 instructions a pair, 32 single lanes' 3.5 -- but they wait for the longest of 32 pairs, at twice the
+// time a step.  With every pair alike (a tie, three steps each; the worst case for half-warps) the two are even at
+// 2,000 pairs and 5,000 take 110 against 76 us; with 2,500 pairs of 6 steps and one of 236 half-warps take 507 us
+// against 984.  The line lies at 4,864 pairs on 152 SMs: at most 0.03 ms lost, half a millisecond won.
+constexpr int FEW_PER_BLOCK = 32;
 
 struct ExactLane {
   AccdStart S;
@@ -367,16 +374,79 @@ struct ExactLane {
 };
 
 // finish a pair: exact t_p, or (stopped) a lower bound
+__device__ __forceinline__ void exact_finish(const CcdArgs& A, int64_t q, int mem, int cls, bool stopped, double t) {
+  A.t_out[q] = t;
+  A.cls_out[q] = (uint8_t)cls | (stopped ? 0 : EXACT);
+  if (!stopped) atomicMin(macc_of(A, mem, MACC_ALPHA), (unsigned long long)__double_as_longlong(t));
+}
 __device__ __forceinline__ void exact_finish(const CcdArgs& A, const ExactLane& L, bool stopped, double t) {
-  A.t_out[L.q] = t;
-  A.cls_out[L.q] = (uint8_t)L.S.cls | (stopped ? 0 : EXACT);
-  if (!stopped) atomicMin(macc_of(A, L.S.mem, MACC_ALPHA), (unsigned long long)__double_as_longlong(t));
+  exact_finish(A, L.q, L.S.mem, L.S.cls, stopped, t);
 }
 
+// a short list: half a warp per pair (accd16.cuh)
+struct ExactJob {
+  const CcdArgs& A;
+  int64_t mf;  // point-triangle pairs, from the list's front
+  int64_t q;
+  int mem, cls;
+
+  __device__ __forceinline__ bool take(int64_t w, cba::Pair16& S) {
+    q = w < mf ? A.list[w] : A.list[A.np - 1 - (w - mf)];
+    const uint64_t key = A.keys[q];
+    const uint32_t ki = cb_key_i(key), kj = cb_key_j(key);
+    const bool ee = cb_key_type(key) != CB_KEY_PT;
+    const int k = cba::quad_vertex();
+    const int v0 = ee ? A.ev0[ki] : (int)ki;
+    mem = A.members > 1 ? A.vsc[v0] : 0;
+    if (!(__double2float_rd(A.t_out[q]) <= member_cap(A, mem))) return false;
+    const uint32_t e = k < 2 ? ki : kj;
+    const int v = ee ? (k & 1 ? A.ev1[e] : A.ev0[e]) : (k == 0 ? v0 : A.tv[(size_t)(k - 1) * A.T + kj]);
+    cba::load16(A.x, A.p, A.n, v, ee, S);
+    return true;
+  }
+  __device__ __forceinline__ bool begin(cba::Pair16& S, double d) {
+    const MemberParams& M = A.mp[mem];
+    cls = (A.cls_out[q] & 3u) == 1u ? 1 : 0;
+    if (cls == 0 && M.core_temp && !M.single && d <= M.xi) cls = 2;
+    S.off = (cls == 0 && !M.single) ? M.xi : 0.0;
+    const double g0 = S.lp != 0.0 ? xsub(d, S.off) : 0.0;
+    if (S.lp == 0.0 || g0 <= 0.0) {
+      if (S.lp != 0.0 && cba::half_leader()) {
+        atomicOr(A.status, (unsigned long long)CB_DEV_PENETRATION);
+        atomicOr(macc_of(A, mem, MACC_STATUS), (unsigned long long)CB_DEV_PENETRATION);
+      }
+      done(S, S.lp == 0.0 ? 1.0 : 0.0, cba::REACHED);
+      return false;
+    }
+    S.hi = __longlong_as_double(*macc_of(A, mem, MACC_HI));
+    S.cap = cap(S);
+    S.g = xmul(ACCD_S, g0);
+    S.tl = xdiv(xmul(xsub(1.0, ACCD_S), g0), S.lp);
+    return true;
+  }
+  __device__ __forceinline__ double cap(const cba::Pair16&) const {
+    return __longlong_as_double(*(volatile unsigned long long*)macc_of(A, mem, MACC_ALPHA));
+  }
+  __device__ __forceinline__ void done(const cba::Pair16&, double t, cba::Done how) const {
+    if (!cba::half_leader()) return;
+    if (how == cba::LIMIT) atomicOr(A.status, (unsigned long long)CB_DEV_ITER_LIMIT);
+    exact_finish(A, q, mem, cls, how == cba::STOPPED, t);
+  }
+};
+
 // fetch: a zeroed counter of the pairs handed out
-__global__ void __launch_bounds__(128) k_ccd_exact(CcdArgs A, unsigned long long* __restrict__ fetch) {
+__global__ void __launch_bounds__(128) k_ccd_exact(CcdArgs A, unsigned long long* __restrict__ fetch, int sms) {
   const int64_t mf = min((int64_t)A.nlist[0], A.np), m = min(mf + (int64_t)A.nlist[1], A.np);
   const unsigned lane = threadIdx.x & 31u;
+  const int blocks = min((int)gridDim.x, sms);  // of the short form: one FP64 warp per SM quarter
+  if (m <= (int64_t)blocks * FEW_PER_BLOCK) {
+    if (blockIdx.x >= blocks) return;
+    ExactJob J{A, mf, 0, 0, 0};
+    const int most = cba::iterate16(J, m, 4 * blocks, (int)(threadIdx.x >> 5) * blocks + (int)blockIdx.x, ACCD_C, ACCD_MAX_ITER);
+    const int wm = __reduce_max_sync(0xffffffffu, most);
+    if (lane == 0 && wm > 0) atomicMax(A.max_iters, (unsigned long long)wm);
+    return;
+  }
   const unsigned below = (1u << lane) - 1u;
   ExactLane L;
   bool have = false, drained = false;
@@ -525,9 +595,9 @@ cb_status ccd_run(cb_scene* s, const double* x, const double* p, double* alpha, 
     k_ccd_bound<<<std::min<int64_t>(cb_grid(np, 128), (int64_t)s->n_sms * 16), 128, 0, cb_count(st)>>>(
         A, bp<uint32_t>(s->dlist), nl);
     k_ccd_refine<<<std::min<int64_t>(cb_grid(np, 128), (int64_t)s->n_sms * 8), 128, 0, cb_count(st)>>>(A);
-    // persistent warps: at most three 128-thread blocks per SM (the kernel's registers)
-    k_ccd_exact<<<std::min<int64_t>(cb_grid(np, 128), (int64_t)s->n_sms * 3), 128, 0, cb_count(st)>>>(
-        A, (unsigned long long*)(sc + SC_FETCH));
+    // persistent warps: at most three 128-thread blocks per SM (the kernel's registers); a block has eight half-warps
+    k_ccd_exact<<<std::min<int64_t>(cb_grid(np, 8), (int64_t)s->n_sms * 3), 128, 0, cb_count(st)>>>(
+        A, (unsigned long long*)(sc + SC_FETCH), s->n_sms);
     CB_CUDA(cudaGetLastError());
   }
   if (alpha) k_alpha_final<<<cb_grid(M), CB_THREADS, 0, cb_count(st)>>>(M, macc, alpha);
@@ -715,11 +785,61 @@ __device__ double na_iterate(const NaArgs& A, int64_t q) {
   return t;
 }
 
+// a short list: half a warp per stencil (accd16.cuh)
+struct NaJob {
+  const NaArgs& A;
+  int64_t mf;
+  int64_t q;
+
+  __device__ __forceinline__ bool bad() const {
+    if (cba::half_leader()) atomicOr(&A.scr[NA_FLAGS], (unsigned long long)CB_NOALLOC_BAD_STENCIL);
+    return false;
+  }
+  __device__ __forceinline__ bool take(int64_t w, cba::Pair16& S) {
+    q = w < mf ? na_list(A)[w] : na_list(A)[A.ns - 1 - (w - mf)];
+    if (!(na_lb(A)[q] <= na_cap(A))) return false;
+    // (listed: its vertex ids and offset are in order)
+    const int v = A.st[4 * q + cba::quad_vertex()];
+    S.off = A.off[q];
+    return cba::load16(A.x, A.p, A.n, v, A.ee[q] != 0, S) || bad();
+  }
+  __device__ __forceinline__ bool begin(cba::Pair16& S, double d) {
+    const double g0 = S.lp != 0.0 ? xsub(d, S.off) : 0.0;
+    if (!isfinite(d) || !isfinite(S.lp) || !isfinite(g0)) return bad();
+    if (S.lp == 0.0) return false;
+    if (g0 <= 0.0) {
+      if (cba::half_leader()) atomicOr(&A.scr[NA_FLAGS], (unsigned long long)CB_DEV_PENETRATION);
+      done(S, 0.0, cba::REACHED);
+      return false;
+    }
+    S.hi = __longlong_as_double(A.scr[NA_HI]);  // no longer moves
+    S.cap = cap(S);
+    S.g = xmul(ACCD_S, g0);
+    S.tl = xdiv(xmul(xsub(1.0, ACCD_S), g0), S.lp);
+    return true;
+  }
+  __device__ __forceinline__ double cap(const cba::Pair16&) const {
+    return __longlong_as_double(*(const volatile unsigned long long*)&A.scr[NA_ALPHA]);
+  }
+  __device__ __forceinline__ void done(const cba::Pair16&, double t, cba::Done how) const {
+    if (!cba::half_leader()) return;
+    if (how == cba::LIMIT) atomicOr(&A.scr[NA_FLAGS], (unsigned long long)CB_DEV_ITER_LIMIT);
+    if (how != cba::STOPPED && t < 1.0) atomicMin(&A.scr[NA_ALPHA], (unsigned long long)__double_as_longlong(t));
+  }
+};
+
 // the listed stencils whose lower bound is still not above the bound; every
 // other stencil has t_p above it, so alpha = min(1, m) exactly
-__global__ void __launch_bounds__(128) k_na_exact(NaArgs A) {
+__global__ void __launch_bounds__(128) k_na_exact(NaArgs A, int sms) {
   const unsigned int* cnt = (const unsigned int*)&A.scr[NA_COUNT];
   const int64_t mf = min((int64_t)cnt[0], A.ns), m = min(mf + (int64_t)cnt[1], A.ns);
+  const int blocks = min((int)gridDim.x, sms);
+  if (m <= (int64_t)blocks * FEW_PER_BLOCK) {
+    if (blockIdx.x >= blocks) return;
+    NaJob J{A, mf, 0};
+    cba::iterate16(J, m, 4 * blocks, (int)(threadIdx.x >> 5) * blocks + (int)blockIdx.x, ACCD_C, ACCD_MAX_ITER);
+    return;
+  }
   for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < m; w += (int64_t)gridDim.x * blockDim.x) {
     const uint32_t q = w < mf ? na_list(A)[w] : na_list(A)[A.ns - 1 - (w - mf)];
     if (!(na_lb(A)[q] <= na_cap(A))) continue;
@@ -817,7 +937,7 @@ cb_status ccd_step_noalloc(const double* x_dev, const double* p_dev, int32_t n_v
     const int g32 = (int)std::min<int64_t>(g, (int64_t)nsm * 8);
     k_na_refine<<<g32, 128, 0, cb_count(st)>>>(A, 0);
     k_na_refine<<<g32, 128, 0, cb_count(st)>>>(A, 1);
-    k_na_exact<<<(int)std::min<int64_t>(g, (int64_t)nsm * 4), 128, 0, cb_count(st)>>>(A);
+    k_na_exact<<<(int)std::min<int64_t>(cb_grid(n_stencils, 8), (int64_t)nsm * 4), 128, 0, cb_count(st)>>>(A, nsm);
   }
   k_na_final<<<1, 32, 0, cb_count(st)>>>(scr, alpha_dev, flags_dev);
   CB_CUDA(cudaGetLastError());
