@@ -301,9 +301,11 @@ __global__ void k_distance_screen(int64_t nc, const uint64_t* __restrict__ cand,
 // formula (typed.cuh); the undecided few wait in shared memory until a block's
 // worth, or the rest, runs the full routine in full warps.  862k pairs of a
 // pleated sheet 458 -> 292 us, of 64 rod scenes 736 -> 326, the energy-only
-// pass of a 181x181 sheet 212 -> 113.
+// pass of a 181x181 sheet 212 -> 113.  One wave of resident blocks (three per SM,
+// 80 registers) instead of several of two per SM: each block ends with its
+// undecided pairs' long chain only once; 292 -> 170 us and 326 -> 278.
 template <bool ENERGY>
-__global__ void k_distance_exact(const uint32_t* __restrict__ list, int64_t cap, const unsigned int* __restrict__ nlist,
+__global__ void __launch_bounds__(CB_THREADS, 3) k_distance_exact(const uint32_t* __restrict__ list, int64_t cap, const unsigned int* __restrict__ nlist,
                                  const uint64_t* __restrict__ cand, const uint8_t* __restrict__ klass_in,
                                  const int32_t* __restrict__ ev0, const int32_t* __restrict__ ev1,
                                  const int32_t* __restrict__ tv, int T, const double* __restrict__ x, int n,
@@ -2138,7 +2140,7 @@ cb_status barrier_run(cb_scene* s, const double* x, double* energy, double* grad
         nc, bp<uint64_t>(s->cand), bp<uint8_t>(s->klass), bp<int32_t>(s->ev0), bp<int32_t>(s->ev1),
         bp<int32_t>(s->tv), s->T, bp<float4>(s->xf), bp<double>(s->bw.cx), bp<int32_t>(s->vsc),
         bp<MemberParams>(s->mp), s->n, bp<uint32_t>(s->dlist), nl);
-    (energy_only ? k_distance_exact<true> : k_distance_exact<false>)<<<std::min<int64_t>(cb_grid(nc), (int64_t)s->n_sms * 16), CB_THREADS, 0, cb_count(st)>>>(
+    (energy_only ? k_distance_exact<true> : k_distance_exact<false>)<<<std::min<int64_t>(cb_grid(nc), (int64_t)s->n_sms * 3), CB_THREADS, 0, cb_count(st)>>>(
         bp<uint32_t>(s->dlist), nc, nl, bp<uint64_t>(s->cand), bp<uint8_t>(s->klass), bp<int32_t>(s->ev0),
         bp<int32_t>(s->ev1), bp<int32_t>(s->tv), s->T, x, s->n, bp<int32_t>(s->vsc), bp<MemberParams>(s->mp),
         bp<double>(s->cd), bp<int8_t>(s->ctype), bp<uint8_t>(s->ccls), bp<uint32_t>(s->clist), bp<uint32_t>(s->aidx),
