@@ -601,55 +601,92 @@ __device__ __forceinline__ void sort_segment(uint32_t* p, unsigned len, unsigned
   }
 }
 
-constexpr unsigned ROW_MAX = 512;  // bucket entries a warp sorts in shared memory
-constexpr int ROW_WARPS = 8;
+constexpr unsigned ROW_MAX = 512;  // bucket entries a warp takes in shared memory
+constexpr int ROW_WARPS = 4;
 
-// a warp per row: its bucket sorted and made distinct in place, the count to
-// uniq; longer buckets are listed for k_row_unique_long
-__global__ void __launch_bounds__(32 * ROW_WARPS) k_row_unique(int n, const uint32_t* __restrict__ off,
+// distinct values of 32 lanes (~0: none), ascending, to out; returns their number
+__device__ __forceinline__ unsigned row_sort32(uint32_t v, int lane, uint32_t* __restrict__ out) {
+  const unsigned full = 0xffffffffu;
+#pragma unroll
+  for (int size = 2; size <= 32; size <<= 1)
+#pragma unroll
+    for (int half = size >> 1; half > 0; half >>= 1) {
+      const int o = half == size >> 1 ? size - 1 : half;
+      const uint32_t u = __shfl_xor_sync(full, v, o);
+      v = (lane & half) ? max(u, v) : min(u, v);
+    }
+  const uint32_t before = __shfl_up_sync(full, v, 1);
+  const bool keep = v != full && (lane == 0 || v != before);
+  const unsigned m = __ballot_sync(full, keep);
+  if (keep) out[__popc(m & ((1u << lane) - 1u))] = v;
+  return (unsigned)__popc(m);
+}
+
+// A warp per row, or per 8 rows where that still fills the chip (rows may be
+// mostly empty): the bucket made distinct and sorted in place, the count to
+// uniq; longer buckets are listed for k_row_unique_long.  Bound by instruction
+// issue, so the many duplicates (a bucket holds its row's columns two to three
+// times over) go first, through an open-addressing set at most half full, and
+// only the distinct columns are sorted -- in registers where 32 lanes hold
+// them.  A pleated 256x256 pass 235 -> 84 us (a warp sorting each whole bucket in
+// shared memory before), two stacked layers 31 -> 15, 64 rod scenes 193 -> 145.
+__global__ void __launch_bounds__(32 * ROW_WARPS) k_row_unique(int n, int per, const uint32_t* __restrict__ off,
                                                                uint32_t* __restrict__ rcol, uint32_t* __restrict__ uniq,
                                                                uint32_t* __restrict__ longs,
                                                                unsigned int* __restrict__ nlong) {
+  __shared__ uint4 set4[ROW_WARPS][2 * ROW_MAX / 4];
   __shared__ uint32_t buf[ROW_WARPS][ROW_MAX];
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  const int r = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  if (r >= n) return;
-  const uint32_t b = off[r], len = off[r + 1] - b;
-  if (len > ROW_MAX) {
-    if (lane == 0) longs[atomicAdd(nlong, 1u)] = (uint32_t)r;
-    return;
-  }
-  if (len <= 32) {
-    uint32_t v = lane < (int)len ? rcol[b + lane] : full;
-#pragma unroll
-    for (int size = 2; size <= 32; size <<= 1)
-#pragma unroll
-      for (int half = size >> 1; half > 0; half >>= 1) {
-        const int o = half == size >> 1 ? size - 1 : half;
-        const uint32_t u = __shfl_xor_sync(full, v, o);
-        v = (lane & half) ? max(u, v) : min(u, v);
-      }
-    const uint32_t before = __shfl_up_sync(full, v, 1);
-    const bool keep = lane < (int)len && (lane == 0 || v != before);
-    const unsigned m = __ballot_sync(full, keep);
-    if (keep) rcol[b + __popc(m & ((1u << lane) - 1u))] = v;
-    if (lane == 0) uniq[r] = (uint32_t)__popc(m);
-    return;
-  }
+  uint32_t* set = (uint32_t*)set4[threadIdx.x >> 5];
   uint32_t* p = buf[threadIdx.x >> 5];
-  for (unsigned i = lane; i < len; i += 32) p[i] = rcol[b + i];
-  __syncwarp();
-  sort_segment(p, len, lane, 32, [] { __syncwarp(); });
-  unsigned at = 0;
-  for (unsigned i0 = 0; i0 < len; i0 += 32) {
-    const unsigned i = i0 + lane;
-    const bool keep = i < len && (i == 0 || p[i] != p[i - 1]);
-    const unsigned m = __ballot_sync(full, keep);
-    if (keep) rcol[b + at + __popc(m & ((1u << lane) - 1u))] = p[i];
-    at += (unsigned)__popc(m);
+  const int64_t r0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per;
+  const uint32_t first = off[min(r0 + lane, (int64_t)n)];
+  const uint32_t mine = __shfl_down_sync(full, first, 1) - first;
+  if (lane < per && r0 + lane < n && mine == 0) uniq[r0 + lane] = 0;
+  for (unsigned todo = __ballot_sync(full, lane < per && r0 + lane < n && mine > 0); todo; todo &= todo - 1u) {
+    const int q = __ffs((int)todo) - 1;
+    const int64_t r = r0 + q;
+    const uint32_t b = __shfl_sync(full, first, q), len = __shfl_sync(full, mine, q);
+    if (len > ROW_MAX) {
+      if (lane == 0) longs[atomicAdd(nlong, 1u)] = (uint32_t)r;
+      continue;
+    }
+    if (len <= 32) {
+      const unsigned m = row_sort32(lane < (int)len ? rcol[b + lane] : full, lane, rcol + b);
+      if (lane == 0) uniq[r] = m;
+      continue;
+    }
+    __syncwarp();  // the last row's reads are over
+    const int bits = 33 - __clz(len - 1);  // 2^bits >= 2 len
+    for (int i = lane; i < 1 << (bits - 2); i += 32) set4[threadIdx.x >> 5][i] = make_uint4(full, full, full, full);
+    __syncwarp();
+    unsigned nu = 0;
+    for (unsigned i0 = 0; i0 < len; i0 += 32) {
+      const unsigned i = i0 + lane;
+      bool fresh = false;
+      uint32_t v = full;
+      if (i < len) {
+        v = rcol[b + i];
+        for (unsigned h = v * 2654435769u >> (32 - bits);; h = (h + 1) & ((1u << bits) - 1u)) {  // ends: half the slots are free
+          const uint32_t u = atomicCAS(&set[h], full, v);
+          fresh = u == full;
+          if (fresh || u == v) break;
+        }
+      }
+      const unsigned m = __ballot_sync(full, fresh);
+      if (fresh) p[nu + __popc(m & ((1u << lane) - 1u))] = v;
+      nu += (unsigned)__popc(m);
+    }
+    __syncwarp();
+    if (nu <= 32) {
+      row_sort32(lane < (int)nu ? p[lane] : full, lane, rcol + b);
+    } else {
+      sort_segment(p, nu, lane, 32, [] { __syncwarp(); });
+      for (unsigned i = lane; i < nu; i += 32) rcol[b + i] = p[i];
+    }
+    if (lane == 0) uniq[r] = nu;
   }
-  if (lane == 0) uniq[r] = at;
 }
 
 // ... a block per long bucket, in global memory
@@ -681,14 +718,16 @@ __global__ void __launch_bounds__(cbp::SCAN_T) k_row_unique_long(const uint32_t*
   }
 }
 
-// the rows' distinct columns to their place
+// the rows' distinct columns to their place, 8 lanes a row (a full warp left most lanes without work: 64 rod scenes
+// with 1.1M rows 142 -> 46 us)
 __global__ void k_row_write(int n, const uint32_t* __restrict__ off, const uint32_t* __restrict__ rcol,
                             const int32_t* __restrict__ row_ptr, int32_t* __restrict__ col) {
-  const int r = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  const int r = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3);
   if (r >= n) return;
-  const uint32_t b = off[r];
   const int o = row_ptr[r], c = row_ptr[r + 1] - o;
-  for (int i = threadIdx.x & 31; i < c; i += 32) col[o + i] = (int32_t)rcol[b + i];
+  if (c == 0) return;
+  const uint32_t b = off[r];
+  for (int i = threadIdx.x & 7; i < c; i += 8) col[o + i] = (int32_t)rcol[b + i];
 }
 
 // Distance types as difference vectors z_m = sum_i C[m][i] x_i (m <= kind):
@@ -2184,8 +2223,9 @@ cb_status barrier_run(cb_scene* s, const double* x, double* energy, double* grad
     cbp::exclusive_scan<uint32_t, uint32_t>(cnt, off, (int64_t)n + 1, bp<uint32_t>(s->scan_tmp), (uint32_t*)nullptr, st);
     k_row_fill<<<(int)std::min<int64_t>(cb_grid((int64_t)m), (int64_t)s->n_sms * 16), CB_THREADS, 0, cb_count(st)>>>(
         bp<uint2>(s->bkey), nbk, off, cursor, bp<uint32_t>(s->rcol));
-    k_row_unique<<<cb_grid((int64_t)n * 32, 32 * ROW_WARPS), 32 * ROW_WARPS, 0, cb_count(st)>>>(
-        n, off, bp<uint32_t>(s->rcol), uniq, longs, nlong);
+    const int per = n >= s->n_sms * 64 * 8 ? 8 : 1;
+    k_row_unique<<<cb_grid(((int64_t)n + per - 1) / per * 32, 32 * ROW_WARPS), 32 * ROW_WARPS, 0, cb_count(st)>>>(
+        n, per, off, bp<uint32_t>(s->rcol), uniq, longs, nlong);
     k_row_unique_long<<<s->n_sms, cbp::SCAN_T, 0, cb_count(st)>>>(off, bp<uint32_t>(s->rcol), uniq, longs, nlong);
     // uniq[n] = 0: the scan's last entry is the block count
     uint32_t* tot = (uint32_t*)(sc + SC_COUNT1);
@@ -2198,7 +2238,7 @@ cb_status barrier_run(cb_scene* s, const double* x, double* energy, double* grad
     CB_TRY(buf_ensure(s->bsr_col, sizeof(int32_t) * (size_t)s->nnzb, st));
     CB_TRY(buf_ensure(s->bsr_val, sizeof(double) * 9 * (size_t)s->nnzb, st));
     CB_CUDA(cudaMemsetAsync(s->bsr_val.p, 0, sizeof(double) * 9 * (size_t)s->nnzb, st));
-    k_row_write<<<cb_grid((int64_t)n * 32), CB_THREADS, 0, cb_count(st)>>>(n, off, bp<uint32_t>(s->rcol),
+    k_row_write<<<cb_grid((int64_t)n * 8), CB_THREADS, 0, cb_count(st)>>>(n, off, bp<uint32_t>(s->rcol),
                                                                           bp<int32_t>(s->bsr_row),
                                                                           bp<int32_t>(s->bsr_col));
     HessArgs A;
