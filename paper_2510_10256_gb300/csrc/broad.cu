@@ -51,18 +51,6 @@ __device__ __forceinline__ float o2f(uint32_t o) {
   return __uint_as_float((o & 0x80000000u) ? (o & 0x7fffffffu) : ~o);
 }
 
-// the IEEE-754 neighbours of a float towards +inf and -inf, from its bit
-// pattern (a float's successor is the next integer bit pattern for x >= +0
-// and the previous one for x < 0; -0 steps to the smallest subnormal; +inf
-// and -inf stay where they are)
-__device__ __forceinline__ float nextup(float v) {
-  const int u = __float_as_int(v);
-  if (u == (int)0x80000000) return __int_as_float(1);
-  if (u == 0x7f800000) return v;
-  return __int_as_float(u >= 0 ? u + 1 : u - 1);
-}
-__device__ __forceinline__ float nextdn(float v) { return -nextup(-v); }
-
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int CL = 32;  // primitives per cluster and clusters per supercluster: a warp's lanes
 
@@ -310,107 +298,168 @@ __device__ __noinline__ bool boxes64_overlap(const TileArgs& A, int4 a, int4 b, 
 
 constexpr int TILE_WARPS = 8;
 
+// (a.x + b.x, a.y + b.y) in one instruction
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  unsigned long long x, y, r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
+  asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+  float2 o;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(o.x), "=f"(o.y) : "l"(r));
+  return o;
+}
+// the smallest of three, NaN if any is
+__device__ __forceinline__ float min3(float a, float b, float c) {
+  float r;
+  asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+
+// A tile's column primitives, as the inner loop reads them
+struct TileColumns {
+  float4 a[CL];   // hi.x, -lo.x, hi.y, -lo.y
+  float4 b[CL];   // hi.z, -lo.z, and the first two vertices
+  int2 c[CL];     // the third vertex (rods: the component), the primitive
+  int2 w[CL];     // rods: the arc-length windows
+  uint16_t code[CL * CL];  // the tile's pairs: row << 5 | column, filtered << 10, culled << 11
+};
+
 // A warp per tile (grid-stride): lane r holds the row cluster's primitive r,
 // the column cluster's primitives lie in shared memory.  Columns whose box
-// misses the row cluster's are skipped for the whole warp; each other costs
-// three broadcast reads, twelve comparisons of the boxes (the plain and the
-// inward-moved test share the column's bounds: moving both sides one ulp
-// inward is moving the row's bound two) and the shared-vertex test.
-// Bound by instruction issue.
+// misses the row cluster's are skipped for the whole warp.  Bound by
+// instruction issue, so a column costs two wide broadcast reads, the six
+// differences of the boxes' bounds in three packed additions, their minimum
+// and two comparisons: its sign is the FP32 test (a rounded difference has the
+// exact one's sign), and above eps = 2^-21 of the row box's coordinates the
+// FP64 boxes, at most an ulp inside on each side, overlap too.  Between the two
+// (and for NaN) the FP64 boxes decide.  Each lane then writes its pairs' codes
+// to shared memory, and the warp turns them into keys 32 at a time.
+// Both broad phases of a pass, from twelve box comparisons a column and keys
+// written column by column, 80 registers and three blocks per SM: pleated
+// 256x256 509 -> 404 us, a 200k-triangle graded sheet 1,068 -> 837, 64 rod
+// scenes 950 -> 665 (the windows and components now come once per tile).
 // The pairs' classes come with them (Sec. 3.2): on shells the rest mesh's
 // filtered pairs are kept as one 32x32 bit mask per pair of clusters, so a
 // tile looks its mask up once and a pair's class is a bit; on rods they are the
 // arc-length windows of the two edges.  (A search of the sorted filtered keys
 // per candidate, in contact_filter and again in the CCD screen, took 0.32 and
 // about 0.2 ms of a pleated 256x256 pass, 0.56 and 0.4 ms of a graded one.)
-__global__ void __launch_bounds__(32 * TILE_WARPS) k_tiles(TileArgs A) {
-  __shared__ float4 s_lo[TILE_WARPS][CL], s_hi[TILE_WARPS][CL];
-  __shared__ int4 s_v[TILE_WARPS][CL];
-  const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5;
-  const unsigned below = (1u << lane) - 1u;
+__global__ void __launch_bounds__(32 * TILE_WARPS, 3) k_tiles(TileArgs A) {
+  __shared__ TileColumns cols_of[TILE_WARPS];
+  const int lane = threadIdx.x & 31;
+  TileColumns& S = cols_of[threadIdx.x >> 5];
   const unsigned long long nt = *A.ntiles, m = nt < A.tile_cap ? nt : A.tile_cap;
   const unsigned long long nw = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
   unsigned n32 = 0, n64 = 0, dense = 0, nf = 0;
-  for (unsigned long long w = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < m; w += nw) {
-    const uint2 t = A.tiles[w];
+  unsigned long long w = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  uint2 next = w < m ? A.tiles[w] : make_uint2(0u, 0u);
+  for (; w < m; w += nw) {
+    const uint2 t = next;
+    if (w + nw < m) next = A.tiles[w + nw];
     const int64_t sr = (int64_t)t.x * CL + lane, sc = (int64_t)t.y * CL + lane;
     const Box a = load_box(A.box, sr), b = load_box(A.box, sc);
     const int4 va = A.slots[sr], vb = A.slots[sc];
     const uint32_t ci = A.cinfo[t.x];
-    const bool pt = (ci & 3u) == 0u && !A.rod, self = t.x == t.y;
+    const bool pt = (ci & 3u) == 0u && !A.rod;
+    const bool windows = A.rod && A.cls;
+    int mine = -1, win = 0, wst = 0;
     __syncwarp();  // the last tile's reads are over
-    s_lo[wb][lane] = b.lo;
-    s_hi[wb][lane] = b.hi;
-    s_v[wb][lane] = vb;
+    S.a[lane] = make_float4(b.hi.x, -b.lo.x, b.hi.y, -b.lo.y);
+    S.b[lane] = make_float4(b.hi.z, -b.lo.z, __int_as_float(vb.x), __int_as_float(vb.y));
+    S.c[lane] = make_int2(windows && vb.x >= 0 ? A.comp[vb.x] : vb.z, vb.w);
+    if (windows) {
+      if (vb.w >= 0) S.w[lane] = make_int2(A.win[vb.w], A.wst[vb.w]);
+      if (va.w >= 0) {
+        mine = A.comp[va.x];
+        win = A.win[va.w];
+        wst = A.wst[va.w];
+      }
+    }
     unsigned cols = __ballot_sync(FULL, overlap(load_box(A.cbox, t.x), b));
     __syncwarp();
-    const float lx = nextup(nextup(a.lo.x)), ly = nextup(nextup(a.lo.y)), lz = nextup(nextup(a.lo.z));
-    const float hx = nextdn(nextdn(a.hi.x)), hy = nextdn(nextdn(a.hi.y)), hz = nextdn(nextdn(a.hi.z));
-    unsigned hit = 0u;
-    for (; cols; cols &= cols - 1u) {
-      const int c = __ffs((int)cols) - 1;
-      const Box q{s_lo[wb][c], s_hi[wb][c]};
-      const int4 v = s_v[wb][c];
-      const bool ov = overlap(a, q);
-      const bool sure = lx <= q.hi.x && q.lo.x <= hx && ly <= q.hi.y && q.lo.y <= hy && lz <= q.hi.z && q.lo.z <= hz;
+    const float2 ax = make_float2(-a.lo.x, a.hi.x), ay = make_float2(-a.lo.y, a.hi.y), az = make_float2(-a.lo.z, a.hi.z);
+    const float eps = fmaf(fmaxf(fmaxf(fmaxf(fabsf(ax.x), fabsf(ax.y)), fmaxf(fabsf(ay.x), fabsf(ay.y))),
+                                 fmaxf(fabsf(az.x), fabsf(az.y))), 4.76837158e-7f, 1e-40f);
+    unsigned hit = 0u, sure = 0u;
+    auto test = [&](int c) {
+      const float4 qa = S.a[c], qb = S.b[c];
+      const int vx = __float_as_int(qb.z), vy = __float_as_int(qb.w);
+      const float2 dx = add2(make_float2(qa.x, qa.y), ax), dy = add2(make_float2(qa.z, qa.w), ay),
+                   dz = add2(make_float2(qb.x, qb.y), az);
+      const float d = min3(min3(dx.x, dx.y, dy.x), min3(dy.y, dz.x, dz.y), dz.y);
       // shared vertices: a point's against the triangle's three, an edge's two against the other's two
-      const bool inc = pt ? (va.x == v.x || va.x == v.y || va.x == v.z)
-                          : (va.x == v.x || va.x == v.y || va.y == v.x || va.y == v.y);
-      bool ok = ov && !inc && (!self || c > lane);
-      if (ok && !sure) {
-        ++n64;
-        ++n32;
-        ok = boxes64_overlap(A, va, v, ci);
-        n32 -= ok ? 1u : 0u;  // counted with the hits below
-      }
-      if (ok) hit |= 1u << c;
+      const bool inc = pt ? (va.x == vx || va.x == vy || va.x == S.c[c].x)
+                          : (va.x == vx || va.x == vy || va.y == vx || va.y == vy);
+      if (!(d < 0.f) && !inc) hit |= 1u << c;
+      if (d > eps) sure |= 1u << c;
+    };
+    while (cols) {  // two columns at a time: their reads overlap
+      const int c0 = __ffs((int)cols) - 1;
+      cols &= cols - 1u;
+      const int c1 = cols ? __ffs((int)cols) - 1 : c0;
+      cols &= cols - 1u;
+      test(c0);
+      test(c1);
+    }
+    if (t.x == t.y) hit &= lane < 31 ? FULL << (lane + 1) : 0u;
+    n32 += (unsigned)__popc(hit);
+    for (unsigned todo = hit & ~sure; todo; todo &= todo - 1u) {
+      const int c = __ffs((int)todo) - 1;
+      ++n64;
+      if (!boxes64_overlap(A, va, A.slots[(int64_t)t.y * CL + c], ci)) hit &= ~(1u << c);
     }
     const unsigned cnt = (unsigned)__popc(hit);
-    n32 += cnt;
     if (A.rod) dense += cnt > CL / 2 ? 1u : 0u;
-    const unsigned total = __reduce_add_sync(FULL, cnt);
+    unsigned at = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned u = __shfl_up_sync(FULL, at, o);
+      if (lane >= o) at += u;
+    }
+    const unsigned total = __shfl_sync(FULL, at, 31);
     if (total == 0) continue;
+    at -= cnt;
+    unsigned long long base = 0;
+    if (lane == 0) base = atomicAdd(A.total, (unsigned long long)total);
     unsigned filt = 0u, cull = 0u;
     if (A.cls) {
       const MemberParams& M = A.mp[ci >> 2];
       if (!A.rod) {
         if (!M.filter_off) filt = hit & A.fm.row(t.x, t.y, lane);
-      } else if (__any_sync(FULL, hit != 0u) && (!M.filter_off || M.cull_radius > 0)) {
-        const int mine = va.x >= 0 ? A.comp[va.x] : -1;
+      } else if (!M.filter_off || M.cull_radius > 0) {
         for (unsigned todo = hit; todo; todo &= todo - 1u) {
           const int c = __ffs((int)todo) - 1;
-          const int4 v = s_v[wb][c];
-          if (A.comp[v.x] != mine) continue;
-          const uint32_t i = (uint32_t)min(va.w, v.w), j = (uint32_t)max(va.w, v.w);
-          if (!M.filter_off && rod_filtered(A.win, A.wst, M.loops != 0, i, j)) filt |= 1u << c;
+          const int2 v = S.c[c], wc = S.w[c];
+          if (v.x != mine) continue;
+          const bool first = va.w < v.y;
+          const int i = first ? va.w : v.y, j = first ? v.y : va.w;
+          if (!M.filter_off && rod_filtered(first ? win : wc.x, first ? wst : wc.y, M.loops != 0, j)) filt |= 1u << c;
           // Kaldor culling: edges are numbered along each polyline, so the gap is j - i (the shorter way round a loop)
-          if (M.cull_radius > 0 && rod_gap(A.rloop, i, j) <= M.cull_radius) cull |= 1u << c;
+          if (M.cull_radius > 0 && rod_gap(A.rloop, (uint32_t)i, (uint32_t)j) <= M.cull_radius) cull |= 1u << c;
         }
       }
       nf += (unsigned)__popc(filt);
     }
-    unsigned long long base = 0;
-    if (lane == 0) base = atomicAdd(A.total, (unsigned long long)total);
+    for (unsigned todo = hit; todo; todo &= todo - 1u, ++at) {
+      const int c = __ffs((int)todo) - 1;
+      S.code[at] = (uint16_t)(lane << 5 | c | ((filt >> c) & 1u) << 10 | ((cull >> c) & 1u) << 11);
+    }
     base = __shfl_sync(FULL, base, 0);
     if (base + total > A.out_cap) continue;  // counted only: the caller grows the list and comes again
-    // column by column, so that the warp writes contiguous runs
+    __syncwarp();
     const uint32_t type = pt ? CB_KEY_PT : (A.rod ? CB_KEY_ROD_EE : CB_KEY_EE);
-    for (unsigned any = __reduce_or_sync(FULL, hit); any; any &= any - 1u) {
-      const int c = __ffs((int)any) - 1;
-      const unsigned rows = __ballot_sync(FULL, (hit >> c) & 1u);
-      if ((hit >> c) & 1u) {
-        uint32_t i = (uint32_t)va.w, j = (uint32_t)s_v[wb][c].w;
-        if (!pt && j < i) {  // edge-edge keys take the lower edge first
-          const uint32_t k = i;
-          i = j;
-          j = k;
-        }
-        const unsigned long long at = base + __popc(rows & below);
-        if (A.cls) A.cls[at] = (cull >> c) & 1u ? (uint8_t)3 : (uint8_t)((filt >> c) & 1u);
-        A.out[at] = A.canonical ? cb_key(type, i, j)
-                                : (((uint64_t)type << (A.bi + A.bj)) | ((uint64_t)i << A.bj) | j);
+    for (unsigned k0 = 0; k0 < total; k0 += 32) {
+      const unsigned k = k0 + lane, e = S.code[min(k, total - 1u)];
+      uint32_t i = (uint32_t)__shfl_sync(FULL, va.w, (int)(e >> 5 & 31u)), j = (uint32_t)S.c[e & 31u].y;
+      if (k >= total) continue;
+      if (!pt && j < i) {  // edge-edge keys take the lower edge first
+        const uint32_t u = i;
+        i = j;
+        j = u;
       }
-      base += __popc(rows);
+      if (A.cls) A.cls[base + k] = e >> 11 & 1u ? (uint8_t)3 : (uint8_t)(e >> 10 & 1u);
+      A.out[base + k] = A.canonical ? cb_key(type, i, j)
+                                    : (((uint64_t)type << (A.bi + A.bj)) | ((uint64_t)i << A.bj) | j);
     }
   }
   if (A.fpstat) {
@@ -774,7 +823,7 @@ cb_status broad_phase(cb_scene* s, BroadWork& w, const double* x, const double* 
     A.out_cap = (unsigned long long)(list.bytes / sizeof(uint64_t));
     A.cls = cls ? bp<uint8_t>(*cls) : nullptr;
     if (cls) A.out_cap = std::min<unsigned long long>(A.out_cap, cls->bytes);
-    k_tiles<<<s->n_sms * 6, 32 * TILE_WARPS, 0, cb_count(st)>>>(A);
+    k_tiles<<<s->n_sms * 3, 32 * TILE_WARPS, 0, cb_count(st)>>>(A);
     CB_CUDA(cudaGetLastError());
     CB_TRY(read_scalars(s, SC_COUNT0, 2, h, st));
     find = h[0] > A.tile_cap;

@@ -40,15 +40,11 @@ struct FilterMasks {
 };
 
 // Rods: edges ki < kj of one polyline are filtered when kj is within the
-// forward window of ki (kj <= win[ki]) or, on a closed loop, within its
-// backward window (kj >= wst[ki] >= 0: the gap the other way round is below
-// the activation).  loops: the member has closed loops (else wst is not read).
-__device__ __forceinline__ bool rod_filtered(const int32_t* __restrict__ win, const int32_t* __restrict__ wst,
-                                             bool loops, uint32_t ki, uint32_t kj) {
-  if ((int)kj <= win[ki]) return true;
-  if (!loops) return false;
-  const int w = wst[ki];
-  return w >= 0 && (int)kj >= w;
+// forward window of ki (kj <= win) or, on a closed loop, within its
+// backward window (kj >= wst >= 0: the gap the other way round is below
+// the activation).  loops: the member has closed loops (else wst is not used).
+__device__ __forceinline__ bool rod_filtered(int win, int wst, bool loops, int kj) {
+  return kj <= win || (loops && wst >= 0 && kj >= wst);
 }
 
 // Rods: the index gap of edges ki < kj of one polyline (Kaldor culling);
