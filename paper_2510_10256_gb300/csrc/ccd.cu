@@ -236,11 +236,11 @@ __global__ void __launch_bounds__(128) k_ccd_screen(CcdArgs A, uint32_t* __restr
         const cbb::f3 p0 = ldf(A.pf, A.n, v[0]), p1 = ldf(A.pf, A.n, v[1]), p2 = ldf(A.pf, A.n, v[2]),
                       p3 = ldf(A.pf, A.n, v[3]);
         const cbb::f3 pm = cbb::fscale3(cbb::fadd3(cbb::fadd3(p0, p1), cbb::fadd3(p2, p3)), 0.25f);
-        const float n0 = sqrtf(cbb::fdot3(cbb::fsub3(p0, pm), cbb::fsub3(p0, pm)));
-        const float n1 = sqrtf(cbb::fdot3(cbb::fsub3(p1, pm), cbb::fsub3(p1, pm)));
-        const float n2 = sqrtf(cbb::fdot3(cbb::fsub3(p2, pm), cbb::fsub3(p2, pm)));
-        const float n3 = sqrtf(cbb::fdot3(cbb::fsub3(p3, pm), cbb::fsub3(p3, pm)));
-        const float lp32 = ee ? fmaxf(n0, n1) + fmaxf(n2, n3) : n0 + fmaxf(fmaxf(n1, n2), n3);
+        const cbb::f3 r0 = cbb::fsub3(p0, pm), r1 = cbb::fsub3(p1, pm), r2 = cbb::fsub3(p2, pm), r3 = cbb::fsub3(p3, pm);
+        const float m0 = cbb::fdot3(r0, r0), m1 = cbb::fdot3(r1, r1), m2 = cbb::fdot3(r2, r2), m3 = cbb::fdot3(r3, r3);
+        // (the root of the larger square is the larger root)
+        const float lp32 = ee ? cbb::qsqrt(fmaxf(m0, m1)) + cbb::qsqrt(fmaxf(m2, m3))
+                              : cbb::qsqrt(m0) + cbb::qsqrt(fmaxf(fmaxf(m1, m2), m3));
         const float Pm = fmaxf(fmaxf(cbb::fmaxabs3(p0), cbb::fmaxabs3(p1)), fmaxf(cbb::fmaxabs3(p2), cbb::fmaxabs3(p3)));
         const float u64 = 3.8146973e-6f;  // 64 u, u = 2^-24: exact
         const float lp_ub = __fadd_ru(__fmul_ru(lp32, 1.f + u64), __fmul_ru(u64, Pm));
@@ -301,8 +301,10 @@ __device__ __forceinline__ float member_cap(const CcdArgs& A, int mem) {
 }
 
 // pass 2: FP32 brackets of the unresolved pairs (grid-stride; the trip count
-// is uniform over a warp so that every lane reaches the appends)
-__global__ void __launch_bounds__(128) k_ccd_refine(CcdArgs A) {
+// is uniform over a warp so that every lane reaches the appends).  Bound by the
+// latency of each pair's chain of steps: 80 registers let six blocks share an SM
+// instead of five (pleated 256x256 174 -> 150 us; at eight the spills cost more)
+__global__ void __launch_bounds__(128, 6) k_ccd_refine(CcdArgs A) {
   const int64_t nu = min((int64_t)*A.nu, A.np);
   for (int64_t w0 = (int64_t)blockIdx.x * blockDim.x; w0 < nu; w0 += (int64_t)gridDim.x * blockDim.x) {
     const int64_t w = w0 + threadIdx.x;
@@ -594,7 +596,7 @@ cb_status ccd_run(cb_scene* s, const double* x, const double* p, double* alpha, 
     k_ccd_screen<<<cb_grid(np, 128), 128, 0, cb_count(st)>>>(A, bp<uint32_t>(s->dlist), nl);
     k_ccd_bound<<<std::min<int64_t>(cb_grid(np, 128), (int64_t)s->n_sms * 16), 128, 0, cb_count(st)>>>(
         A, bp<uint32_t>(s->dlist), nl);
-    k_ccd_refine<<<std::min<int64_t>(cb_grid(np, 128), (int64_t)s->n_sms * 8), 128, 0, cb_count(st)>>>(A);
+    k_ccd_refine<<<std::min<int64_t>(cb_grid(np, 128), (int64_t)s->n_sms * 16), 128, 0, cb_count(st)>>>(A);
     // persistent warps: at most three 128-thread blocks per SM (the kernel's registers); a block has eight half-warps
     k_ccd_exact<<<std::min<int64_t>(cb_grid(np, 8), (int64_t)s->n_sms * 3), 128, 0, cb_count(st)>>>(
         A, (unsigned long long*)(sc + SC_FETCH), s->n_sms);
