@@ -371,7 +371,8 @@ __host__ __device__ __forceinline__ void plane_block(const PlaneBlocks& P, int p
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int j = 0; j < 3; ++j) blk[3 * i + j] = a * P.M0[s6[3 * i + j]] + l[i] * P.n[j] + P.n[i] * m[j];
+    for (int j = 0; j < 3; ++j)  // a diagonal block is symmetric: its lower triangle is copied
+      blk[3 * i + j] = p == r && j < i ? blk[3 * j + i] : a * P.M0[s6[3 * i + j]] + l[i] * P.n[j] + P.n[i] * m[j];
 }
 
 // Point-edge pair: q off the edge e0 e1, w = q - e0, u = e1 - e0; points in the order q, e0, e1.  Block (p, r) is
@@ -444,7 +445,13 @@ __host__ __device__ __forceinline__ void edge_block(const EdgeBlocks& P, int p, 
   for (int j = 0; j < 3; ++j) {
     const double x = al * P.e[j] + be * P.n[j], y = ga * P.e[j] + P.sig[k] * P.n[j];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) blk[3 * i + j] = P.e[i] * x + P.n[i] * y;
+    for (int i = 0; i < 3; ++i)
+      if (p != r || i <= j) blk[3 * i + j] = P.e[i] * x + P.n[i] * y;
+  }
+  if (p == r) {  // symmetric
+    blk[3] = blk[1];
+    blk[6] = blk[2];
+    blk[7] = blk[5];
   }
 }
 
