@@ -438,10 +438,8 @@ __global__ void k_to_f32(int n, const double* __restrict__ v, const double* __re
 // and each row's short bucket is sorted and made distinct by a warp
 // (k_row_unique; a block for buckets past ROW_MAX, k_row_unique_long).  On a
 // pleated 256x256 pass (862k active pairs, 1.7M blocks) the keys take 0.11 ms,
-// fill, unique and write 0.38; a set of 4,096 keys per run and a radix sort of
-// the survivors (five digits) with its flags and scans took 0.18 and 0.75 (the
-// whole barrier pass 2.79 -> 2.38 ms; 64 rod scenes 3.40 -> 3.06, a chain of
-// 2,000 loops 0.68 -> 0.54, a woven patch 0.28 -> 0.20).
+// fill, unique and write 0.16; a set of 4,096 keys per run and a radix sort of
+// the survivors (five digits) with its flags and scans took 0.18 and 0.75.
 //
 // A run of active pairs (in candidate order, i.e. tile by tile) shares most of
 // its vertices, so its 4 x BK_PAIRS vertices become few local numbers through
@@ -563,13 +561,27 @@ __global__ void __launch_bounds__(BK_PAIRS) k_block_keys(ActiveList act, const u
   }
 }
 
-// the columns of the keys into their rows' buckets
+// The columns of the keys into their rows' buckets.  A run's keys of one row
+// are neighbours, so one lane reserves the places of all of a row's keys in its
+// warp: an atomic with a returned value per key, to places scattered over the
+// buckets, had bound the kernel (pleated 256x256 124 -> 64 us, 64 rod scenes
+// 96 -> 50, two stacked layers 25 -> 7).
 __global__ void k_row_fill(const uint2* __restrict__ bkey, const unsigned int* __restrict__ m_in,
                            const uint32_t* __restrict__ off, uint32_t* __restrict__ cursor, uint32_t* __restrict__ rcol) {
+  const unsigned full = 0xffffffffu;
   const int64_t m = *m_in;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-    const uint2 k = bkey[i];
-    rcol[off[k.x] + atomicAdd(&cursor[k.x], 1u)] = k.y;
+  const int lane = threadIdx.x & 31;
+  for (int64_t w0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; w0 < m; w0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = w0 + lane;
+    const uint2 k = i < m ? bkey[i] : make_uint2(full, 0u);
+    const uint32_t before = __shfl_up_sync(full, k.x, 1);
+    const unsigned heads = __ballot_sync(full, lane == 0 || before != k.x);
+    const int head = 31 - __clz((int)(heads & (full >> (31 - lane))));
+    const unsigned rest = heads & ~(full >> (31 - lane));
+    uint32_t at = 0;
+    if (head == lane && i < m) at = off[k.x] + atomicAdd(&cursor[k.x], (unsigned)((rest ? __ffs((int)rest) - 1 : 32) - lane));
+    at = __shfl_sync(full, at, head);
+    if (i < m) rcol[at + (uint32_t)(lane - head)] = k.y;
   }
 }
 
@@ -1928,11 +1940,6 @@ __global__ void k_energy_final(int count, const unsigned long long* __restrict__
   double e = __longlong_as_double(macc[(size_t)m * MACC_STRIDE + MACC_E]);
   if (macc[(size_t)m * MACC_STRIDE + MACC_STATUS] & CB_DEV_PENETRATION) e = __longlong_as_double(0x7ff0000000000000LL);
   out[m] = e;
-}
-
-__global__ void k_macc_reset(int count, unsigned long long* __restrict__ macc, int slot, unsigned long long v) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m < count) macc[(size_t)m * MACC_STRIDE + slot] = v;
 }
 
 __global__ void k_set_u64(unsigned long long* p, unsigned long long v) { *p = v; }
