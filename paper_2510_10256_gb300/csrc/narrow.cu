@@ -1190,8 +1190,9 @@ __device__ void ee_distance_derivs(int ty, const d3 (&X)[4], double d, LocalDeri
                         0.75 * g * r5 * Nd.g[i] * Nd.g[j]);
 }
 
-// one thread per mollified pair (listed by k_distance_exact)
-__global__ void __launch_bounds__(128) k_moll_hess(HessArgs A) {
+// One thread per mollified pair (listed by k_distance_exact); bound by the latency of its chain, so blocks of one
+// warp spread a short list over all SMs (10,231 pairs: 576 us in blocks of 128, 365 in blocks of 32)
+__global__ void __launch_bounds__(32) k_moll_hess(HessArgs A) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   double e_local = 0.0;
   int mem = -1;
@@ -2243,7 +2244,7 @@ cb_status barrier_run(cb_scene* s, const double* x, double* energy, double* grad
     CB_CUDA(cudaGetLastError());
     if (mollify) {
       // the queue's length stays on the device; a warp per pair while the queue is short
-      k_moll_hess<<<cb_grid(na, 128), 128, 0, cb_count(st)>>>(A);
+      k_moll_hess<<<cb_grid(na, 32), 32, 0, cb_count(st)>>>(A);
       if (na <= PL_MAX_ACTIVE) {
         const int smem = PL_SMEM * (int)sizeof(double) * PL_PAIRS;
         k_hess_proj_lanes<<<(int)((na + PL_PAIRS - 1) / PL_PAIRS), PL_THREADS, smem, cb_count(st)>>>(A);
