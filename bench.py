@@ -30,27 +30,27 @@ UNIT = "pairs/s"
 # FP64 peak from the part's unit counts and clock: 152 SMs x 2070 MHz x 4 FP64
 # flop/clk/SM (2 DFMA) = 1.26 TFLOP/s, the 1.25 TFLOP/s dense FP64 figure.
 FP64_PEAK_TFLOPS = 152 * 2.070e9 * 4 / 1e12
-# FP64 flop of the stage-(d) kernels per pair each one handles: DADD + DMUL +
-# 2 DFMA thread instructions executed, counted by ncu on the 128x128 pleated
-# sheet (195,263 active pairs: 30,807 face / line-line, 151,976 point-edge in
-# their frame) and divided by the pairs of each kernel.  k_hess_prep per
-# active pair, k_hess_proj<9> per face / line-line pair, k_hess_proj_pe per
-# point-edge pair in its own frame; k_hess_proj<6> (generic point-edge pairs,
-# none in that capture) is scaled from k_hess_proj<9> by (6/9)^3.
-HESS_FLOPS = {"prep": 549.1, "face": 11471.0, "pe_frame": 1091.0, "pe": 11471.0 * (6 / 9) ** 3}
-# DRAM bytes (read + write) of the stage-(d) kernels per active pair, from one
-# ncu capture of a full-size pass (256x256 sheet, 805,423 active pairs):
-# k_hess_prep 289.1 MB, k_hess_proj_pe 266.8 MB, k_hess_proj<9> 191.5 MB,
-# k_hess_proj<6> 0.1 MB
-HESS_DRAM_BYTES_PER_ACTIVE = 747.48e6 / 805423
-HESS_TRAFFIC_SOURCE = "ncu dram__bytes_read+write of the four stage-(d) kernels of one 256x256 pass, per active pair"
+# FP64 flop of the stage-(d) kernels per pair: DADD + DMUL + 2 DFMA thread
+# instructions executed, counted by ncu on a pleated 97x97 sheet, two stacked
+# layers, a woven patch and a chain of loops.  k_pair_hess: a base per pair and
+# a part more per face / line-line and per point-edge pair (the four counts give
+# the three numbers to 1e-4).  k_moll_hess + k_hess_proj: per mollified pair
+# (10,231 pairs of a pleated 128x128 sheet).
+HESS_FLOPS = {"pair": 173.0, "face": 1525.4, "pe": 407.0, "mollified": 21970.0}
+# DRAM bytes (read + write) of k_pair_hess per active pair, from one ncu
+# capture of a full-size pass (256x256 sheet, 861,805 active pairs: 391.9 MB
+# read, 138.0 MB written)
+HESS_DRAM_BYTES_PER_ACTIVE = 529.9e6 / 861805
+HESS_TRAFFIC_SOURCE = "ncu dram__bytes_read+write of k_pair_hess in one 256x256 pass, per active pair"
+HESS_KERNELS = "k_pair_hess (FP64 stage d; mollified pairs k_moll_hess + k_hess_proj)"
 
 
 def hess_flops(st) -> float:
-    """FP64 flop of one pass's stage-(d) kernels: per-kernel counts per pair
-    times the pairs each kernel handled."""
-    return (HESS_FLOPS["prep"] * st["n_active"] + HESS_FLOPS["face"] * st["n_hess_face"]
-            + HESS_FLOPS["pe_frame"] * st["n_hess_pe_frame"] + HESS_FLOPS["pe"] * st["n_hess_pe"])
+    """FP64 flop of one pass's stage-(d) kernels: counts per pair times the
+    pairs of each kind (mollified pairs are counted among the face pairs)."""
+    moll = st["n_mollified"]
+    return (HESS_FLOPS["pair"] * (st["n_active"] - moll) + HESS_FLOPS["face"] * (st["n_hess_face"] - moll)
+            + HESS_FLOPS["pe"] * (st["n_hess_pe_frame"] + st["n_hess_pe"]) + HESS_FLOPS["mollified"] * moll)
 L2_FLUSH_BYTES = 256 << 20
 
 
@@ -90,8 +90,9 @@ def stage_roofline(st: dict, med: list, scenes) -> dict:
     once, outputs written once; no hash, sort or re-gather traffic) over the
     stage's device time, against the measured HBM copy bandwidth; stage (d)
     also against the FP64 peak.  Bytes per stage:
-      a  24n + 12T + 8E + 8|C|          (positions, topology, candidate keys)
-      b  16|C| + table                  (keys in, classes out; rods 12E, shells 4|F_rest|)
+      a  24n + 12T + 8E + 9|C| + table  (positions, topology, the filter's table -- rods 12E, shells 4|F_rest| --
+                                         in; candidate keys and classes out)
+      b  16                             (two counters: the classes come with the candidates)
       cd 8|C| + 24n + 8|A| + 24n + 76 nnzb + 4(n+1)  (keys+x in; active, gradient, BSR out)
          of which c: 8|C| + 24n (keys, x in) and d: 8|A| + 24n + 76 nnzb + 4(n+1)
       e  8|C_ccd| + 48n + 8             (keys, x, p in; alpha out)"""
@@ -101,8 +102,8 @@ def stage_roofline(st: dict, med: list, scenes) -> dict:
     C, A, nnzb, Cc = st["n_candidates"], st["n_active"], st["nnzb"], st["n_ccd"]
     shell = scenes[0].kind == "shell"
     table = 4 * st["n_rest_filtered"] if shell else 12 * E
-    by = {"contact_build": 24 * n + 12 * T + 8 * E + 8 * C,
-          "contact_filter": 16 * C + table,
+    by = {"contact_build": 24 * n + 12 * T + 8 * E + 9 * C + table,
+          "contact_filter": 16,
           "barrier_eval": 8 * C + 24 * n + 8 * A + 24 * n + 76 * nnzb + 4 * (n + 1),
           "distances_c": 8 * C + 24 * n,
           "assembly_d": 8 * A + 24 * n + 76 * nnzb + 4 * (n + 1),
@@ -396,7 +397,7 @@ def bench_batch(args, rank, world, local, dist):
                                  "superset_ratio": st["n_candidates_fp32"] / max(1, n_cand),
                                  "fp64_decided": st["n_fp64_decided"]},
             "stage_ms": _stage_dict(med),
-            "roofline": {"bound": "alu", "kernel": "k_hess_prep + k_hess_proj<9> + k_hess_proj_pe (FP64 stage d)", "achieved": achieved,
+            "roofline": {"bound": "alu", "kernel": HESS_KERNELS, "achieved": achieved,
                          "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": achieved / FP64_PEAK_TFLOPS,
                          "traffic": None, "flops_per_pass": hess_flops(st), "kernel_ms": hess_ms,
                          "peak_source": "derived: 152 SM x 2070 MHz x 4 FP64 flop/clk/SM"},
@@ -891,7 +892,7 @@ def _single_line(args, r, world) -> dict:
         fp32_meas = CT.measure_fma_tflops(False, iters=65536)
     except Exception:
         fp64_meas = fp32_meas = None
-    roofline = {"bound": "alu", "kernel": "k_hess_prep + k_hess_proj<9> + k_hess_proj_pe (FP64 stage d)",
+    roofline = {"bound": "alu", "kernel": HESS_KERNELS,
                 "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": achieved / FP64_PEAK_TFLOPS,
                 "peak_fp64_fma_measured": fp64_meas, "peak_fp32_fma_measured": fp32_meas,
                 "traffic": HESS_DRAM_BYTES_PER_ACTIVE * na if HESS_DRAM_BYTES_PER_ACTIVE else None,

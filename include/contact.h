@@ -170,9 +170,9 @@ typedef struct {
   int64_t n_candidates_fp32;  /* last contact_build: non-incident pairs passing the FP32 box test
                                  (a superset of the candidates; the FP32 effect on |C| is this / n_candidates) */
   int64_t n_fp64_decided;     /* ... of which the FP32 test was not conclusive and the FP64 boxes decided */
-  int64_t n_hess_face;        /* last barrier_eval: active face / line-line pairs (9x9 projection) */
-  int64_t n_hess_pe_frame;    /* ... point-edge pairs projected in their own frame (3x3 + 2x2) */
-  int64_t n_hess_pe;          /* ... point-edge pairs on the generic 6x6 projection */
+  int64_t n_hess_face;        /* last barrier_eval: active face / line-line pairs, and mollified ones */
+  int64_t n_hess_pe_frame;    /* ... point-edge pairs, without */
+  int64_t n_hess_pe;          /* ... those nearly on their edge's line, |w| |u| > 64 |u x w| */
   int64_t n_pair_overflow;    /* last broad phase of a rod scene (ccd_step's, once a pass ran it): crowded rows --
                                  an edge against a cluster of 32 others with more than 16 of them its partners
                                  (shell scenes: 0) */
