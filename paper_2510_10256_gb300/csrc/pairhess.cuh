@@ -36,8 +36,8 @@
 // Measured on GB300, the Hessian kernels of one pass (from the derivatives and
 // an FP32 + FP64 Jacobi eigenproblem per pair, three kernels and their queues
 // in memory, to one kernel): pleated 256x256 sheet (862k active pairs, 153k of
-// them face / line-line) 5.56 -> 1.09 ms; 64 rod scenes (1.01M active, 243k)
-// 7.11 -> 1.56 ms; two 12x12 layers (9.6k, 577) 0.67 -> 0.08 ms, where one
+// them face / line-line) 5.56 -> 0.98 ms; 64 rod scenes (1.01M active, 243k)
+// 7.11 -> 1.36 ms; two 12x12 layers (9.6k, 577) 0.67 -> 0.09 ms, where one
 // thread's chain of Jacobi sweeps had set the time.  Against 40-digit results
 // the largest error of a face / line-line block, relative to its largest
 // entry, is 3 to 10 times below the eigenproblem's for edges at angles of

@@ -21,7 +21,8 @@
 // 97 % of a pleated sheet's active pairs are certain (regular meshes hold many
 // parallel edges), 99.9 % of a weave's and of stacked layers'.  The additive-CCD
 // iteration runs the rule at every step: 9,600 active pairs in layers 264 ->
-// 106 us, 64 rod scenes with up to 236 steps 2.03 -> 0.98 ms.
+// 106 us, 64 rod scenes with up to 236 steps 2.03 -> 0.98 ms (one lane a pair;
+// 68 us and 0.5 ms with half a warp, accd16.cuh).
 #pragma once
 #include "bound32.cuh"
 #include "geometry.cuh"
