@@ -24,6 +24,16 @@ __device__ __forceinline__ unsigned half_mask() { return 0xffffu << (threadIdx.x
 __device__ __forceinline__ int quad_vertex() { return (int)(threadIdx.x & 15u) >> 2; }
 __device__ __forceinline__ int quad_component() { return min((int)(threadIdx.x & 3u), 2); }
 __device__ __forceinline__ bool half_leader() { return (threadIdx.x & 15u) == 0; }
+// A value read by one lane of the half for all 16.  Other warps lower the
+// bounds of the smallest t_p while they are read, so lanes that read them for
+// themselves could see different values and part before a shuffle that names
+// them all; every branch on such a bound takes it from here.
+template <class Read>
+__device__ __forceinline__ auto half_read(Read read) -> decltype(read()) {
+  decltype(read()) v{};
+  if (half_leader()) v = read();
+  return __shfl_sync(half_mask(), v, 0, 16);
+}
 
 // One pair on its half-warp: component c of vertex v on each lane, the rest alike on all 16.
 struct Pair16 {
@@ -108,9 +118,12 @@ __device__ __forceinline__ bool load16(const double* __restrict__ x, const doubl
 __device__ __forceinline__ long long bits(double a) { return __double_as_longlong(a); }
 
 // The iteration over pairs [0, m), split evenly over the half-warps of `warps`
-// warps.  J.take(w, S) loads pair w (false: nothing to iterate), J.begin(S, d)
-// takes its first distance (false: finished), J.cap(S) reads the smallest t_p
-// found, J.done(S, t, how) ends a pair.  Returns the most steps of a pair.
+// warps.  J.wanted(w) compares pair w's lower bound with the bounds found so
+// far (1: not above them), J.load(w, S) loads it (false: nothing to iterate),
+// J.begin(S, d) takes its first distance (false: finished), J.cap() reads the
+// smallest t_p found, J.done(S, t, how) ends a pair.  wanted and cap read values that other warps write: half_read takes the leader's answer; the
+// rest of a pair is the same arithmetic on all 16 lanes.  Returns the most
+// steps of a pair.
 enum Done { REACHED, STOPPED, LIMIT };
 template <class Job>
 __device__ __forceinline__ int iterate16(Job& J, int64_t m, int warps, int warp, double c_step, int max_iter) {
@@ -123,7 +136,7 @@ __device__ __forceinline__ int iterate16(Job& J, int64_t m, int warps, int warp,
   bool have = false;
   int most = 0;
   for (;;) {
-    for (; !have && w < m; w += 2 * warps) have = J.take(w, S);
+    for (; !have && w < m; w += 2 * warps) have = half_read([&] { return J.wanted(w); }) && J.load(w, S);
     if (!__any_sync(FULL, have)) break;
     if (!S.first) S.y = xadd(S.y, xmul(S.tl, S.q));
     const double d = distance16(S, have);
@@ -132,6 +145,7 @@ __device__ __forceinline__ int iterate16(Job& J, int64_t m, int warps, int warp,
       S.t = 0.0;
       S.it = 0;
       have = J.begin(S, d);
+      if (have) S.cap = half_read([&] { return J.cap(); });
     } else if (have) {
       const int it = S.it++;
       const double gap = xsub(d, S.off);
@@ -145,7 +159,7 @@ __device__ __forceinline__ int iterate16(Job& J, int64_t m, int warps, int warp,
           J.done(S, 1.0, REACHED);
           have = false;
         } else {
-          if ((it & 7) == 7) S.cap = J.cap(S);
+          if ((it & 7) == 7) S.cap = half_read([&] { return J.cap(); });
           if (number && ((bits(S.cap) < bits(1.0) && bits(S.t) >= bits(S.cap)) || bits(S.t) > bits(S.hi))) {  // t_p >= t: this pair cannot lower the minimum
             J.done(S, S.t, STOPPED);
             have = false;

@@ -392,15 +392,23 @@ struct ExactJob {
   int64_t q;
   int mem, cls;
 
-  __device__ __forceinline__ bool take(int64_t w, cba::Pair16& S) {
-    q = w < mf ? A.list[w] : A.list[A.np - 1 - (w - mf)];
+  __device__ __forceinline__ int64_t pair(int64_t w) const { return w < mf ? A.list[w] : A.list[A.np - 1 - (w - mf)]; }
+  __device__ __forceinline__ int member(uint64_t key) const {
+    const uint32_t ki = cb_key_i(key);
+    return A.members > 1 ? A.vsc[cb_key_type(key) != CB_KEY_PT ? A.ev0[ki] : (int)ki] : 0;
+  }
+  __device__ __forceinline__ int wanted(int64_t w) const {
+    const int64_t k = pair(w);
+    return __double2float_rd(A.t_out[k]) <= member_cap(A, member(A.keys[k]));
+  }
+  __device__ __forceinline__ bool load(int64_t w, cba::Pair16& S) {
+    q = pair(w);
     const uint64_t key = A.keys[q];
     const uint32_t ki = cb_key_i(key), kj = cb_key_j(key);
     const bool ee = cb_key_type(key) != CB_KEY_PT;
     const int k = cba::quad_vertex();
+    mem = member(key);
     const int v0 = ee ? A.ev0[ki] : (int)ki;
-    mem = A.members > 1 ? A.vsc[v0] : 0;
-    if (!(__double2float_rd(A.t_out[q]) <= member_cap(A, mem))) return false;
     const uint32_t e = k < 2 ? ki : kj;
     const int v = ee ? (k & 1 ? A.ev1[e] : A.ev0[e]) : (k == 0 ? v0 : A.tv[(size_t)(k - 1) * A.T + kj]);
     cba::load16(A.x, A.p, A.n, v, ee, S);
@@ -420,13 +428,12 @@ struct ExactJob {
       done(S, S.lp == 0.0 ? 1.0 : 0.0, cba::REACHED);
       return false;
     }
-    S.hi = __longlong_as_double(*macc_of(A, mem, MACC_HI));
-    S.cap = cap(S);
+    S.hi = __longlong_as_double(*macc_of(A, mem, MACC_HI));  // no longer moves
     S.g = xmul(ACCD_S, g0);
     S.tl = xdiv(xmul(xsub(1.0, ACCD_S), g0), S.lp);
     return true;
   }
-  __device__ __forceinline__ double cap(const cba::Pair16&) const {
+  __device__ __forceinline__ double cap() const {
     return __longlong_as_double(*(volatile unsigned long long*)macc_of(A, mem, MACC_ALPHA));
   }
   __device__ __forceinline__ void done(const cba::Pair16&, double t, cba::Done how) const {
@@ -793,13 +800,14 @@ struct NaJob {
   int64_t mf;
   int64_t q;
 
+  __device__ __forceinline__ int64_t pair(int64_t w) const { return w < mf ? na_list(A)[w] : na_list(A)[A.ns - 1 - (w - mf)]; }
   __device__ __forceinline__ bool bad() const {
     if (cba::half_leader()) atomicOr(&A.scr[NA_FLAGS], (unsigned long long)CB_NOALLOC_BAD_STENCIL);
     return false;
   }
-  __device__ __forceinline__ bool take(int64_t w, cba::Pair16& S) {
-    q = w < mf ? na_list(A)[w] : na_list(A)[A.ns - 1 - (w - mf)];
-    if (!(na_lb(A)[q] <= na_cap(A))) return false;
+  __device__ __forceinline__ int wanted(int64_t w) const { return na_lb(A)[pair(w)] <= na_cap(A); }
+  __device__ __forceinline__ bool load(int64_t w, cba::Pair16& S) {
+    q = pair(w);
     // (listed: its vertex ids and offset are in order)
     const int v = A.st[4 * q + cba::quad_vertex()];
     S.off = A.off[q];
@@ -815,12 +823,11 @@ struct NaJob {
       return false;
     }
     S.hi = __longlong_as_double(A.scr[NA_HI]);  // no longer moves
-    S.cap = cap(S);
     S.g = xmul(ACCD_S, g0);
     S.tl = xdiv(xmul(xsub(1.0, ACCD_S), g0), S.lp);
     return true;
   }
-  __device__ __forceinline__ double cap(const cba::Pair16&) const {
+  __device__ __forceinline__ double cap() const {
     return __longlong_as_double(*(const volatile unsigned long long*)&A.scr[NA_ALPHA]);
   }
   __device__ __forceinline__ void done(const cba::Pair16&, double t, cba::Done how) const {
