@@ -294,9 +294,9 @@ __global__ void __launch_bounds__(32 * PAIR_WARPS) k_cluster_pairs(int nj, const
       unsigned mine = 0u;  // the columns of row `lane`
 #pragma unroll 8
       for (int r = 0; r < CL; ++r) {
-        unsigned m = __ballot_sync(FULL, overlap(rows[r], cb));
+        unsigned m = __ballot_sync(FULL, lane < C.y && overlap(rows[r], cb));
         if (J.x == col) m &= FULL << r;  // each pair of clusters once (and the cluster with itself)
-        if (lane == r) mine = m;
+        if (lane == r && r < R.y) mine = m;  // (an empty box's bounds do meet an infinite box's: the counts decide)
       }
       const unsigned cnt = (unsigned)__popc(mine);
       unsigned inc = cnt;
@@ -436,7 +436,8 @@ __global__ void __launch_bounds__(32 * TILE_WARPS, 3) k_tiles(TileArgs A) {
         wst = A.wst[va.w];
       }
     }
-    unsigned cols = __ballot_sync(FULL, overlap(load_box(A.cbox, t.x), b));
+    // empty slots take no part: a primitive reaching from -inf to +inf on every axis would meet even their empty boxes
+    unsigned cols = __ballot_sync(FULL, vb.w >= 0 && overlap(load_box(A.cbox, t.x), b));
     __syncwarp();
     const float2 ax = make_float2(-a.lo.x, a.hi.x), ay = make_float2(-a.lo.y, a.hi.y), az = make_float2(-a.lo.z, a.hi.z);
     const float eps = fmaf(fmaxf(fmaxf(fmaxf(fabsf(ax.x), fabsf(ax.y)), fmaxf(fabsf(ay.x), fabsf(ay.y))),
@@ -462,6 +463,7 @@ __global__ void __launch_bounds__(32 * TILE_WARPS, 3) k_tiles(TileArgs A) {
       test(c0);
       test(c1);
     }
+    if (va.w < 0) hit = 0u;
     if (t.x == t.y) hit &= lane < 31 ? FULL << (lane + 1) : 0u;
     n32 += (unsigned)__popc(hit);
     for (unsigned todo = hit & ~sure; todo; todo &= todo - 1u) {
