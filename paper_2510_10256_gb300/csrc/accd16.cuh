@@ -114,8 +114,10 @@ __device__ __forceinline__ bool load16(const double* __restrict__ x, const doubl
 }
 
 // FP64 values as integers of the same order, for comparisons off the FP64 pipe: t, the bounds and g are not
-// negative (a negative gap compares below them as it should), and NaN lies above infinity
+// negative, and a negative gap compares below them as it should.  NaN has no place in that order (its sign may be
+// set): a comparison that must be false for it asks number() as well.
 __device__ __forceinline__ long long bits(double a) { return __double_as_longlong(a); }
+__device__ __forceinline__ bool number(double a) { return (bits(a) & 0x7fffffffffffffffll) <= 0x7ff0000000000000ll; }
 
 // The iteration over pairs [0, m), split evenly over the half-warps of `warps`
 // warps.  J.wanted(w) compares pair w's lower bound with the bounds found so
@@ -149,18 +151,18 @@ __device__ __forceinline__ int iterate16(Job& J, int64_t m, int warps, int warp,
     } else if (have) {
       const int it = S.it++;
       const double gap = xsub(d, S.off);
-      if (bits(S.t) > 0 && bits(gap) < bits(S.g)) {
+      if (bits(S.t) > 0 && bits(gap) < bits(S.g) && number(gap)) {
         J.done(S, S.t, REACHED);
         have = false;
       } else {
         S.t = xadd(S.t, S.tl);
-        const bool number = bits(S.t) <= 0x7ff0000000000000ll;
-        if (number && bits(S.t) > bits(1.0)) {
+        const bool some = number(S.t);
+        if (some && bits(S.t) > bits(1.0)) {
           J.done(S, 1.0, REACHED);
           have = false;
         } else {
           if ((it & 7) == 7) S.cap = half_read([&] { return J.cap(); });
-          if (number && ((bits(S.cap) < bits(1.0) && bits(S.t) >= bits(S.cap)) || bits(S.t) > bits(S.hi))) {  // t_p >= t: this pair cannot lower the minimum
+          if (some && ((bits(S.cap) < bits(1.0) && bits(S.t) >= bits(S.cap)) || bits(S.t) > bits(S.hi))) {  // t_p >= t: this pair cannot lower the minimum
             J.done(S, S.t, STOPPED);
             have = false;
           } else if (it + 1 >= max_iter) {

@@ -36,6 +36,7 @@ struct Job {
     S.hi = 1.0;
     S.g = xmul(0.1, g0);
     S.tl = xdiv(xmul(xsub(1.0, 0.1), g0), S.lp);
+    if (isinf(bound)) S.off = NAN;  // every later gap is NaN
     return true;
   }
   __device__ double cap() const { return cba::half_leader() ? bound : (threadIdx.x & 1 ? 0.0 : 1e-3); }
@@ -111,3 +112,24 @@ def test_only_the_leaders_reading_counts(so, m, blocks, bound):
         assert np.array_equal(stop[below], ref[below] >= bound)
         assert np.all((t[stop] >= bound) & (t[stop] <= ref[stop]))
         assert np.array_equal(t[want & ~stop], ref[want & ~stop])  # (1 may be reached in one step across the bound)
+
+
+@pytest.mark.parametrize("m", [1, 5])
+def test_a_gap_that_is_no_number_ends_nothing(so, m):
+    """As in the one-lane iteration, whose comparisons with NaN are false: only
+    the limit of steps ends such a pair."""
+    import torch
+    dev = torch.device("cuda:0")
+    x, p, ee = _pairs(m, 50 + m)
+    p *= 8.0  # the first step stays below 1
+
+    def on(a):
+        return torch.from_numpy(np.ascontiguousarray(a)).to(dev)
+
+    bufs = [on(x.reshape(-1, 3).T), on(p.reshape(-1, 3).T), on(np.full(m, 0.0625)), on(ee.astype(np.uint8)),
+            on(np.ones(m, np.uint8))]
+    t = torch.full((m,), -1.0, dtype=torch.float64, device=dev)
+    how = torch.full((m,), -1, dtype=torch.int32, device=dev)
+    torch.cuda.synchronize()
+    assert so.run(*[b.data_ptr() for b in bufs], 4 * m, float("inf"), t.data_ptr(), how.data_ptr(), m, 1) == 0
+    assert np.all(how.cpu().numpy() == 2) and np.all(np.isnan(t.cpu().numpy()))
