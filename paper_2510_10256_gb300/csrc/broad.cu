@@ -898,12 +898,14 @@ cb_status broad_phase(cb_scene* s, BroadWork& w, const double* x, const double* 
     A.out_cap = (unsigned long long)(list.bytes / sizeof(uint64_t));
     A.cls = cls ? bp<uint8_t>(*cls) : nullptr;
     if (cls) A.out_cap = std::min<unsigned long long>(A.out_cap, cls->bytes);
+    // candidates are numbered in 32 bits, whatever room an earlier call left in the list
+    A.out_cap = std::min<unsigned long long>(A.out_cap, 0xffffffffull);
     k_tiles<<<s->n_sms * 3, 32 * TILE_WARPS, 0, cb_count(st)>>>(A);
     CB_CUDA(cudaGetLastError());
     CB_TRY(read_scalars(s, SC_COUNT0, 2, h, st));
     find = h[0] > A.tile_cap;
     if (!find && h[1] <= A.out_cap) break;
-    if (h[1] > 0xffffffffull) return CB_ERR_TOO_LARGE;  // candidates are numbered in 32 bits
+    if (h[1] > 0xffffffffull) return CB_ERR_TOO_LARGE;
     if (find) {
       CB_TRY(buf_ensure(w.tiles, sizeof(uint2) * (size_t)h[0], st));
     } else {
