@@ -36,7 +36,7 @@ struct Job {
     S.hi = 1.0;
     S.g = xmul(0.1, g0);
     S.tl = xdiv(xmul(xsub(1.0, 0.1), g0), S.lp);
-    if (isinf(bound)) S.off = NAN;  // every later gap is NaN
+    if (isinf(bound)) S.off = -NAN;  // every later gap is NaN, its sign set (as in inf - inf on the device)
     return true;
   }
   __device__ double cap() const { return cba::half_leader() ? bound : (threadIdx.x & 1 ? 0.0 : 1e-3); }
