@@ -85,7 +85,7 @@ static cb_status upload(DevBuf& b, const T* h, size_t count, cudaStream_t st) {
 
 static void scene_release(cb_scene* s) {
   cudaStream_t st = s->last_stream;
-  DevBuf* bufs[] = {&s->ev0, &s->ev1, &s->tv, &s->comp, &s->rest, &s->rod_ptr, &s->slots, &s->cinfo, &s->supers, &s->jobs, &s->S, &s->win, &s->wst,
+  DevBuf* bufs[] = {&s->ev0, &s->ev1, &s->tv, &s->comp, &s->rest, &s->rod_ptr, &s->vcomp, &s->prank, &s->slots, &s->cinfo, &s->supers, &s->jobs, &s->S, &s->win, &s->wst,
                     &s->rloop, &s->rlast, &s->elen2, &s->mlist, &s->ruv, &s->frest,
                     &s->frest_dbar, &s->fmask_key, &s->fmask_bits, &s->dbar_comp, &s->cand, &s->klass, &s->cand_alt, &s->klass_alt, &s->cd, &s->cflag, &s->cpos, &s->ctype, &s->ccls, &s->clist, &s->aidx,
                     &s->bkey, &s->rcol, &s->bsr_row, &s->bsr_col, &s->bsr_val,
@@ -429,7 +429,7 @@ cb_status cb_scene_create(const cb_scene_desc* d, const cb_allocator* allocator,
   if (d->kind == CB_SHELL && (rc = buf_ensure(s->rloop, 16, st)) != CB_OK) return fail(rc);
   for (auto& e : s->ev)
     if (cudaEventCreate(&e) != cudaSuccess) return fail(CB_ERR_CUDA);
-  if ((rc = clusters_build(s, d->rest_xyz, st)) != CB_OK) return fail(rc);
+  if ((rc = clusters_build(s, d->rest_xyz, comp, e0, tris, st)) != CB_OK) return fail(rc);
   // the rest broad phase reads the member parameters (box inflation)
   if ((rc = upload_members(s, st)) != CB_OK) return fail(rc);
   if ((rc = filter_precompute(s, st)) != CB_OK) return fail(rc);
@@ -448,8 +448,7 @@ cb_status cb_scene_create(const cb_scene_desc* d, const cb_allocator* allocator,
     if ((rc = read_scalars(s, SC_COUNT1, 1, &h, st)) != CB_OK) return fail(rc);
     s->n_frest_pt = (int64_t)h;
   }
-  // the filtered pairs lie in the tiles of the rest broad phase
-  if ((rc = filter_masks_build(s, s->bw.n_tiles, st)) != CB_OK) return fail(rc);
+  if ((rc = filter_masks_build(s, st)) != CB_OK) return fail(rc);
   if (cudaStreamSynchronize(st) != cudaSuccess) return fail(CB_ERR_CUDA);
   *out = s;
   return CB_OK;
@@ -597,9 +596,7 @@ cb_status cb_batch_create(cb_scene* const* members, int32_t count, const cb_allo
                                sizeof(unsigned long long) * cnt, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
       return fail(CB_ERR_CUDA);
   }
-  int64_t tiles = 0;
-  for (int m = 0; m < count; ++m) tiles += members[m]->n_fmask;
-  if ((rc = filter_masks_build(b, tiles, st)) != CB_OK) return fail(rc);
+  if ((rc = filter_masks_build(b, st)) != CB_OK) return fail(rc);
   for (auto& e : b->ev)
     if (cudaEventCreate(&e) != cudaSuccess) return fail(CB_ERR_CUDA);
   if ((rc = upload_members(b, st)) != CB_OK) return fail(rc);

@@ -81,7 +81,7 @@ struct BroadWork {
   DevBuf bounds;      // per member: 6 x uint32 ordered-float min/max
   DevBuf cx;          // per member: double centre[3], X (max |coordinate - centre|)
   DevBuf tiles;       // uint2 pairs of overlapping clusters
-  int64_t n_tiles = 0;  // of the last call
+  int64_t tiles_laid = 0;  // their number after the clusters were last laid out again for this phase
   DevBuf ckey[2];     // uint64 compact candidate keys (ping-pong; sorted lists only)
   DevBuf scan_tmp;
   DevBuf hist;
@@ -122,7 +122,16 @@ struct cb_scene {
   DevBuf comp;          // int32 [n]
   DevBuf rest;          // double [3][n]
   DevBuf rod_ptr;       // int32 [n_rods+1] (rods)
-  // clusters of 32 primitives and superclusters of 32 clusters (broad.cu), fixed at creation
+  // connected components (rods: polylines), numbered by label, members' ones behind each other
+  int n_comps = 0;
+  std::vector<int32_t> hcomp;         // [n] component of each vertex (-1: in none)
+  std::vector<int32_t> comp_cnt[3];   // their vertices, triangles and edges (rods: edges only)
+  std::vector<uint64_t> comp_place;   // their places: Morton code at rest, or at the positions of the last lay_out_again
+  std::vector<int64_t> coff;          // member offsets of the components (count + 1)
+  bool has_packed = false;            // several components share clusters
+  DevBuf vcomp;         // int32 [n] hcomp
+  DevBuf prank;         // int32 [n_prims] rank of each primitive among those of its kind and component
+  // clusters of 32 primitives and superclusters of 32 clusters (broad.cu)
   int n_clusters = 0, n_supers = 0, n_jobs = 0;
   DevBuf slots;         // int4 [n_clusters][32]: a primitive's vertices (-1: none) and its index within its kind (-1: pad)
   DevBuf cinfo;         // uint32 [n_clusters] member << 2 | kind (0 vertex, 1 triangle, 2 edge)
@@ -146,9 +155,10 @@ struct cb_scene {
   double dbar_fmax = 0.0;  // largest per-component dbar_min (finite), or dbar_min
   int64_t n_frest = 0;
   // shells: frest as bit masks over pairs of clusters (frest.cuh, FilterMasks)
-  DevBuf fmask_key;     // uint64 [fmask_cap]
+  DevBuf fmask_key;     // uint64 [fmask_cap], a power of two
   DevBuf fmask_bits;    // uint32 [fmask_cap][32]
-  uint32_t fmask_cap = 0;
+  uint32_t fmask_mask = 0;  // fmask_cap - 1
+  bool masks_stale = false;  // the clusters changed and the masks do not fit them yet
   int64_t n_fmask = 0;  // pairs of clusters with filtered pairs
 
   // pass state
@@ -260,10 +270,11 @@ constexpr uint8_t CB_CCD_EXACT = 0x80, CB_CCD_ONE = 0x40;
 cb_status read_scalars(cb_scene* s, int first, int count, uint64_t* out, cudaStream_t st);
 
 // broad.cu
-// The clusters of a new scene (topology and rest positions on the device;
-// rest_host the same positions on the host) or of a batch (its members' ones,
-// renumbered).
-cb_status clusters_build(cb_scene* s, const double* rest_host, cudaStream_t st);
+// The clusters of a new scene (topology and rest positions on the device; on
+// the host the same positions, the vertices' component labels, the edges'
+// first vertices and the triangles) or of a batch (of its members' components).
+cb_status clusters_build(cb_scene* s, const double* rest_host, const std::vector<int32_t>& label,
+                         const std::vector<int32_t>& e0, const std::vector<int32_t>& tris, cudaStream_t st);
 cb_status clusters_concat(cb_scene* b, cb_scene* const* members, cudaStream_t st);
 // Candidate pairs of x (p == nullptr) or of the sweep x -> x + p.  Boxes are
 // inflated per member by a/2 (static) or xi/2 (swept = true).  Writes the
@@ -272,8 +283,8 @@ cb_status clusters_concat(cb_scene* b, cb_scene* const* members, cudaStream_t st
 // 3 culled, else 0) into *cls unless null, and their count into *n_out.
 cb_status broad_phase(cb_scene* s, BroadWork& w, const double* x, const double* p, bool swept, bool sort_out,
                       DevBuf& out, DevBuf* cls, int64_t* n_out, cudaStream_t st);
-// the bit masks of the filtered pairs s->frest, which lie in at most max_tiles pairs of clusters
-cb_status filter_masks_build(cb_scene* s, int64_t max_tiles, cudaStream_t st);
+// the bit masks of the filtered pairs s->frest
+cb_status filter_masks_build(cb_scene* s, cudaStream_t st);
 
 // narrow.cu
 cb_status filter_precompute(cb_scene* s, cudaStream_t st);
