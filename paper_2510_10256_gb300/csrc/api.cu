@@ -88,7 +88,7 @@ static void scene_release(cb_scene* s) {
   DevBuf* bufs[] = {&s->ev0, &s->ev1, &s->tv, &s->comp, &s->rest, &s->rod_ptr, &s->vcomp, &s->prank, &s->slots, &s->cinfo, &s->supers, &s->jobs, &s->S, &s->win, &s->wst,
                     &s->rloop, &s->rlast, &s->elen2, &s->mlist, &s->ruv, &s->frest,
                     &s->frest_dbar, &s->fmask_key, &s->fmask_bits, &s->dbar_comp, &s->cand, &s->klass, &s->cand_alt, &s->klass_alt, &s->cd, &s->cflag, &s->cpos, &s->ctype, &s->ccls, &s->clist, &s->aidx,
-                    &s->bkey, &s->rcol, &s->bsr_row, &s->bsr_col, &s->bsr_val,
+                    &s->bkey, &s->rcol, &s->hkey, &s->hflag, &s->hhist, &s->bsr_row, &s->bsr_col, &s->bsr_val,
                     &s->row_cnt, &s->hB9, &s->xf, &s->pf, &s->dlist, &s->mp, &s->vsc, &s->macc, &s->ccd_keys, &s->ccd_t, &s->ccd_cls, &s->ccd_list, &s->ccd_ulist, &s->scan_tmp,
                     &s->fr_key, &s->fr_st, &s->fr_dat, &s->fr_hw, &s->dev_scalars};
   for (DevBuf* b : bufs) buf_free(*b, st);

@@ -435,8 +435,9 @@ __global__ void k_to_f32(int n, const double* __restrict__ v, const double* __re
 // stencil, columns ascending in each row, without sorting the keys: each run of
 // BK_PAIRS active pairs makes its blocks distinct in shared memory
 // (k_block_keys), the survivors are bucketed by row (counts, scan, k_row_fill),
-// and each row's short bucket is sorted and made distinct by a warp
-// (k_row_unique; a block for buckets past ROW_MAX, k_row_unique_long).  On a
+// and each row's short bucket is made distinct and sorted by a warp
+// (k_row_unique; a block for buckets past ROW_MAX, k_row_unique_long; those past
+// ROW_BLOCK_MAX go through a radix sort together, huge_rows).  On a
 // pleated 256x256 pass (862k active pairs, 1.7M blocks) the keys take 0.11 ms,
 // fill, unique and write 0.16; a set of 4,096 keys per run and a radix sort of
 // the survivors (five digits) with its flags and scans took 0.18 and 0.75.
@@ -701,45 +702,129 @@ __global__ void __launch_bounds__(32 * ROW_WARPS) k_row_unique(int n, int per, c
   }
 }
 
-// ... a block per long bucket, in global memory
-__global__ void __launch_bounds__(cbp::SCAN_T) k_row_unique_long(const uint32_t* __restrict__ off, uint32_t* rcol,
-                                                                 uint32_t* __restrict__ uniq,
-                                                                 const uint32_t* __restrict__ longs,
-                                                                 const unsigned int* __restrict__ nlong) {
-  __shared__ unsigned tot;
-  __shared__ uint32_t last;
+// ... a block per long bucket of up to ROW_BLOCK_MAX entries: duplicates go through an open-addressing set at most half
+// full, the distinct columns are sorted in shared memory.  Longer buckets are numbered in hrow, with the first of
+// their entries among all such buckets' in hstart; `huge` counts both (buckets << 32 | entries).  Bound by the latency
+// of the sort's steps, which a block's 1,024 threads and shared memory shorten and the set keeps to distinct columns
+// (before, 256 threads sorted a whole bucket of any length in global memory): the barrier stage without its Hessian
+// kernel with one edge across 700 needles 184 -> 144 us, across 4,000 525 -> 215.
+constexpr unsigned ROW_BLOCK_MAX = 16384;
+constexpr int ROW_LONG_T = 1024;
+constexpr int ROW_LONG_SMEM = 3 * (int)ROW_BLOCK_MAX * 4;
+
+__global__ void __launch_bounds__(ROW_LONG_T) k_row_unique_long(const uint32_t* __restrict__ off, uint32_t* rcol,
+                                                            uint32_t* __restrict__ uniq,
+                                                            const uint32_t* __restrict__ longs,
+                                                            const unsigned int* __restrict__ nlong,
+                                                            uint32_t* __restrict__ hrow, uint32_t* __restrict__ hstart,
+                                                            unsigned long long* __restrict__ huge) {
+  extern __shared__ uint32_t long_smem[];
+  uint32_t *set = long_smem, *p = long_smem + 2 * ROW_BLOCK_MAX;
+  __shared__ unsigned nu;
   for (unsigned q = blockIdx.x; q < *nlong; q += gridDim.x) {
     const uint32_t r = longs[q], b = off[r], len = off[r + 1] - b;
-    uint32_t* p = rcol + b;
-    sort_segment(p, len, threadIdx.x, blockDim.x, [] { __syncthreads(); });
-    unsigned at = 0;
-    for (unsigned i0 = 0; i0 < len; i0 += blockDim.x) {
-      const unsigned i = i0 + threadIdx.x;
-      const uint32_t v = i < len ? p[i] : 0u;
-      // the entry before the chunk may have been overwritten already: it is carried in `last`
-      const uint32_t u = i < len && threadIdx.x > 0 ? p[i - 1] : (i0 > 0 ? last : 0u);
-      const bool keep = i < len && (i == 0 || v != u);
-      const unsigned pos = cbp::block_excl_scan<unsigned>(keep ? 1u : 0u, &tot);
-      if (i < len && threadIdx.x == blockDim.x - 1) last = v;  // every read of this chunk is over
-      if (keep) p[at + pos] = v;
-      at += tot;
-      __syncthreads();
+    if (len > ROW_BLOCK_MAX) {
+      if (threadIdx.x == 0) {
+        const unsigned long long at = atomicAdd(huge, 1ull << 32 | len);  // (the buckets hold fewer than 2^32 entries)
+        hrow[at >> 32] = r;
+        hstart[at >> 32] = (uint32_t)at;
+      }
+      continue;
     }
-    if (threadIdx.x == 0) uniq[r] = at;
+    const int bits = 33 - __clz(len - 1);  // 2^bits >= 2 len
+    for (unsigned i = threadIdx.x; i < 1u << bits; i += ROW_LONG_T) set[i] = 0xffffffffu;
+    if (threadIdx.x == 0) nu = 0;
     __syncthreads();
+    for (unsigned i = threadIdx.x; i < len; i += ROW_LONG_T) {
+      const uint32_t v = rcol[b + i];
+      for (unsigned h = v * 2654435769u >> (32 - bits);; h = (h + 1) & ((1u << bits) - 1u)) {  // ends: half the slots are free
+        const uint32_t u = atomicCAS(&set[h], 0xffffffffu, v);
+        if (u == 0xffffffffu) p[atomicAdd(&nu, 1u)] = v;
+        if (u == 0xffffffffu || u == v) break;
+      }
+    }
+    __syncthreads();
+    const unsigned m = nu;
+    sort_segment(p, m, threadIdx.x, ROW_LONG_T, [] { __syncthreads(); });
+    for (unsigned i = threadIdx.x; i < m; i += ROW_LONG_T) rcol[b + i] = p[i];
+    if (threadIdx.x == 0) uniq[r] = m;
+    __syncthreads();  // before the next bucket takes the set
   }
 }
 
+// ... the buckets past ROW_BLOCK_MAX together: their entries as (bucket, column) keys, radix sorted, made distinct and put
+// back.  One bucket's time in a block grows with its length, and the pass waits for it; the sort spreads over the chip,
+// for one more host wait.  Without the Hessian kernel, a sheet of 65k vertices on two triangles (four rows of 65k
+// columns) 6.79 -> 0.35 ms, an edge across 100,000 needles 41.9 -> 0.56.  The line: 20 buckets of 8,000 entries take
+// 291 us in blocks against 378 sorted, of 16,200 534 against 527 -- and a block's shared memory ends at 16,384.
+struct HugeRows {
+  unsigned n, entries;
+  int cbits;  // bits of a column
+  const uint32_t* __restrict__ row;
+  const uint32_t* __restrict__ start;
+  const uint32_t* __restrict__ off;
+  __device__ __forceinline__ unsigned bucket_of(unsigned i) const {
+    unsigned lo = 0, hi = n;  // the last bucket that starts at or before entry i
+    while (hi - lo > 1) {
+      const unsigned mid = (lo + hi) >> 1;
+      if (start[mid] <= i) lo = mid;
+      else hi = mid;
+    }
+    return lo;
+  }
+};
+
+__global__ void k_huge_keys(HugeRows H, const uint32_t* __restrict__ rcol, uint64_t* __restrict__ key) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= H.entries) return;
+  const unsigned k = H.bucket_of((unsigned)i);
+  key[i] = (uint64_t)k << H.cbits | rcol[H.off[H.row[k]] + ((unsigned)i - H.start[k])];
+}
+__global__ void k_huge_flag(unsigned entries, const uint64_t* __restrict__ key, uint32_t* __restrict__ flag) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i <= entries) flag[i] = i < entries && (i == 0 || key[i] != key[i - 1]) ? 1u : 0u;
+}
+__global__ void k_huge_write(HugeRows H, const uint64_t* __restrict__ key, const uint32_t* __restrict__ flag,
+                             const uint32_t* __restrict__ pos, uint32_t* __restrict__ rcol, uint32_t* __restrict__ uniq) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= H.entries || !flag[i]) return;
+  const unsigned k = (unsigned)(key[i] >> H.cbits), first = H.start[k], end = k + 1 < H.n ? H.start[k + 1] : H.entries;
+  const uint32_t r = H.row[k];
+  rcol[H.off[r] + (pos[i] - pos[first])] = (uint32_t)(key[i] & ((1ull << H.cbits) - 1ull));
+  if (i == first) uniq[r] = pos[end] - pos[first];
+}
+
 // the rows' distinct columns to their place, 8 lanes a row (a full warp left most lanes without work: 64 rod scenes
-// with 1.1M rows 142 -> 46 us)
+// with 1.1M rows 142 -> 46 us); rows past ROW_MAX columns take a block, those past ROW_BLOCK_MAX a thread per entry
 __global__ void k_row_write(int n, const uint32_t* __restrict__ off, const uint32_t* __restrict__ rcol,
                             const int32_t* __restrict__ row_ptr, int32_t* __restrict__ col) {
   const int r = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3);
   if (r >= n) return;
   const int o = row_ptr[r], c = row_ptr[r + 1] - o;
-  if (c == 0) return;
+  if (c == 0 || c > (int)ROW_MAX) return;
   const uint32_t b = off[r];
   for (int i = threadIdx.x & 7; i < c; i += 8) col[o + i] = (int32_t)rcol[b + i];
+}
+__global__ void __launch_bounds__(ROW_LONG_T) k_row_write_long(const uint32_t* __restrict__ longs, unsigned nlong,
+                                                               const uint32_t* __restrict__ off,
+                                                               const uint32_t* __restrict__ rcol,
+                                                               const int32_t* __restrict__ row_ptr,
+                                                               int32_t* __restrict__ col) {
+  for (unsigned q = blockIdx.x; q < nlong; q += gridDim.x) {
+    const uint32_t r = longs[q], b = off[r];
+    const int o = row_ptr[r], c = row_ptr[r + 1] - o;
+    if (c <= (int)ROW_MAX || c > (int)ROW_BLOCK_MAX) continue;
+    for (int i = threadIdx.x; i < c; i += ROW_LONG_T) col[o + i] = (int32_t)rcol[b + i];
+  }
+}
+__global__ void k_huge_cols(HugeRows H, const uint32_t* __restrict__ rcol, const int32_t* __restrict__ row_ptr,
+                            int32_t* __restrict__ col) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= H.entries) return;
+  const unsigned k = H.bucket_of((unsigned)i);
+  const uint32_t r = H.row[k];
+  const int o = row_ptr[r], c = row_ptr[r + 1] - o, q = (int)((unsigned)i - H.start[k]);
+  if (c > (int)ROW_BLOCK_MAX && q < c) col[o + q] = (int32_t)rcol[H.off[r] + q];
 }
 
 // Distance types as difference vectors z_m = x_plus - x_minus:
@@ -1958,6 +2043,31 @@ __global__ void k_pass_reset(unsigned long long* __restrict__ sc, uint32_t sc_ma
 
 }  // namespace
 
+// the distinct columns of the buckets past ROW_BLOCK_MAX (counted in `huge`)
+static cb_status huge_rows(cb_scene* s, const HugeRows& H, uint32_t* uniq, cudaStream_t st) {
+  int bits = H.cbits;
+  while ((uint64_t)(H.n - 1) >> (bits - H.cbits)) ++bits;
+  const int64_t L = H.entries;
+  CB_TRY(buf_ensure(s->hkey, sizeof(uint64_t) * (size_t)L, st));
+  CB_TRY(buf_ensure(s->hflag, sizeof(uint32_t) * 2 * (size_t)(L + 1), st));
+  CB_TRY(buf_ensure(s->hhist, sizeof(uint32_t) * (size_t)cbp::radix_hist_elems(L), st));
+  CB_TRY(buf_ensure(s->scan_tmp, sizeof(uint64_t) * (size_t)(std::max(cbp::scan_tmp_elems(cbp::radix_hist_elems(L)),
+                                                                      cbp::scan_tmp_elems(L + 1)) + 8), st));
+  // the blocks' keys are in their buckets by now: their memory (16 an active pair) holds these
+  uint64_t *k0 = bp<uint64_t>(s->bkey), *k1 = bp<uint64_t>(s->hkey);
+  uint32_t *flag = bp<uint32_t>(s->hflag), *pos = flag + (L + 1);
+  k_huge_keys<<<cb_grid(L), CB_THREADS, 0, cb_count(st)>>>(H, bp<uint32_t>(s->rcol), k0);
+  const uint64_t* key = cbp::radix_sort<uint64_t, uint32_t, false>(k0, nullptr, k1, nullptr, L, 0, bits,
+                                                                   bp<uint32_t>(s->hhist), bp<uint32_t>(s->scan_tmp), st)
+                            ? k1
+                            : k0;
+  k_huge_flag<<<cb_grid(L + 1), CB_THREADS, 0, cb_count(st)>>>((unsigned)L, key, flag);
+  cbp::exclusive_scan<uint32_t, uint32_t>(flag, pos, L + 1, bp<uint32_t>(s->scan_tmp), (uint32_t*)nullptr, st);
+  k_huge_write<<<cb_grid(L), CB_THREADS, 0, cb_count(st)>>>(H, key, flag, pos, bp<uint32_t>(s->rcol), uniq);
+  CB_CUDA(cudaGetLastError());
+  return CB_OK;
+}
+
 __global__ void k_fill_u64(int64_t n, unsigned long long* __restrict__ p, unsigned long long v) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) p[i] = v;
@@ -2123,7 +2233,8 @@ cb_status barrier_run(cb_scene* s, const double* x, double* energy, double* grad
   // the pass's counters (the queue lengths stay readable until the next pass)
   {
     const uint32_t scm = (1u << SC_NCORE) | (1u << SC_NLIST) | (1u << SC_KSPLIT) | (1u << SC_NMOLL) |
-                         (1u << SC_N9) | (1u << SC_N6) | (1u << SC_N4) | (1u << SC_NBK) | (1u << SC_NLONG);
+                         (1u << SC_N9) | (1u << SC_N6) | (1u << SC_N4) | (1u << SC_NBK) | (1u << SC_NLONG) |
+                         (1u << SC_HUGE);
     k_pass_reset<<<cb_grid(std::max(M, (int)SC_N)), CB_THREADS, 0, cb_count(st)>>>(
         (unsigned long long*)sc, scm, M, macc, (1u << MACC_E) | (1u << MACC_STATUS));
   }
@@ -2193,21 +2304,41 @@ cb_status barrier_run(cb_scene* s, const double* x, double* energy, double* grad
     const int per = n >= s->n_sms * 64 * 8 ? 8 : 1;
     k_row_unique<<<cb_grid(((int64_t)n + per - 1) / per * 32, 32 * ROW_WARPS), 32 * ROW_WARPS, 0, cb_count(st)>>>(
         n, per, off, bp<uint32_t>(s->rcol), uniq, longs, nlong);
-    k_row_unique_long<<<s->n_sms, cbp::SCAN_T, 0, cb_count(st)>>>(off, bp<uint32_t>(s->rcol), uniq, longs, nlong);
-    // uniq[n] = 0: the scan's last entry is the block count
-    uint32_t* tot = (uint32_t*)(sc + SC_COUNT1);
-    cbp::exclusive_scan<uint32_t, int32_t>(uniq, bp<int32_t>(s->bsr_row), (int64_t)n + 1,
-                                           (int32_t*)bp<uint32_t>(s->scan_tmp), (int32_t*)tot, st);
-    CB_CUDA(cudaGetLastError());
-    uint64_t h;
-    CB_TRY(read_scalars(s, SC_COUNT1, 1, &h, st));
-    s->nnzb = (int64_t)(uint32_t)h;
+    // rows, and the first entries, of the buckets past ROW_BLOCK_MAX: the counts and cursors are of no more use
+    uint32_t *hrow = cnt, *hstart = cursor;
+    CB_CUDA(cudaFuncSetAttribute(k_row_unique_long, cudaFuncAttributeMaxDynamicSharedMemorySize, ROW_LONG_SMEM));
+    k_row_unique_long<<<s->n_sms, ROW_LONG_T, ROW_LONG_SMEM, cb_count(st)>>>(off, bp<uint32_t>(s->rcol), uniq, longs, nlong, hrow,
+                                                                     hstart, (unsigned long long*)(sc + SC_HUGE));
+    uint64_t h[SC_HUGE - SC_COUNT1 + 1];
+    auto row_pointers = [&]() -> cb_status {
+      // uniq[n] = 0: the scan's last entry is the block count
+      uint32_t* tot = (uint32_t*)(sc + SC_COUNT1);
+      cbp::exclusive_scan<uint32_t, int32_t>(uniq, bp<int32_t>(s->bsr_row), (int64_t)n + 1,
+                                             (int32_t*)bp<uint32_t>(s->scan_tmp), (int32_t*)tot, st);
+      CB_CUDA(cudaGetLastError());
+      return read_scalars(s, SC_COUNT1, SC_HUGE - SC_COUNT1 + 1, h, st);
+    };
+    CB_TRY(row_pointers());
+    const uint64_t huge = h[SC_HUGE - SC_COUNT1];
+    HugeRows H{(unsigned)(huge >> 32), (unsigned)huge, 1, hrow, hstart, off};
+    while ((int64_t)(n - 1) >> H.cbits) ++H.cbits;
+    if (H.n > 0) {
+      CB_TRY(huge_rows(s, H, uniq, st));
+      CB_TRY(row_pointers());
+    }
+    s->nnzb = (int64_t)(uint32_t)h[0];
     CB_TRY(buf_ensure(s->bsr_col, sizeof(int32_t) * (size_t)s->nnzb, st));
     CB_TRY(buf_ensure(s->bsr_val, sizeof(double) * 9 * (size_t)s->nnzb, st));
     CB_CUDA(cudaMemsetAsync(s->bsr_val.p, 0, sizeof(double) * 9 * (size_t)s->nnzb, st));
     k_row_write<<<cb_grid((int64_t)n * 8), CB_THREADS, 0, cb_count(st)>>>(n, off, bp<uint32_t>(s->rcol),
                                                                           bp<int32_t>(s->bsr_row),
                                                                           bp<int32_t>(s->bsr_col));
+    if (const unsigned rows = (unsigned)h[SC_NLONG - SC_COUNT1])
+      k_row_write_long<<<(int)std::min<int64_t>(rows, (int64_t)s->n_sms * 2), ROW_LONG_T, 0, cb_count(st)>>>(
+          longs, rows, off, bp<uint32_t>(s->rcol), bp<int32_t>(s->bsr_row), bp<int32_t>(s->bsr_col));
+    if (H.n > 0)
+      k_huge_cols<<<cb_grid(H.entries), CB_THREADS, 0, cb_count(st)>>>(H, bp<uint32_t>(s->rcol), bp<int32_t>(s->bsr_row),
+                                                                      bp<int32_t>(s->bsr_col));
     HessArgs A;
     A.act = act;
     A.cand = bp<uint64_t>(s->cand);

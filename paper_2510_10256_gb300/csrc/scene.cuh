@@ -190,6 +190,8 @@ struct cb_scene {
   DevBuf bsr_col;       // int32 [nnzb]
   DevBuf bsr_val;       // double [nnzb][9]
   DevBuf row_cnt;       // uint32 [5][n+1]: keys, fill cursor, distinct columns and bucket offset of each row; long rows
+                        // (from k_row_unique_long on: the first two the rows past ROW_BLOCK_MAX and their first entries)
+  DevBuf hkey, hflag, hhist;  // rows past ROW_BLOCK_MAX (narrow.cu): uint64 keys, uint32 flags and positions, digit counts
   int64_t nnzb = 0;
   DevBuf mlist;         // uint32 [nc] active candidates with a mollifier below 1 (CB_EE_MOLLIFIER)
   DevBuf hB9;           // CB_EE_MOLLIFIER: queued reduced Hessians (packed, element-major)
@@ -254,7 +256,8 @@ enum {
   SC_NX = 23,           // ccd_step: two uint32 counters, point-triangle and edge-edge pairs of the FP64 iteration
   SC_NLONG = 24,        // barrier_eval: rows of the pattern with buckets past a warp's
   SC_NFB = 25,          // contact_build: filtered pairs among the candidates
-  SC_N = 26
+  SC_HUGE = 26,         // barrier_eval: rows of the pattern with buckets past a block's << 32 | their entries
+  SC_N = 27
 };
 // read_scalars stages up to SC_N scalars through the pinned host scratch
 static_assert(SC_N <= 32, "the scalars must fit the pinned scratch and a 32-bit mask");
