@@ -1759,8 +1759,10 @@ constexpr int PL_THREADS = 32 * PL_PAIRS;   // one warp per pair: three lanes pe
 // doubles per pair: A, X (A J; later the Hadamard staging, 108), V, and the
 // FP32 phase's A, X, V (3 x 81 floats)
 constexpr int PL_SMEM = 81 + 108 + 81 + 122;
-// queues of at most this many active pairs take the lane-parallel form
-constexpr int64_t PL_MAX_ACTIVE = 4096;
+// Queues of at most this many (mollified) pairs take the lane-parallel form.  Stage (d) with n such pairs, lane-parallel
+// against one thread a pair: 100 pairs 374 / 713 us, 2,000 486 / 722, 4,000 629 / 724, 5,000 708 / 730, 6,000 819 / 733;
+// a pleated 97x97 sheet with 1,296 of 47,510 active pairs mollified 627 / 1,180.
+constexpr int64_t PL_MAX_PAIRS = 4096;
 
 // sum over the warp: a butterfly, so every lane gets the same bits
 template <typename R>
@@ -2240,6 +2242,7 @@ cb_status barrier_run(cb_scene* s, const double* x, double* energy, double* grad
   }
   if (grad) CB_CUDA(cudaMemsetAsync(grad, 0, sizeof(double) * 3 * (size_t)s->n, st));
   s->n_active = s->n_plane = 0;
+  int64_t nmoll = 0;
   s->nnzb = 0;
   CB_TRY(buf_ensure(s->bsr_row, sizeof(int32_t) * ((size_t)s->n + 1), st));
   CB_CUDA(cudaMemsetAsync(s->bsr_row.p, 0, sizeof(int32_t) * ((size_t)s->n + 1), st));
@@ -2269,10 +2272,11 @@ cb_status barrier_run(cb_scene* s, const double* x, double* energy, double* grad
       return CB_OK;
     }
     CB_CUDA(cudaGetLastError());
-    uint64_t h;
-    CB_TRY(read_scalars(s, SC_KSPLIT, 1, &h, st));
-    s->n_plane = (int64_t)(uint32_t)h;
-    s->n_active = s->n_plane + (int64_t)(h >> 32);
+    uint64_t h[SC_NMOLL - SC_KSPLIT + 1];
+    CB_TRY(read_scalars(s, SC_KSPLIT, SC_NMOLL - SC_KSPLIT + 1, h, st));
+    s->n_plane = (int64_t)(uint32_t)h[0];
+    s->n_active = s->n_plane + (int64_t)(h[0] >> 32);
+    nmoll = (int64_t)(uint32_t)h[SC_NMOLL - SC_KSPLIT];
     s->act_cap = nc;
     // end of stage (c): distances, classes and the active set
     if (s->timing) cudaEventRecord(s->ev[12], st);
@@ -2361,26 +2365,25 @@ cb_status barrier_run(cb_scene* s, const double* x, double* energy, double* grad
     A.val = bp<double>(s->bsr_val);
     A.grad = grad;
     A.status = status;
-    if (mollify) CB_TRY(buf_ensure(s->hB9, sizeof(double) * 45 * (size_t)na, st));
+    if (nmoll > 0) CB_TRY(buf_ensure(s->hB9, sizeof(double) * 45 * (size_t)nmoll, st));
     A.B9 = bp<double>(s->hB9);
     A.n9 = (unsigned int*)(sc + SC_N9);
     A.n6 = (unsigned int*)(sc + SC_N6);
     A.n4 = (unsigned int*)(sc + SC_N4);
-    A.cap = na;
+    A.cap = nmoll;
     A.mlist = bp<uint32_t>(s->mlist);
     A.nmoll = (const unsigned*)(sc + SC_NMOLL);
     A.elen2 = bp<double>(s->elen2);
     if (s->timing) cudaEventRecord(s->ev[10], st);
     k_pair_hess<<<cb_grid(na, PAIR_T), PAIR_T, 0, cb_count(st)>>>(A);
     CB_CUDA(cudaGetLastError());
-    if (mollify) {
-      // the queue's length stays on the device; a warp per pair while the queue is short
-      k_moll_hess<<<cb_grid(na, 32), 32, 0, cb_count(st)>>>(A);
-      if (na <= PL_MAX_ACTIVE) {
+    if (nmoll > 0) {
+      k_moll_hess<<<cb_grid(nmoll, 32), 32, 0, cb_count(st)>>>(A);
+      if (nmoll <= PL_MAX_PAIRS) {
         const int smem = PL_SMEM * (int)sizeof(double) * PL_PAIRS;
-        k_hess_proj_lanes<<<(int)((na + PL_PAIRS - 1) / PL_PAIRS), PL_THREADS, smem, cb_count(st)>>>(A);
+        k_hess_proj_lanes<<<(int)((nmoll + PL_PAIRS - 1) / PL_PAIRS), PL_THREADS, smem, cb_count(st)>>>(A);
       } else {
-        CB_TRY(launch_proj(s, A, na, st));
+        CB_TRY(launch_proj(s, A, nmoll, st));
       }
       CB_CUDA(cudaGetLastError());
     }
