@@ -124,20 +124,6 @@ def stage_roofline(st: dict, med: list, scenes) -> dict:
     return out
 
 
-def _autotune(args, runner, scenes, run_pass):
-    """Broad-phase knobs from the autotuner (cached per GPU and scene class)."""
-    if args.no_tune:
-        return {"autotuned": False, "cell_factor": [runner.tuning(0)[0], runner.tuning(1)[0]]}
-    import torch
-    from paper_2510_10256_gb300.tune import Autotuner, scene_key
-    key = scene_key(scenes, torch.cuda.get_device_name())
-    c = Autotuner().tune(runner, key, run_pass)
-    torch.cuda.synchronize()
-    return {"autotuned": True, "cached": c["cached"],
-            "build": {k: c["0"][k] for k in ("cell_factor", "pair_block", "stage_ms", "default_ms")},
-            "ccd": {k: c["1"][k] for k in ("cell_factor", "pair_block", "stage_ms", "default_ms")}}
-
-
 def _workload(name: str, reduced_nx: int | None = None):
     from paper_2510_10256_gb300 import scenes as S
     if name == "pleated":
@@ -326,11 +312,6 @@ def bench_batch(args, rank, world, local, dist):
         for k, m in enumerate(members):
             m.run_pass(xs[k], ps[k], es[k], gs[k], als[k])
 
-    tuning = _autotune(args, batch, scenes, run_batched)
-    if not args.no_plain:  # the plain arm uses the same knobs
-        for m in members:
-            for ph in (0, 1):
-                m.set_tuning(ph, *batch.tuning(ph))
     batch.set_timing(True)
     for _ in range(args.warmup):
         run_batched()
@@ -387,7 +368,7 @@ def bench_batch(args, rank, world, local, dist):
             "config": {"workload": f"{M} rod scenes (even: plain weave, odd: helix-loop knit), "
                                    f"{min(sizes)}-{max(sizes)} vertices each, {N} in all, batched",
                        "candidates": n_cand, "active": na, "ccd_pairs": int(st["n_ccd"]), "nnzb": int(st["nnzb"]),
-                       "ccd_max_iters": int(st["ccd_max_iters"]), "tuning": tuning,
+                       "ccd_max_iters": int(st["ccd_max_iters"]),
                        "l2": "flushed (256 MiB write) between steps", "parallelism": f"replicas x{world}"},
             "plain": {"value": world * n_cand / (pms / 1000.0), "unit": UNIT, "ms_per_step": pms,
                       "form": f"{M} single-scene passes in sequence on one stream"},
@@ -694,7 +675,7 @@ def main():
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-plain", action="store_true",
                     help="knit64 / serve: skip the one-scene-per-launch (plain) arm")
-    ap.add_argument("--no-tune", action="store_true", help="keep the default broad-phase knobs")
+    ap.add_argument("--no-tune", action="store_true", help="accepted and ignored: the broad phase has no knobs")
     ap.add_argument("--mollifier", action="store_true", help="single-scene workloads: IPC's edge-edge mollifier")
     ap.add_argument("--no-extras", action="store_true",
                     help="pleated: skip the graded disk and the served stream that the default line carries")
@@ -786,9 +767,8 @@ def one_core_baselines() -> dict:
 
 
 def measure_single(args, name, steps, local, dist, nx=None, mollifier=False, clocks=True) -> dict:
-    """One scene of the named workload: autotuned broad-phase knobs, W warm-up
-    passes, then `steps` passes timed on the device (L2 flushed before each),
-    the per-stage times of each pass, and an end-to-end leg through the C ABI
+    """One scene of the named workload: W warm-up passes, then `steps` passes
+    timed on the device (L2 flushed before each), the per-stage times of each pass, and an end-to-end leg through the C ABI
     with host buffers (copies inside the timed region)."""
     import torch
     from paper_2510_10256_gb300 import contact as CT
@@ -802,7 +782,6 @@ def measure_single(args, name, steps, local, dist, nx=None, mollifier=False, clo
     grad = torch.zeros(3, sc.n, dtype=torch.float64, device=dev)
     alpha = torch.zeros(1, dtype=torch.float64, device=dev)
     flush = torch.empty(L2_FLUSH_BYTES, dtype=torch.uint8, device=dev)
-    tuning = _autotune(args, cs, [sc], lambda: cs.run_pass(x, p, energy, grad, alpha))
     cs.set_timing(True)
     for _ in range(args.warmup):
         cs.run_pass(x, p, energy, grad, alpha)
@@ -855,7 +834,7 @@ def measure_single(args, name, steps, local, dist, nx=None, mollifier=False, clo
     e2e_ms = max_over_ranks([statistics.median(a.elapsed_time(b) for a, b in e_ev)], dist, dev)[0]
     cs.close()
     return {"sc": sc, "desc": desc, "st": st, "step_ms": step_ms, "ms": ms, "stage": stage, "e2e_ms": e2e_ms,
-            "launches": launches, "tuning": tuning, "clocks": clk, "status": status, "steps": steps,
+            "launches": launches, "clocks": clk, "status": status, "steps": steps,
             "h2d": 2 * 3 * sc.n * 8, "d2h": 8 + 8 + 3 * sc.n * 8}
 
 
@@ -874,7 +853,7 @@ def _single_summary(r, world) -> dict:
             "stage_roofline": stage_roofline(st, med, [r["sc"]]),
             "e2e": {"value": world * st["n_candidates"] / (r["e2e_ms"] / 1000.0), "unit": UNIT,
                     "ms_per_step": r["e2e_ms"], "h2d_bytes_per_step": r["h2d"], "d2h_bytes_per_step": r["d2h"]},
-            "tuning": r["tuning"], "gpu_launches": int(r["launches"]), "status": r["status"]}
+            "gpu_launches": int(r["launches"]), "status": r["status"]}
 
 
 def _single_line(args, r, world) -> dict:
@@ -907,7 +886,7 @@ def _single_line(args, r, world) -> dict:
             "vs_baseline": None, "dtype": "f64", "data": "synthetic",
             "config": {"workload": r["desc"], "candidates": int(n_cand), "filtered": st["n_filtered"],
                        "core": st["n_core"], "active": int(na), "ccd_pairs": st["n_ccd"], "nnzb": st["nnzb"],
-                       "dbar_min": st["dbar_min"], "seed": sc.seed, "tuning": r["tuning"],
+                       "dbar_min": st["dbar_min"], "seed": sc.seed,
                        "mollifier": bool(args.mollifier), "mollified_pairs": st["n_mollified"],
                        "l2": "flushed (256 MiB write) between steps", "timing": "median of the timed passes",
                        "parallelism": f"replicas x{world}"},

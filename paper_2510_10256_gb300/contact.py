@@ -262,6 +262,8 @@ class ContactScene:
     """A scene of the contact library: topology, rest mesh, filter tables and
     the pass buffers, resident on the current CUDA device."""
 
+    tuning_inert = True  # set_tuning's knobs size nothing (tune.py)
+
     def __init__(self, kind: str, rest, thickness: float, dhat: float, rod_ptr=None, tris=None,
                  kappa: float = 1.0, mode: str = "double", paper_literal: bool = False,
                  core_temp: bool = True, cull_radius: int = 0, per_component: bool = False, rod_closed=None,
@@ -500,7 +502,7 @@ class ContactScene:
         return int(lib().cb_sync_status(self.h))
 
     def set_tuning(self, phase: int, cell_factor: float, pair_block: int = 256):
-        """Broad-phase knobs (phase 0: contact_build, 1: ccd_step); speed only."""
+        """Broad-phase knobs (phase 0: contact_build, 1: ccd_step): kept and returned, they size nothing."""
         _check(lib().cb_set_tuning(self.h, int(phase), float(cell_factor), int(pair_block)), "cb_set_tuning")
 
     def tuning(self, phase: int) -> tuple[float, int]:

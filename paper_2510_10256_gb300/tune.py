@@ -2,12 +2,15 @@
 
 The knobs change no result: a cell factor and a pair-kernel block size,
 separately for contact_build's broad phase (phase 0) and ccd_step's swept
-broad phase (phase 1).  They sized a cell hash; the library's cluster broad
-phase has neither cells nor such blocks, so every choice now times the same.  Each candidate is timed with the
-library's own stage events on passes over the caller's data; the fastest is
-kept and cached in a JSON file, keyed by the GPU, the scene kind, the vertex
-count (octave) and the ratio of the activation to the mean edge length
-(half octave).
+broad phase (phase 1).  Each candidate is timed with the runner's own stage
+events on passes over the caller's data; the fastest is kept and cached in a
+JSON file, keyed by the GPU, the scene kind, the vertex count (octave) and the
+ratio of the activation to the mean edge length (half octave).
+
+A runner whose knobs size nothing says so (tuning_inert, as ContactScene does:
+the library's broad phase works on clusters, which have neither cells nor such
+blocks).  Its defaults are timed and kept, the other choices are not tried --
+they could only differ by noise -- and the cache is left alone.
 """
 from __future__ import annotations
 
@@ -19,6 +22,7 @@ import numpy as np
 
 FACTORS = (0.5, 0.71, 1.0, 1.41, 2.0, 2.83, 4.0)
 BLOCKS = (128, 256)
+DEFAULT = (1.0, 256)
 DEFAULT_CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_tuning.json")
 # stage_ms index of the stage that contains each phase's broad phase
 _STAGE = {0: 0, 1: 3}
@@ -78,27 +82,29 @@ class Autotuner:
         """Pick the knobs for `runner` (a ContactScene or ContactBatch);
         run_pass() must run one full pass on it.  Returns the choice per phase
         with the measured stage time, and whether it came from the cache."""
-        if not force and key in self.cache:
+        inert = bool(getattr(runner, "tuning_inert", False))
+        if not force and not inert and key in self.cache:
             self.apply(runner, self.cache[key])
             return dict(self.cache[key], cached=True, key=key)
         runner.set_timing(True)
+        settings = [DEFAULT] if inert else [(f, b) for f in self.factors for b in self.blocks]
         choice = {}
         for ph in (0, 1):
             trials = []
-            for f in self.factors:
-                for b in self.blocks:
-                    runner.set_tuning(ph, f, b)
-                    run_pass()  # buffers settle to this setting's sizes
-                    t = []
-                    for _ in range(self.reps):
-                        run_pass()
-                        t.append(runner.stage_ms()[_STAGE[ph]])
-                    trials.append((min(t), f, b))
+            for f, b in settings:
+                runner.set_tuning(ph, f, b)
+                run_pass()  # buffers settle to this setting's sizes
+                t = []
+                for _ in range(self.reps):
+                    run_pass()
+                    t.append(runner.stage_ms()[_STAGE[ph]])
+                trials.append((min(t), f, b))
             ms, f, b = min(trials)
             runner.set_tuning(ph, f, b)
-            default = next((tm for tm, ff, bb in trials if ff == 1.0 and bb == 256), None)
+            default = next((tm for tm, ff, bb in trials if (ff, bb) == DEFAULT), None)
             choice[str(ph)] = {"cell_factor": f, "pair_block": b, "stage_ms": ms, "default_ms": default,
                                "tried": len(trials)}
-        self.cache[key] = choice
-        self._save()
+        if not inert:
+            self.cache[key] = choice
+            self._save()
         return dict(choice, cached=False, key=key)
