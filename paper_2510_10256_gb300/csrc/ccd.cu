@@ -266,8 +266,8 @@ __global__ void __launch_bounds__(128) k_ccd_bound(CcdArgs A, const uint32_t* __
                                                    const unsigned int* __restrict__ nlist) {
   const unsigned m = *nlist;
   // uniform trip count per block so that every lane reaches the append
-  for (unsigned w0 = blockIdx.x * blockDim.x; w0 < m; w0 += gridDim.x * blockDim.x) {
-    const unsigned w = w0 + threadIdx.x;
+  for (int64_t w0 = (int64_t)blockIdx.x * blockDim.x; w0 < m; w0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t w = w0 + threadIdx.x;
     bool unres = false;
     uint32_t qq = 0;
     if (w < m) {

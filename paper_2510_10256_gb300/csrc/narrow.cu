@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(CB_THREADS, 3) k_distance_exact(const uint32_t
   if (threadIdx.x == 0) n_unsure = 0;
   __syncthreads();
   // block-uniform: the next CB_THREADS queued pairs, or as many of the undecided ones once enough wait (or no others are left)
-  for (unsigned w0 = blockIdx.x * blockDim.x;;) {
+  for (int64_t w0 = (int64_t)blockIdx.x * blockDim.x;;) {  // (64 bits: the last step of a list near 2^32 pairs passes it)
     const unsigned nu = n_unsure;
     const bool more = w0 < m, typed = more && nu < CB_THREADS;
     if (!more && nu == 0) break;
@@ -335,9 +335,9 @@ __global__ void __launch_bounds__(CB_THREADS, 3) k_distance_exact(const uint32_t
     int e_mem = -1;
     bool live;
     if (typed) {
-      const unsigned w = w0 + threadIdx.x;
+      const int64_t w = w0 + threadIdx.x;
       live = w < m;
-      if (live) c = w < m0 ? list[w] : list[cap - 1 - (int64_t)(w - m0)];
+      if (live) c = w < m0 ? list[w] : list[cap - 1 - (w - m0)];
       w0 += gridDim.x * blockDim.x;
     } else {
       const unsigned take = min(nu, (unsigned)CB_THREADS);
