@@ -75,7 +75,7 @@ typedef enum {
                                        smallest reference distance of that component's filtered pairs)
                                        instead of the scene's */
 #define CB_PER_STENCIL 64           /* per-stencil activation (Sec. 3.3 leaves it for later; the paper's
-                                       hash uses the full activation): after the filter, a class-F
+                                       broad phase uses the full activation): after the filter, a class-F
                                        candidate stays a candidate only if its two primitives' FP64 boxes,
                                        each inflated by half the pair's own width (dbar_min, or its
                                        component's), overlap (closed intervals).  A dropped pair is farther

@@ -936,9 +936,10 @@ __device__ __forceinline__ void add_block(const HessArgs& A, int64_t bi, const d
 // energy, gradient scatter, the PSD-projected Hessian in closed form
 // (pairhess.cuh) and its scatter into the BSR values.  PAIR_T threads a block:
 // the work is a few hundred to a thousand FP64 instructions per warp, of which
-// an SM completes one per ~19 cycles with four warps resident, so small blocks
-// spread a short list over more SMs and cost a long one nothing.  It loads only
-// the points its type needs and subtracts them once (a type's matrix of signs
+// an SM completes one per 16 cycles at best (full occupancy, independent chains)
+// and one per 19 with four warps of dependent ones, so small blocks spread a
+// short list over more SMs and cost a long one nothing.  It loads only the
+// points its type needs and subtracts them once (a type's matrix of signs
 // took 27 multiply-adds and nine conversions more, symmetric blocks their lower
 // triangles): 666 -> 594 FP64 instructions a warp, pleated 97x97 189 -> 157 us.
 constexpr int PAIR_T = 64;
@@ -1739,8 +1740,8 @@ __global__ void __launch_bounds__(S) k_hess_proj(HessArgs A) {
 // One thread per pair runs some 8,500 dependent FP64 instructions, and an FP64
 // warp instruction occupies a warp for 64 cycles however many of its lanes
 // are active (measured on GB300: 64 cycles per dependent or independent DFMA
-// of a lone warp; 76 with one warp per SM sub-partition, the SM's FP64 unit
-// then full at one warp instruction per ~19 cycles), so a short queue (a
+// of a lone warp; 76 with one warp per SM sub-partition, one per 19 cycles and
+// SM, near the unit's rate of one per 16), so a short queue (a
 // small scene) waits for that chain however idle the device is.  This form
 // spreads one pair over a warp, the three lanes (r, t) = (l / 3, l % 3) of
 // row r (lanes 0..26) owning entries t, t + 3, t + 6 of row and column r,

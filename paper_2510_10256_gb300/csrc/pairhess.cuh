@@ -26,8 +26,8 @@
 // rational in the root.  The projection is T - sum (negative eigenpairs).
 //
 // This replaces an iterative 9x9 (3x3 for point-edge) eigenproblem per pair.
-// The Hessian stage is bound by the FP64 pipe (one warp instruction per about
-// 19 cycles and SM, a 64th of the FP32 rate): the roots are found in FP32 by
+// The Hessian stage is bound by the FP64 pipe (one warp instruction per 16
+// cycles and SM at best, a 64th of the FP32 rate): the roots are found in FP32 by
 // an iteration whose model has the equation's poles, and polished to FP64 by
 // two Newton steps whose slopes come from FP32.  All poles, gaps and sums are
 // formed from terms of one sign, so the roots and every component of the
