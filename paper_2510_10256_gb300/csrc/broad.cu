@@ -43,7 +43,7 @@
 //
 // Measured on GB300, contact_build (cell hash, sorted and swept in x -> tiles):
 // pleated 256x256 sheet (14.8M candidates) 1.73 -> 0.24 ms, 200k-triangle graded
-// disk (26.1M) 2.81 -> 0.49, 64 rod scenes (7.2M) 1.60 -> 0.42, woven patch of
+// disk (26.1M) 2.81 -> 0.49, 64 rod scenes (7.2M) 1.60 -> 0.32, woven patch of
 // 4,112 vertices 0.17 -> 0.04 (some 30 launches and three host waits -> four
 // and one).
 #include <algorithm>
@@ -412,7 +412,8 @@ struct TileColumns {
 // Both broad phases of a pass, from twelve box comparisons a column and keys
 // written column by column, 80 registers and three blocks per SM: pleated
 // 256x256 509 -> 404 us, a 200k-triangle graded sheet 1,068 -> 837, 64 rod
-// scenes 950 -> 665 (the windows and components now come once per tile).
+// scenes 950 -> 665 (the windows and components now come once per tile), and
+// 467 with their clusters cut by yarn.
 // The pairs' classes come with them (Sec. 3.2): on shells the rest mesh's
 // filtered pairs are kept as one 32x32 bit mask per pair of clusters, so a
 // tile looks its mask up once and a pair's class is a bit; on rods they are the
