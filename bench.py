@@ -768,8 +768,9 @@ def one_core_baselines() -> dict:
 
 def measure_single(args, name, steps, local, dist, nx=None, mollifier=False, clocks=True) -> dict:
     """One scene of the named workload: W warm-up passes, then `steps` passes
-    timed on the device (L2 flushed before each), the per-stage times of each pass, and an end-to-end leg through the C ABI
-    with host buffers (copies inside the timed region)."""
+    timed on the device (L2 flushed before each), the per-stage times of each
+    pass, and an end-to-end leg through the C ABI with host buffers (copies
+    inside the timed region)."""
     import torch
     from paper_2510_10256_gb300 import contact as CT
     sc, desc = _workload(name, reduced_nx=nx)
